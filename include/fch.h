@@ -86,27 +86,23 @@ typedef struct {
     int prec;            /* fch_precision */
     int sync_every;      /* adaptive runs: trial steps enqueued between host checks */
     int fft_path;        /* 0: automatic; 1: shared-memory Stockham passes for every N;
-                          * 2: warp-transform passes where available (FCH_MIXED, N = 1024) */
+                          * 2: warp-transform column passes where available (FCH_MIXED, N = 1024) */
     int autotune;        /* 1: fch_create takes the tiles fch_autotune picks for (n, prec)
                           * (timing them on first use in the process); 2: the tiles
                           * fch_autotune_step picks; 0: tile_row/tile_col */
-    int tile_row, tile_col; /* pass tiles: 0 default (at n = 1024 two-block-cluster
-                          * column passes for FCH_FP64 / FCH_FP32X2, warp-level row passes
-                          * for FCH_MIXED; in FCH_FP64 and FCH_FP32X2 at n = 128 / 256 the
-                          * generic kernels with 2 / 1 rows a block and columns as -3, and
-                          * in FCH_FP32X2 at n = 512 columns as -3; else the kernel built
-                          * for the grid size); -1 the shared-memory kernels built for the
-                          * size, without clusters or warp-level rows; -2 (tile_col,
-                          * FCH_MIXED at n = 1024) the warp-level column passes; r > 0 the
-                          * generic row kernel with r rows per block / the generic column
-                          * kernel with r column pairs per block; tile_col = -2 - P
-                          * (-3, -4, -6, ...) the generic column kernel with P pairs per
-                          * block at four points a thread (radix-4 stages, twice the
-                          * threads), tile_row = -2 - R the generic row kernel with R
-                          * rows per block at four points a thread. Generic tiles are powers of two that fit whole
-                          * warps, the row kernel's 256 threads or the column kernel's
-                          * 1024 threads a block and a block's shared memory; else
-                          * FCH_EINVAL */
+    int tile_row, tile_col; /* pass tiles: 0 default (n = 64 ... 2048: the passes built
+                          * for the grid size; else the generic kernels); -1 the generic
+                          * shared-memory kernels at the size's default launch shape; -2
+                          * (tile_col, FCH_MIXED at n = 1024) the warp-level column
+                          * passes; r > 0 the generic row kernel with r rows per block /
+                          * the generic column kernel with r column pairs per block;
+                          * tile_col = -2 - P (-3, -4, -6, ...) the generic column kernel
+                          * with P pairs per block at four points a thread (radix-4
+                          * stages, twice the threads), tile_row = -2 - R the generic row
+                          * kernel with R rows per block at four points a thread. Generic
+                          * tiles are powers of two that fit whole warps, the row
+                          * kernel's 256 threads or the column kernel's 1024 threads a
+                          * block and a block's shared memory; else FCH_EINVAL */
 } fch_params;
 
 typedef struct {

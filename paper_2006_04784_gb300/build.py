@@ -32,8 +32,22 @@ def _deps():
         os.path.join(HERE, "..", "include", "fch.h")]
 
 
-def _compile(src: str, extra) -> str:
-    obj = os.path.join(OUT, os.path.basename(src) + ".o")
+# fch_reg.cu holds the passes built for one (precision, grid size): one object each
+REG_SRC = os.path.join(CSRC, "fch_reg.cu")
+REG_TYPES = (("fch::df", "dfl"), ("double", "f64"), ("float", "f32"))
+REG_LOGN = range(6, 12)
+
+
+def _units():
+    """(source, object name, extra flags) of every compilation, the longest first"""
+    reg = [(REG_SRC, f"fch_reg_{sfx}_{l}.o", [f"-DFCH_T={t}", f"-DFCH_SUFFIX={sfx}", f"-DFCH_LOGN={l}"])
+           for t, sfx in REG_TYPES for l in reversed(REG_LOGN)]
+    rest = [(s, os.path.basename(s) + ".o", []) for s in sorted(glob.glob(os.path.join(CSRC, "*.cu"))) if s != REG_SRC]
+    return rest + reg
+
+
+def _compile(src: str, name: str, extra) -> str:
+    obj = os.path.join(OUT, name)
     newest = max(os.path.getmtime(p) for p in _deps() + [src, __file__])
     if os.path.exists(obj) and os.path.getmtime(obj) >= newest:
         return obj
@@ -47,10 +61,10 @@ def _compile(src: str, extra) -> str:
 def build(verbose: bool = False, extra=()) -> str:
     """Compile every CUDA source of the package; returns the library path."""
     os.makedirs(OUT, exist_ok=True)
-    srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+    units = _units()
     extra = list(extra) + (["-Xptxas", "-v"] if verbose else [])
-    with cf.ThreadPoolExecutor(max_workers=len(srcs)) as ex:
-        objs = list(ex.map(lambda s: _compile(s, extra), srcs))
+    with cf.ThreadPoolExecutor(max_workers=os.cpu_count() or 8) as ex:
+        objs = list(ex.map(lambda u: _compile(u[0], u[1], u[2] + extra), units))
     newest = max(os.path.getmtime(o) for o in objs)
     if not os.path.exists(LIB) or os.path.getmtime(LIB) < newest:
         tmp = LIB + f".{os.getpid()}.tmp"

@@ -30,7 +30,8 @@ fch_geom fch_geometry(int N, int prec)
     const int SL = N + N / 8; // skewed sequence length in shared memory
     g.col_smem = (N + 2 * P * SL) * csz;
     if (N == 1024 && csz == 16) {
-        // two-block clusters, one column of a pair per block, twiddles in global memory
+        // two-block clusters, one column of a pair per block (the passes built for 1024 keep
+        // this grid; the generic kernel takes the tile -1 geometry below)
         g.col_threads = N / 8;
         g.col_blocks = N;
         g.col_smem = SL * csz;
@@ -46,6 +47,14 @@ fch_geom fch_geometry(int N, int prec)
     g.row_blocks = N / rpb;
     g.row_smem = rpb * SL * csz;
     return g;
+}
+
+// blocks of the column passes built for a grid size (RegCfg in fch_reg.cuh): a column pair
+// each in 16-byte elements, at N = 1024 a column; two pairs in 8-byte ones; 0: none built
+int fch_reg_col_blocks(int N, int prec)
+{
+    if (N < 64 || N > 2048) return 0;
+    return prec == 1 ? N / 4 : N == 1024 ? N : N / 2;
 }
 
 fch_geom fch_geometry_tiled(int N, int prec, int tile_row, int tile_col)
@@ -123,10 +132,10 @@ bool fch_tile_valid(int N, int prec, int tile_row, int tile_col)
 
 // ---------------------------------------------------------------------------
 // control kernel: one block of 256 threads running ctrl_block
-__global__ void __launch_bounds__(256) fch_ctrl_kernel(const fch_kparams kp, int op, int na, double arg0)
+template <int OP> __global__ void __launch_bounds__(256) fch_ctrl_kernel(const fch_kparams kp, int na, double arg0)
 {
     pdl_begin();
-    ctrl_block(kp, op, na, arg0);
+    ctrl_block<OP>(kp, na, arg0);
 }
 
 cudaError_t fch_launch_ctrl(int op, const fch_kparams &kp, int na, int, double arg0, cudaStream_t s)
@@ -134,7 +143,13 @@ cudaError_t fch_launch_ctrl(int op, const fch_kparams &kp, int na, int, double a
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     fch_pdl_config(cfg, at, dim3(1), dim3(256), 0, s, kp.pdl != 0);
-    return cudaLaunchKernelEx(&cfg, fch_ctrl_kernel, kp, op, na, arg0);
+    switch (op) {
+    case OP_INIT_TRIAL: return cudaLaunchKernelEx(&cfg, fch_ctrl_kernel<OP_INIT_TRIAL>, kp, na, arg0);
+    case OP_DECIDE_INIT: return cudaLaunchKernelEx(&cfg, fch_ctrl_kernel<OP_DECIDE_INIT>, kp, na, arg0);
+    case OP_ACCEPT: return cudaLaunchKernelEx(&cfg, fch_ctrl_kernel<OP_ACCEPT>, kp, na, arg0);
+    case OP_ACCEPT_INIT: return cudaLaunchKernelEx(&cfg, fch_ctrl_kernel<OP_ACCEPT_INIT>, kp, na, arg0);
+    }
+    return cudaErrorInvalidValue;
 }
 
 // launch configuration of a pass or control kernel: programmatic stream
@@ -686,19 +701,9 @@ extern "C" fch_status fch_create(const fch_grid *g, const fch_params *p, void *s
         trow = t.tile_row;
         tcol = t.tile_col;
     }
-    // At 128^2 and 256^2 in double and double-float the compile-time kernels give a
-    // block several rows (column pairs): 8 to 32 blocks for 152 SMs, each pair's chain
-    // of dependent work long. There the default (tile 0, asked for or tuned) is the
-    // row tile the step tuner (fch_autotune_step, adaptive IMEX trials) picked on GB300
-    // and one column pair a block at four points a thread (tile_col -3), and in
-    // double-float at 512^2 the same columns; -1 still asks for the compile-time
-    // kernels. Against those: 2.0x the trials per second in double, 1.3-1.4x in
-    // double-float; 1.09x at 512^2.
-    if (ctx->prec != FCH_MIXED) {
-        if (trow == 0 && (N == 128 || N == 256)) trow = N == 128 ? 2 : 1;
-        if (tcol == 0 && (N == 128 || N == 256 || (N == 512 && ctx->prec == FCH_FP32X2))) tcol = -3;
-    }
     ctx->geom = fch_geometry_tiled(N, ctx->prec == FCH_MIXED, trow, tcol);
+    if (tcol == 0 && fch_reg_col_blocks(N, ctx->prec == FCH_MIXED))
+        ctx->geom.col_blocks = fch_reg_col_blocks(N, ctx->prec == FCH_MIXED); // a partial sum each
     void **bufs[] = {&ctx->U[0], &ctx->U[1], &ctx->U[2], &ctx->F[0], &ctx->F[1], &ctx->F[2],
                      &ctx->Pb, &ctx->Qb, &ctx->Vb, &ctx->Nb};
     for (void **b : bufs)
@@ -729,14 +734,11 @@ extern "C" fch_status fch_create(const fch_grid *g, const fch_params *p, void *s
     ctx->kp.P = ctx->geom.P;
     ctx->kp.tile_row = trow;
     ctx->kp.tile_col = tcol;
-    // Programmatic dependent launch pays where every pass is one full wave: the default
-    // tiles at 1024^2 in double and double-float (1024 blocks of 128 threads, seven a
-    // SM), where a successor's blocks can only take the slots the tail frees. Where a
-    // pass leaves SMs free (smaller grids) the successor's waiting blocks take them
-    // early and the running pass ends up packed onto fewer SMs (512^2: 2.3x slower
-    // trials in double); where it has several waves (2048^2) they take later waves'
-    // slots.
-    ctx->kp.pdl = N == 1024 && ctx->prec != FCH_MIXED && trow == 0 && tcol == 0;
+    // Programmatic dependent launch with the passes built for a size, which let their
+    // successor start when it pays (RegCfg::early); the generic kernels of other tiles let
+    // it start at once, which crowds passes that leave SMs free (512^2: 2.3x slower trials
+    // in double), and launch without it.
+    ctx->kp.pdl = fch_reg_col_blocks(N, ctx->prec == FCH_MIXED) && trow == 0 && tcol == 0;
     for (int i = 0; i < 3; i++) {
         ctx->kp.U[i] = ctx->U[i];
         ctx->kp.F[i] = ctx->F[i];
@@ -2013,14 +2015,17 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
     // plans, one pair)
     const int np = prec == FCH_FP32X2 ? 1 : plan_chunk(n, prec);
     const size_t rb = (size_t)n * n * rsz, cb = (size_t)(n / 2 + 1) * n * csz;
-    void *x = nullptr, *Z = nullptr, *X = nullptr, *tw = nullptr, *tw2 = nullptr;
+    void *x = nullptr, *Z = nullptr, *X = nullptr, *tw = nullptr, *tw4 = nullptr, *tw2 = nullptr;
     cudaError_t e = cudaMalloc(&x, 2 * np * rb);
     if (e == cudaSuccess) e = cudaMalloc(&Z, (size_t)np * n * n * csz);
     if (e == cudaSuccess) e = cudaMalloc(&X, 2 * np * cb);
     if (e == cudaSuccess) e = cudaMalloc(&tw, (size_t)n * csz);
+    if (e == cudaSuccess) e = cudaMalloc(&tw4, (size_t)n * csz);
     if (e == cudaSuccess) e = cudaMemsetAsync(x, 0, 2 * np * rb, s);
     fch_ctx dummy;
-    if (e == cudaSuccess && upload_twiddles(&dummy, n, prec, tw, s) != FCH_OK) e = cudaErrorUnknown;
+    if (e == cudaSuccess && (upload_twiddles(&dummy, n, prec, tw, s) != FCH_OK ||
+                             upload_twiddles(&dummy, n, prec, tw4, s, 2) != FCH_OK))
+        e = cudaErrorUnknown;
     if (e == cudaSuccess && single && n == 1024) e = upload_tw2(&tw2, s);
     fch_kparams kp;
     memset(&kp, 0, sizeof(kp));
@@ -2029,6 +2034,7 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
     kp.inv_n2 = 1.0 / ((double)n * n);
     kp.Z = Z;
     kp.tw = tw;
+    kp.tw4 = tw4;
     kp.tw2 = tw2;
     kp.tail_op = -1;
     kp.flags = FCH_FL_NOSKIP | (single ? 0 : FCH_FL_F64IO);
@@ -2090,7 +2096,7 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
         }
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (void *b : {x, Z, X, tw, tw2})
+    for (void *b : {x, Z, X, tw, tw4, tw2})
         if (b) cudaFree(b);
     if (e != cudaSuccess) {
         snprintf(g_plan_err, sizeof(g_plan_err), "fch_autotune: %s", cudaGetErrorString(e));
@@ -2227,7 +2233,7 @@ struct fch_fft_plan {
     cudaStream_t stream;
     fch_geom geom;
     fch_kparams kp;
-    void *Z, *tw, *tw2;
+    void *Z, *tw, *tw4, *tw2;
     int *err; // device word: set by a pass whose bounded wait on a bulk copy ran out
 };
 
@@ -2258,6 +2264,7 @@ extern "C" fch_status fch_fft_plan_create(int n, int prec, void *stream, fch_fft
     const size_t csz = prec ? 8 : 16;
     cudaError_t e = cudaMalloc(&pl->Z, (size_t)pl->chunk * n * n * csz);
     if (e == cudaSuccess) e = cudaMalloc(&pl->tw, (size_t)n * csz);
+    if (e == cudaSuccess) e = cudaMalloc(&pl->tw4, (size_t)n * csz);
     if (e == cudaSuccess) e = cudaMalloc(&pl->err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(pl->err, 0, sizeof(int), pl->stream);
     if (e != cudaSuccess) {
@@ -2265,7 +2272,8 @@ extern "C" fch_status fch_fft_plan_create(int n, int prec, void *stream, fch_fft
         return e == cudaErrorMemoryAllocation ? FCH_ENOMEM : FCH_ECUDA;
     }
     fch_ctx dummy;
-    if (upload_twiddles(&dummy, n, prec, pl->tw, pl->stream) != FCH_OK) {
+    if (upload_twiddles(&dummy, n, prec, pl->tw, pl->stream) != FCH_OK ||
+        upload_twiddles(&dummy, n, prec, pl->tw4, pl->stream, 2) != FCH_OK) {
         fch_fft_plan_destroy(pl);
         return FCH_ECUDA;
     }
@@ -2282,6 +2290,7 @@ extern "C" fch_status fch_fft_plan_create(int n, int prec, void *stream, fch_fft
     pl->kp.cd.inv_n2 = pl->kp.inv_n2;
     pl->kp.Z = pl->Z;
     pl->kp.tw = pl->tw;
+    pl->kp.tw4 = pl->tw4;
     pl->kp.err = pl->err;
     if (prec && n == 1024) {
         if (upload_tw2(&pl->tw2, pl->stream) != cudaSuccess) {
@@ -2299,6 +2308,7 @@ extern "C" fch_status fch_fft_plan_destroy(fch_fft_plan *pl)
     if (!pl) return FCH_OK;
     if (pl->Z) cudaFree(pl->Z);
     if (pl->tw) cudaFree(pl->tw);
+    if (pl->tw4) cudaFree(pl->tw4);
     if (pl->tw2) cudaFree(pl->tw2);
     if (pl->err) cudaFree(pl->err);
     free(pl);

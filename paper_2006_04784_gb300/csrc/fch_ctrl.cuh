@@ -15,6 +15,8 @@
 // complete (its writes visible), before it reads anything, then allows its own
 // successor to begin launching; the successor's blocks wait in turn. Launched
 // without the attribute, both instructions return at once.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -46,12 +48,13 @@ __device__ inline double root6_nr(double x)
     return x * z2 * z2 * z;
 }
 
-// one control operation; returns false when the run stopped (done or failure)
-__device__ inline bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, int op, double S0, double S1,
-                               double arg0)
+// one control operation; returns false when the run stopped (done or failure). The
+// operation is a template argument: a kernel holds the code (and the registers) of the
+// operations it can run only.
+template <int OP>
+__device__ __forceinline__ bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, double S0, double S1, double arg0)
 {
-    switch (op) {
-    case OP_INIT_TRIAL: {
+    if constexpr (OP == OP_INIT_TRIAL) {
         double k1;
         if (arg0 > 0) {
             k1 = arg0; // fixed step
@@ -97,9 +100,7 @@ __device__ inline bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, int op, doubl
         }
         c->psd_conv = 0;
         c->psd_iter = 0;
-        break;
-    }
-    case OP_SAV_E1: {
+    } else if constexpr (OP == OP_SAV_E1) {
         const double e1 = kp.h2 * S0;
         const double v = e1 + kp.D0;
         if (!isfinite(v) || v <= 0) {
@@ -111,9 +112,7 @@ __device__ inline bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, int op, doubl
         c->inv_sqrt_e1 = 1.0 / sqrt(v);
         if (arg0 == 1.0) c->r_n = sqrt(v);
         if (arg0 == 2.0) c->r_m = sqrt(v);
-        break;
-    }
-    case OP_SAV_R: {
+    } else if constexpr (OP == OP_SAV_R) {
         // eq. (4.8) with u^{n+1} = p + r q:
         // r (a - a (X, q)/2) = -b r^n - c r^{n-1} + (X, a p + b u^n + c u^{n-1})/2
         const double sc = kp.h2 * kp.inv_n2; // Parseval on the unnormalised half spectra
@@ -125,9 +124,7 @@ __device__ inline bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, int op, doubl
             return false;
         }
         c->r_new = r;
-        break;
-    }
-    case OP_PSD_CHECK: {
+    } else if constexpr (OP == OP_PSD_CHECK) {
         const double ratio = sqrt(S0) / sqrt(S1); // ||d|| / ||v_{s+1}||, h cancels
         c->psd_iter++;
         c->n_psd_iter++;
@@ -143,9 +140,7 @@ __device__ inline bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, int op, doubl
             c->done = 1;
             c->last_psd_iter = c->psd_iter;
         }
-        break;
-    }
-    case OP_DECIDE: {
+    } else if constexpr (OP == OP_DECIDE) {
         // Steps 3-4 of the adaptive algorithm, Sec. 3.2, with e^2 = S0/S1:
         // accept iff S0 <= sigma^2 S1 (or k <= k_min);
         // A_dp = rho_s k (sigma/e)^(1/3) = rho_s k (sigma^2 S1 / S0)^(1/6), e >= 1e-16
@@ -181,9 +176,7 @@ __device__ inline bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, int op, doubl
             c->accepted_last = 0;
         }
         c->ktrial = kn;
-        break;
-    }
-    case OP_ACCEPT: {
+    } else if constexpr (OP == OP_ACCEPT) {
         const int un = c->iu_n, um = c->iu_m;
         c->iu_m = un;
         c->iu_n = c->iu_new;
@@ -201,12 +194,8 @@ __device__ inline bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, int op, doubl
         c->t += c->k1;
         c->n_steps++;
         c->n_attempts++;
-        break;
-    }
-    case OP_ENERGY: {
+    } else if constexpr (OP == OP_ENERGY) {
         c->energy = kp.h2 * S0;
-        break;
-    }
     }
     return !c->done;
 }
@@ -236,7 +225,7 @@ __device__ inline void sync_coef_lanes(fch_ctrl *c, int lane)
 // first na partials of slots 0 and 1 are summed in a fixed order (per-thread
 // strided sums, warp shuffles, then thread 0 over the warp sums), thread 0 runs
 // the operation, and the block writes the control block back.
-__device__ inline void ctrl_block(const fch_kparams &kp, int op, int na, double arg0)
+template <int OP> __device__ __forceinline__ void ctrl_block(const fch_kparams &kp, int na, double arg0)
 {
     __shared__ double sh[2][32];
     __shared__ fch_ctrl cs;
@@ -251,7 +240,7 @@ __device__ inline void ctrl_block(const fch_kparams &kp, int op, int na, double 
     }
     __syncthreads();
     if (cs.done && !(kp.flags & FCH_FL_NOSKIP)) return;
-    if (op == OP_PSD_CHECK && cs.psd_conv) return;
+    if (OP == OP_PSD_CHECK && cs.psd_conv) return;
     for (int o = 16; o > 0; o >>= 1) {
         s0 += __shfl_down_sync(0xffffffffu, s0, o);
         s1 += __shfl_down_sync(0xffffffffu, s1, o);
@@ -268,24 +257,13 @@ __device__ inline void ctrl_block(const fch_kparams &kp, int op, int na, double 
             S1 += sh[1][w];
         }
         // the combined operations: the decision (adaptive) or the acceptance of a fixed
-        // step, then the set-up of the next trial (adaptive: arg0 -1; fixed: arg0 = dt)
-        bool again = false;
-        double next_arg = -1.0;
-        if (op == OP_DECIDE_INIT) {
-            op = OP_DECIDE;
-            again = true;
-        } else if (op == OP_ACCEPT_INIT) {
-            op = OP_ACCEPT;
-            next_arg = arg0;
-            arg0 = 0.0;
-            again = true;
-        }
-        for (;;) {
-            if (!ctrl_op(&cs, kp, op, S0, S1, arg0)) break;
-            if (!again) break;
-            again = false;
-            op = OP_INIT_TRIAL;
-            arg0 = next_arg;
+        // step, then the set-up of the next trial (adaptive: -1; fixed: arg0 = dt)
+        if constexpr (OP == OP_DECIDE_INIT) {
+            if (ctrl_op<OP_DECIDE>(&cs, kp, S0, S1, arg0)) ctrl_op<OP_INIT_TRIAL>(&cs, kp, S0, S1, -1.0);
+        } else if constexpr (OP == OP_ACCEPT_INIT) {
+            if (ctrl_op<OP_ACCEPT>(&cs, kp, S0, S1, 0.0)) ctrl_op<OP_INIT_TRIAL>(&cs, kp, S0, S1, arg0);
+        } else {
+            ctrl_op<OP>(&cs, kp, S0, S1, arg0);
         }
     }
     if (threadIdx.x < 32) {
@@ -296,11 +274,13 @@ __device__ inline void ctrl_block(const fch_kparams &kp, int op, int na, double 
     for (int i = threadIdx.x; i < nw; i += nthr) ((long long *)kp.ctrl)[i] = ((const long long *)&cs)[i];
 }
 
-// Called by every block of a pass after its partial sums are written: the last
-// block to arrive (atomic ticket after a fence) runs the control operation
-// kp.tail_op over the partials of all gridDim.x blocks, then resets the ticket.
-__device__ inline void pass_tail(const fch_kparams &kp)
+// Called by every block of a pass after its partial sums are written (where the launch
+// asks for it, kp.tail_op >= 0): the last block to arrive (atomic ticket after a fence)
+// runs the control operation of the pass over the partials of all gridDim.x blocks, then
+// resets the ticket.
+template <int OP> __device__ __forceinline__ void pass_tail(const fch_kparams &kp)
 {
+    if (kp.tail_op < 0) return;
     __shared__ unsigned int last;
     __threadfence();
     __syncthreads();
@@ -308,6 +288,6 @@ __device__ inline void pass_tail(const fch_kparams &kp)
     __syncthreads();
     if (!last) return;
     __threadfence();
-    ctrl_block(kp, kp.tail_op, gridDim.x, kp.tail_arg);
+    ctrl_block<OP>(kp, gridDim.x, kp.tail_arg);
     if (threadIdx.x == 0) *kp.ticket = 0;
 }

@@ -88,7 +88,8 @@ struct fch_kparams {
     long long pstride_in, pstride_out; // bytes from one pair's in0/in1 (out0/out1) to the next's
     int src;                        // spectrum a start pass reads (FCH_SRC_*)
     int flags;                      // FCH_FL_*
-    int tail_op;                    // < 0: none; else the control op the pass's last block runs
+    int tail_op;                    // < 0: none; else the pass's last block runs the control op of its mode
+                                    // (row_tail_op, col_tail_op)
     double tail_arg;
     unsigned int *ticket;           // arrival counter of the blocks of a pass (reset by the last)
     int *err;                       // set to 1 by a pass whose bounded wait on a bulk copy ran out (may be null)
@@ -101,7 +102,6 @@ enum { FCH_SRC_UN = 0, FCH_SRC_UNEW = 1, FCH_SRC_V = 2, FCH_SRC_IN0 = 3 };
 enum {
     FCH_FL_AM3 = 1,        // F finish: also form the AM3 predictor and the LTE norms
     FCH_FL_PACK_F = 2,     // solve passes: pack (u_new, Lap u_new) for F(u_new)
-    FCH_FL_ENERGY = 4,     // F row pass: also accumulate the energy density
     FCH_FL_NOSKIP = 8,     // ignore ctrl->done (host-driven single evaluations)
     FCH_FL_COPYV = 16,     // F start from the PSD iterate: copy it into the trial slot
     FCH_FL_PSDSKIP = 32,   // pass belongs to a PSD iteration: return if converged
@@ -131,7 +131,7 @@ enum {
     RM_R2C_LOAD = 0,   // real fields -> forward rows (standalone R2C, device fields)
     RM_C2R_STORE,      // inverse rows -> real fields
     RM_NIMEX,          // (u, Lap u) -> pieces of N_IMEX(u)
-    RM_F,              // (u, Lap u) -> pieces of mu(u) (+ energy density)
+    RM_F,              // (u, Lap u) -> pieces of mu(u)
     RM_SAV,            // (u, Lap u) -> pieces of V[u] (+ G(u) density)
     RM_ENERGY,         // (u, Lap u) -> energy density only
     RM_NIMEX_DIRECT,   // (u*, Lap u*) from the stored real-space slots -> pieces of N_IMEX(u*)
@@ -152,6 +152,17 @@ enum {
     OP_ACCEPT_INIT     // OP_ACCEPT of a fixed step, then OP_INIT_TRIAL with step size arg0
 };
 
+// the control operation of a mode's block sums, run by the pass's last block (-1: the mode
+// sums nothing, or a control launch of its own reads the sums)
+constexpr int row_tail_op(int mode)
+{
+    return mode == RM_SAV || mode == RM_SAV_DIRECT ? OP_SAV_E1 : mode == RM_ENERGY ? OP_ENERGY : -1;
+}
+constexpr int col_tail_op(int mode)
+{
+    return mode == CM_SAV_PQ ? OP_SAV_R : mode == CM_PSD_ITER ? OP_PSD_CHECK : -1;
+}
+
 // pass geometry for grid N and precision (0 = f64, 1 = f32)
 struct fch_geom {
     int col_blocks, col_threads, col_smem;
@@ -170,6 +181,18 @@ cudaError_t fch_launch_col_f32(int mode, const fch_kparams &kp, cudaStream_t s);
 cudaError_t fch_launch_row_f32(int mode, const fch_kparams &kp, cudaStream_t s);
 cudaError_t fch_launch_col_dfl(int mode, const fch_kparams &kp, cudaStream_t s);
 cudaError_t fch_launch_row_dfl(int mode, const fch_kparams &kp, cudaStream_t s);
+// the passes built for a grid size (fch_reg.cu), one pair of launchers per (precision, log2 N)
+#define FCH_REG_DECL1(sfx, l)                                                               \
+    cudaError_t fch_reg_col_##sfx##_##l(int mode, const fch_kparams &kp, cudaStream_t s);   \
+    cudaError_t fch_reg_row_##sfx##_##l(int mode, const fch_kparams &kp, cudaStream_t s);
+#define FCH_REG_DECL(sfx)                                                                   \
+    FCH_REG_DECL1(sfx, 6) FCH_REG_DECL1(sfx, 7) FCH_REG_DECL1(sfx, 8)                       \
+    FCH_REG_DECL1(sfx, 9) FCH_REG_DECL1(sfx, 10) FCH_REG_DECL1(sfx, 11)
+FCH_REG_DECL(f64)
+FCH_REG_DECL(f32)
+FCH_REG_DECL(dfl)
+// blocks of their column pass at grid size N (one partial sum each), prec as fch_geometry
+int fch_reg_col_blocks(int N, int prec);
 // launch configuration with programmatic stream serialization (when enabled)
 bool fch_pdl_enabled();
 void fch_pdl_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, dim3 grid, dim3 block, size_t smem,

@@ -408,6 +408,46 @@ template <typename C> __device__ __forceinline__ C *pair_Z(const fch_kparams &kp
     return (C *)kp.Z + (size_t)blockIdx.y * N * N;
 }
 
+// the coefficients and buffers of a column pass from the control block (each block once)
+template <typename T>
+__device__ __forceinline__ void load_colbufs(const fch_kparams &kp, fch_coef<T> &co, ColBufs<typename CT<T>::t> &bf)
+{
+    typedef typename CT<T>::t C;
+    bf.i0 = (const C *)pair_in(kp.in0, kp);
+    bf.i1 = (const C *)pair_in(kp.in1, kp);
+    bf.o0 = (C *)pair_out(kp.out0, kp);
+    bf.o1 = (C *)pair_out(kp.out1, kp);
+    if (kp.ctrl) {
+        const fch_ctrl *cs = kp.ctrl;
+        co = load_coef<T>(cs);
+        bf.Un = (const C *)kp.U[cs->iu_n];
+        bf.Um = (const C *)kp.U[cs->iu_m];
+        bf.Unew = (C *)kp.U[cs->iu_new];
+        bf.Fn = (const C *)kp.F[cs->if_n];
+        bf.Fm = (const C *)kp.F[cs->if_m];
+        switch (kp.src) {
+        case FCH_SRC_UN: bf.src = bf.Un; bf.dst = (C *)kp.F[cs->if_n]; break;
+        case 5: bf.src = bf.Um; bf.dst = (C *)kp.F[cs->if_m]; break;
+        case FCH_SRC_UNEW: bf.src = bf.Unew; bf.dst = (C *)kp.F[cs->if_new]; break;
+        case FCH_SRC_V: bf.src = (const C *)kp.Vb; bf.dst = nullptr; break;
+        default: bf.src = (const C *)kp.in0; bf.dst = (C *)kp.out0; break;
+        }
+    } else {
+        bf.Un = bf.Um = bf.src = bf.Fn = bf.Fm = nullptr;
+        bf.Unew = bf.dst = nullptr;
+        co = fch_coef<T>();
+    }
+}
+
+// The mean mode (k = 0) of a BDF2 solve, which carries the mass: a u + b u^n + c u^{n-1} = 0
+// with a + b + c = 0 is u = u^n + (c / a) (u^n - u^{n-1}). In this form the mean stays the
+// same to the last bit while u^n and u^{n-1} share it, where the quotient of the two
+// products would round once a step (a random walk of the mass over thousands of steps).
+template <typename T, typename C> __device__ __forceinline__ C mean_mode(const fch_coef<T> &co, C un, C um)
+{
+    return cadd(un, cscale(csub(un, um), co.c * recip(co.a)));
+}
+
 template <typename T, int MODE>
 __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_consts<T> &K,
                                           const fch_coef<T> &co, const ColBufs<typename CT<T>::t> &bf,
@@ -448,11 +488,7 @@ __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_const
     } else if (MODE == CM_IMEX_SOLVE) {
         // eq. (IMEX-eq): (a + |k|^2 s) u^{n+1} = -b u^n - c u^{n-1} - |k|^2 N_IMEX(u*)^
         if ((kx | ky) == 0) {
-            // the mean mode (k = 0) carries the mass: renormalised arithmetic and a
-            // division there, where a bias of the one-Newton-step reciprocal (or the
-            // coarser rounding of unrenormalised low words) would repeat every step
-            const C rhs = csub(cscale(ldg(bf.Un + idx), -co.b), cscale(ldg(bf.Um + idx), co.c));
-            v = mk<C>(rhs.x / co.a, rhs.y / co.a);
+            v = mean_mode(co, ldg(bf.Un + idx), ldg(bf.Um + idx));
         } else {
             const C Nh = bsub(A, lscale(B, rmul(K.e2, k2)));
             const C rhs =
@@ -494,9 +530,8 @@ __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_const
         const T den = radd(co.a, rmul(k2, l0));
         const T iden = recip(den);
         C p;
-        if ((kx | ky) == 0) { // the mean mode: as in the IMEX solve
-            const C pr = csub(cscale(un, -co.b), cscale(um, co.c));
-            p = mk<C>(pr.x / co.a, pr.y / co.a);
+        if ((kx | ky) == 0) {
+            p = mean_mode(co, un, um);
         } else {
             p = lnorm(lscale(bsub(lscale(un, -co.b), badd(lscale(um, co.c), lscale(us, rmul(k2, l1)))), iden));
         }
@@ -561,32 +596,6 @@ __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_const
     }
 }
 
-// column pairs per block at a compile-time size, the same rule as fch_geometry:
-// max(pmin, 1024 / N), pmin = 2 for 8-byte elements and 1 for 16-byte ones
-template <typename T, int LOGN> constexpr int spec_pairs()
-{
-    return (1024 >> LOGN) > (sizeof(T) == 4 ? 2 : 1) ? (1024 >> LOGN) : (sizeof(T) == 4 ? 2 : 1);
-}
-
-// Resident blocks per SM a compile-time pass is built for: four blocks of 256
-// threads (at most 64 registers a thread) at N <= 1024, so that the 512 blocks of a
-// 1024^2 pass run in one wave on the 152 SMs (with three per SM, 56 blocks would be
-// left for a second wave); other sizes keep the compiler's choice.
-template <int THREADS, int LOGN> constexpr int pass_min_blocks()
-{
-    return (LOGN > 0 && LOGN <= 10 && THREADS == 256) ? 4 : 1;
-}
-// The standalone transforms' column passes of 512 threads (single precision, N = 1024,
-// two column pairs a block) are built for three resident blocks an SM (at most 42
-// registers a thread): their launches carry many field pairs, so occupancy, not the
-// wave count, is what they need.
-template <int THREADS, int LOGN, int MODE> constexpr int col_min_blocks()
-{
-    return (THREADS == 512 && LOGN == 10 && (MODE == CM_FWD_STORE || MODE == CM_INV_LOAD))
-               ? 3
-               : pass_min_blocks<THREADS, LOGN>();
-}
-
 // Pair 0 of a column tile of an N-point transform (columns kx = 0 in slot s0 and
 // kx = N/2 in slot s1 of a tile whose row n sits at skew(n) * nc), work item ky in [0, N/2]: rows ky and -ky of
 // both columns (one row where they coincide). Each of the two columns is the
@@ -643,27 +652,20 @@ __device__ __forceinline__ void pair0_item(const fch_kparams &kp, const fch_cons
     }
 }
 
-// LOGN > 0: the grid size is a compile-time constant (N = 2^LOGN >= 512), so the
-// index arithmetic of the transforms folds into immediates; LOGN = 0 reads N and P
-// from the parameters. PPT: points of a column a thread transforms (8: radix-8
-// stages, nc N / 8 threads; 4, generic kernel only: radix-4 stages, twice the threads
-// and half the dependent work a thread, for small grids whose passes are too few
-// warps to fill the GPU; twiddles from kp.tw4).
-template <typename T, int MODE, int LOGN, int PPT = 8>
-__global__ void __launch_bounds__(LOGN ? ((spec_pairs<T, LOGN>() << LOGN) >> 2) : 1024,
-                                  col_min_blocks<LOGN ? ((spec_pairs<T, LOGN>() << LOGN) >> 2) : 1024, LOGN, MODE>())
-col_pass(const fch_kparams kp)
+// The generic column pass: any N and number of column pairs a block (kp.P), as tiles ask.
+// PPT: points of a column a thread transforms (8: radix-8 stages, nc N / 8 threads; 4:
+// radix-4 stages, twice the threads and half the dependent work a thread; twiddles from
+// kp.tw4).
+template <typename T, int MODE, int PPT = 8> __global__ void __launch_bounds__(1024) col_pass(const fch_kparams kp)
 {
-    static_assert(PPT == 8 || (PPT == 4 && LOGN == 0), "four points a thread in the generic kernel only");
+    static_assert(PPT == 8 || PPT == 4, "eight or four points a thread");
     typedef typename CT<T>::t C;
     typedef ColTraits<MODE> TR;
     pdl_begin();
     if (pass_skipped(kp)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red_scratch[FCH_NRED * 32];
-    const int N = LOGN ? (1 << LOGN) : kp.N, P = LOGN ? spec_pairs<T, LOGN>() : kp.P, nc = 2 * P;
-    const int logN = LOGN ? LOGN : kp.logN;
-    const int nthr = LOGN ? (P << LOGN) / 4 : (int)blockDim.x;
+    const int N = kp.N, P = kp.P, nc = 2 * P, logN = kp.logN, nthr = blockDim.x;
     C *tw = (C *)smem_raw;
     C *tile = tw + N;
     const int c = threadIdx.x % nc, t = threadIdx.x / nc;
@@ -677,30 +679,7 @@ col_pass(const fch_kparams kp)
     // per-block constants from the control block
     fch_coef<T> co;
     ColBufs<C> bf;
-    bf.i0 = (const C *)pair_in(kp.in0, kp);
-    bf.i1 = (const C *)pair_in(kp.in1, kp);
-    bf.o0 = (C *)pair_out(kp.out0, kp);
-    bf.o1 = (C *)pair_out(kp.out1, kp);
-    if (kp.ctrl) {
-        const fch_ctrl *cs = kp.ctrl;
-        co = load_coef<T>(cs);
-        bf.Un = (const C *)kp.U[cs->iu_n];
-        bf.Um = (const C *)kp.U[cs->iu_m];
-        bf.Unew = (C *)kp.U[cs->iu_new];
-        bf.Fn = (const C *)kp.F[cs->if_n];
-        bf.Fm = (const C *)kp.F[cs->if_m];
-        switch (kp.src) {
-        case FCH_SRC_UN: bf.src = bf.Un; bf.dst = (C *)kp.F[cs->if_n]; break;
-        case 5: bf.src = bf.Um; bf.dst = (C *)kp.F[cs->if_m]; break;
-        case FCH_SRC_UNEW: bf.src = bf.Unew; bf.dst = (C *)kp.F[cs->if_new]; break;
-        case FCH_SRC_V: bf.src = (const C *)kp.Vb; bf.dst = nullptr; break;
-        default: bf.src = (const C *)kp.in0; bf.dst = (C *)kp.out0; break;
-        }
-    } else {
-        bf.Un = bf.Um = bf.src = bf.Fn = bf.Fm = nullptr;
-        bf.Unew = bf.dst = nullptr;
-        co = fch_coef<T>();
-    }
+    load_colbufs<T>(kp, co, bf);
 
     const C *twsrc = (const C *)(PPT == 8 ? kp.tw : kp.tw4);
     for (int i = threadIdx.x; i < N; i += nthr) tw[i] = ldg(twsrc + i);
@@ -756,7 +735,7 @@ col_pass(const fch_kparams kp)
     }
     if (has_red) {
         block_partials<2>(red, kp.part, red_scratch);
-        if (kp.tail_op >= 0) pass_tail(kp);
+        if constexpr (col_tail_op(MODE) >= 0) pass_tail<col_tail_op(MODE)>(kp);
     }
     if (inv) {
         fft_smem<+1, false, PPT>(tile, N, logN, nc, c, tw, t);
@@ -769,190 +748,54 @@ col_pass(const fch_kparams kp)
     }
 }
 
-// ---------------------------------------------------------------------------
-// Column pass for 16-byte elements at N = 1024 as clusters of two blocks: block
-// rank r of cluster p owns column slot r of pair p (r = 0: kx, r = 1: N - kx; pair
-// 0: kx = 0 and N/2), 128 threads, one column in shared memory, twiddles read from
-// global memory. The spectral stage couples the pair's columns (the Hermitian split
-// reads Z(kx, ky) and Z(N - kx, -ky)); each block takes half of the pair's work
-// items and reaches the partner's column through distributed shared memory, with a
-// cluster barrier before (forward transforms done) and after (before the inverse
-// transforms, and before any block may exit while its partner still reads it).
-// 1024 blocks of 128 threads fit seven to an SM: one wave over the 152 SMs at six or
-// seven blocks each, where 512 blocks of a pair each leave a fifth of the SM time idle.
+// the pointwise stage of a row pass at one point, z = (u, Lap u): the pair of pieces to
+// transform forward; density sums into red[0]
 template <typename T, int MODE>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, 7) col_pass_cl(const fch_kparams kp)
+__device__ __forceinline__ typename CT<T>::t pointwise_elem(const fch_kparams &kp, const fch_consts<T> &K,
+                                                            typename CT<T>::t z, T *red)
 {
     typedef typename CT<T>::t C;
-    typedef ColTraits<MODE> TR;
-    namespace cg = cooperative_groups;
-    pdl_begin();
-    if (pass_skipped(kp)) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red_scratch[FCH_NRED * 32];
-    constexpr int N = 1024, LOGN = 10, NT = 128;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank(), p = blockIdx.x >> 1;
-    C *tile = (C *)smem_raw;                      // own column, skewed
-    C *peer = cluster.map_shared_rank(tile, rank ^ 1); // the partner's column
-    const C *tw = (const C *)kp.tw;
-    const fch_consts<T> &K = consts<T>(kp);
-    const bool inv = TR::INV_ALWAYS || (TR::INV_OPT && (kp.flags & FCH_FL_PACK_F));
-    const bool has_red = MODE == CM_SAV_PQ || MODE == CM_PSD_ITER ||
-                         (MODE == CM_F_FINISH && (kp.flags & FCH_FL_AM3));
-    C *Z = pair_Z<C>(kp, N);
-    const int col = 2 * p + rank; // pair-layout slot of this block's column
-
-    fch_coef<T> co;
-    ColBufs<C> bf;
-    bf.i0 = (const C *)pair_in(kp.in0, kp);
-    bf.i1 = (const C *)pair_in(kp.in1, kp);
-    bf.o0 = (C *)pair_out(kp.out0, kp);
-    bf.o1 = (C *)pair_out(kp.out1, kp);
-    if (kp.ctrl) {
-        const fch_ctrl *cs = kp.ctrl;
-        co = load_coef<T>(cs);
-        bf.Un = (const C *)kp.U[cs->iu_n];
-        bf.Um = (const C *)kp.U[cs->iu_m];
-        bf.Unew = (C *)kp.U[cs->iu_new];
-        bf.Fn = (const C *)kp.F[cs->if_n];
-        bf.Fm = (const C *)kp.F[cs->if_m];
-        switch (kp.src) {
-        case FCH_SRC_UN: bf.src = bf.Un; bf.dst = (C *)kp.F[cs->if_n]; break;
-        case 5: bf.src = bf.Um; bf.dst = (C *)kp.F[cs->if_m]; break;
-        case FCH_SRC_UNEW: bf.src = bf.Unew; bf.dst = (C *)kp.F[cs->if_new]; break;
-        case FCH_SRC_V: bf.src = (const C *)kp.Vb; bf.dst = nullptr; break;
-        default: bf.src = (const C *)kp.in0; bf.dst = (C *)kp.out0; break;
-        }
-    } else {
-        bf.Un = bf.Um = bf.src = bf.Fn = bf.Fm = nullptr;
-        bf.Unew = bf.dst = nullptr;
-        co = fch_coef<T>();
+    const T u = z.x, lu = z.y; // u and Lap u
+    T W, W1, W2;
+    well<T>(K, u, W, W1, W2,
+            MODE == RM_SAV || MODE == RM_SAV_DIRECT || MODE == RM_ENERGY);
+    C o = mk<C>(0, 0);
+    if (MODE == RM_NIMEX || MODE == RM_NIMEX_DIRECT) {
+        // N_IMEX = [eps^2 (am - W'' + eta1) Lap u + W''W' - am^2 u - eta2 W'] + eps^2 Lap (am u - W')
+        o.x = rsub(rsub(radd(rmul(rmul(K.e2, radd(rsub(K.am, W2), K.eta1)), lu), rmul(W2, W1)),
+                        rmul(K.am2, u)),
+                   rmul(K.eta2, W1));
+        o.y = rsub(rmul(K.am, u), W1);
+    } else if (MODE == RM_F || MODE == RM_ENERGY) {
+        // mu = eps^2 Lap w - W'' w + eps^2 eta1 Lap u - eta2 W', w = eps^2 Lap u - W'
+        const T w = rsub(rmul(K.e2, lu), W1);
+        o.x = W1;
+        o.y = radd(rsub(rmul(-W2, w), rmul(K.eta2, W1)), rmul(rmul(K.e2, K.eta1), lu));
+        if (MODE == RM_ENERGY)
+            red[0] += (T)0.5 * w * w - K.eta2 * W + (T)0.5 * K.e2 * K.eta1 * u * lu;
+    } else if (MODE == RM_SAV || MODE == RM_SAV_DIRECT) {
+        // V = -eps^2 Lap (W' + zeta u) + [-eps^2 (W'' + zeta) Lap u + W' W'' - eta2 W']
+        o.x = radd(W1, rmul(K.zeta, u));
+        o.y = rsub(radd(rmul(rmul(-K.e2, radd(W2, K.zeta)), lu), rmul(W1, W2)), rmul(K.eta2, W1));
+        red[0] += -K.e2 * lu * (W1 + K.zeta * u) + (T)0.5 * W1 * W1 - K.eta2 * W;
     }
-
-    if (TR::FWD) {
-        C ld[8];
-#pragma unroll
-        for (int k = 0; k < 8; k++) ld[k] = Z[(long)(threadIdx.x + k * NT) * N + col];
-#pragma unroll
-        for (int k = 0; k < 8; k++) tile[skew(threadIdx.x + k * NT)] = ld[k];
-        fft_smem<-1, true>(tile, N, LOGN, 1, 0, tw, (int)threadIdx.x);
-    }
-    cluster.sync(); // both columns transformed (or, without a forward part, nothing read yet)
-
-    // slot 0 / slot 1 of the pair at skewed row r: own tile or the partner's
-    auto s0 = [&](int r) -> C & { return rank == 0 ? tile[skew(r)] : peer[skew(r)]; };
-    auto s1 = [&](int r) -> C & { return rank == 1 ? tile[skew(r)] : peer[skew(r)]; };
-    T red[FCH_NRED] = {0, 0, 0, 0};
-    if (p > 0) {
-        // items ky in [rank N/2, (rank + 1) N/2): rows ky of slot 0 and -ky of slot 1
-#pragma unroll 1
-        for (int it = 0; it < 4; it++) {
-            const int ky = rank * (N / 2) + threadIdx.x + it * NT;
-            const int mky = (N - ky) & (N - 1);
-            C A = mk<C>(0, 0), B = mk<C>(0, 0);
-            if (TR::FWD) {
-                const C z0 = s0(ky), z1 = cconj(s1(mky));
-                A = cscale_p2(badd(z0, z1), (T)0.5);
-                const C dm = bsub(z0, z1);
-                B = mk<C>(mul_p2(dm.y, (T)0.5), mul_p2(dm.x, (T)-0.5));
-            }
-            C Co = mk<C>(0, 0), Do = mk<C>(0, 0);
-            spec_elem<T, MODE>(kp, K, co, bf, p, ky, A, B, Co, Do, red);
-            if (inv) {
-                s0(ky) = mk<C>(rsub(Co.x, Do.y), radd(Co.y, Do.x));
-                s1(mky) = mk<C>(radd(Co.x, Do.y), rsub(Do.x, Co.y));
-            }
-        }
-    } else {
-        // pair 0: columns kx = 0 (slot 0) and kx = N/2 (slot 1), items ky in [0, N/2]
-        // (rows ky and -ky of both), even ky to rank 0 and odd ky to rank 1
-#pragma unroll 1
-        for (int ky = rank + 2 * (int)threadIdx.x; ky <= (N >> 1); ky += 2 * NT) {
-            const int mky = (N - ky) & (N - 1);
-            const int nrow = (ky == 0 || ky == (N >> 1)) ? 1 : 2;
-            C za[2], zb[2];
-            za[0] = s0(ky);
-            za[1] = s0(mky);
-            zb[0] = s1(ky);
-            zb[1] = s1(mky);
-            C outa[2], outb[2];
-#pragma unroll
-            for (int side = 0; side < 2; side++) {
-                const int kx = side ? (N >> 1) : 0;
-#pragma unroll
-                for (int rr = 0; rr < 2; rr++) {
-                    if (rr >= nrow) break;
-                    const int kyy = rr ? mky : ky;
-                    const C zr = side ? zb[rr] : za[rr];
-                    const C zo = side ? zb[rr ^ 1] : za[rr ^ 1];
-                    C A = mk<C>(0, 0), B = mk<C>(0, 0);
-                    if (TR::FWD) {
-                        const C z1 = cconj(zo);
-                        A = cscale_p2(badd(zr, z1), (T)0.5);
-                        const C dm = bsub(zr, z1);
-                        B = mk<C>(mul_p2(dm.y, (T)0.5), mul_p2(dm.x, (T)-0.5));
-                    }
-                    C Co = mk<C>(0, 0), Do = mk<C>(0, 0);
-                    spec_elem<T, MODE>(kp, K, co, bf, kx, kyy, A, B, Co, Do, red);
-                    const C o = mk<C>(rsub(Co.x, Do.y), radd(Co.y, Do.x));
-                    if (side)
-                        outb[rr] = o;
-                    else
-                        outa[rr] = o;
-                }
-            }
-            if (inv) {
-                s0(ky) = outa[0];
-                s1(ky) = outb[0];
-                if (nrow == 2) {
-                    s0(mky) = outa[1];
-                    s1(mky) = outb[1];
-                }
-            }
-        }
-    }
-    if (has_red) {
-        block_partials<2>(red, kp.part, red_scratch);
-        if (kp.tail_op >= 0) pass_tail(kp);
-    }
-    cluster.sync(); // every write into the partner's column is done and visible
-    if (inv) {
-        fft_smem<+1, true>(tile, N, LOGN, 1, 0, tw, (int)threadIdx.x);
-#pragma unroll
-        for (int k = 0; k < 8; k++) Z[(long)(threadIdx.x + k * NT) * N + col] = tile[skew(threadIdx.x + k * NT)];
-    }
+    return o;
 }
 
 // ---------------------------------------------------------------------------
 // row pass: [inverse rows] -> pointwise stage -> [forward rows]
-// Threads a compile-time row pass is built for: one row of 128 threads at N = 1024
-// (seven blocks an SM with at most 73 registers a thread: the 1024 rows run in one
-// wave on the 152 SMs, six or seven to an SM), N/8 at N = 2048, else 256.
-template <int LOGN> constexpr int row_threads()
+// The generic row pass: any N and number of rows a block, as tiles ask. PPT: points of a
+// row a thread transforms (8: radix-8 stages; 4: radix-4 stages and twice the threads,
+// twiddles from kp.tw4), as in col_pass.
+template <typename T, int MODE, int PPT = 8> __global__ void __launch_bounds__(256) row_pass(const fch_kparams kp)
 {
-    return LOGN == 10 ? 128 : (LOGN >= 11 ? (1 << LOGN) / 8 : 256);
-}
-template <int LOGN> constexpr int row_min_blocks()
-{
-    return LOGN == 10 ? 7 : pass_min_blocks<256, LOGN>();
-}
-
-// PPT: points of a row a thread transforms (8: radix-8 stages; 4, generic kernel only:
-// radix-4 stages and twice the threads, twiddles from kp.tw4), as in col_pass.
-template <typename T, int MODE, int LOGN, int PPT = 8>
-__global__ void __launch_bounds__(LOGN ? row_threads<LOGN>() : 256, LOGN ? row_min_blocks<LOGN>() : 1)
-row_pass(const fch_kparams kp)
-{
-    static_assert(PPT == 8 || (PPT == 4 && LOGN == 0), "four points a thread in the generic kernel only");
+    static_assert(PPT == 8 || PPT == 4, "eight or four points a thread");
     typedef typename CT<T>::t C;
     pdl_begin();
     if (pass_skipped(kp)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red_scratch[FCH_NRED * 32];
-    const int N = LOGN ? (1 << LOGN) : kp.N, tps = N / PPT, SL = skewed_len(N);
-    const int logN = LOGN ? LOGN : kp.logN;
-    const int nthr = LOGN ? row_threads<LOGN>() : (int)blockDim.x;
+    const int N = kp.N, tps = N / PPT, SL = skewed_len(N), logN = kp.logN, nthr = blockDim.x;
     if (kp.nfft && blockIdx.x == 0 && threadIdx.x == 0)
         atomicAdd(kp.nfft, (MODE == RM_R2C_LOAD || MODE == RM_C2R_STORE || MODE == RM_ENERGY) ? 2ull : 4ull);
     // twiddles stay in global memory (read-only cache): the shared memory holds
@@ -1046,38 +889,13 @@ row_pass(const fch_kparams kp)
                 }
                 continue;
             }
-            T W, W1, W2;
-            well<T>(K, u, W, W1, W2,
-                    MODE == RM_SAV || MODE == RM_SAV_DIRECT || MODE == RM_ENERGY ||
-                        (MODE == RM_F && (kp.flags & FCH_FL_ENERGY)));
-            C o = mk<C>(0, 0);
-            if (MODE == RM_NIMEX || MODE == RM_NIMEX_DIRECT) {
-                // N_IMEX = [eps^2 (am - W'' + eta1) Lap u + W''W' - am^2 u - eta2 W'] + eps^2 Lap (am u - W')
-                o.x = rsub(rsub(radd(rmul(rmul(K.e2, radd(rsub(K.am, W2), K.eta1)), lu), rmul(W2, W1)),
-                                rmul(K.am2, u)),
-                           rmul(K.eta2, W1));
-                o.y = rsub(rmul(K.am, u), W1);
-            } else if (MODE == RM_F || MODE == RM_ENERGY) {
-                // mu = eps^2 Lap w - W'' w + eps^2 eta1 Lap u - eta2 W', w = eps^2 Lap u - W'
-                const T w = rsub(rmul(K.e2, lu), W1);
-                o.x = W1;
-                o.y = radd(rsub(rmul(-W2, w), rmul(K.eta2, W1)), rmul(rmul(K.e2, K.eta1), lu));
-                if (MODE == RM_ENERGY || (kp.flags & FCH_FL_ENERGY))
-                    red[0] += (T)0.5 * w * w - K.eta2 * W + (T)0.5 * K.e2 * K.eta1 * u * lu;
-            } else if (MODE == RM_SAV || MODE == RM_SAV_DIRECT) {
-                // V = -eps^2 Lap (W' + zeta u) + [-eps^2 (W'' + zeta) Lap u + W' W'' - eta2 W']
-                o.x = radd(W1, rmul(K.zeta, u));
-                o.y = rsub(radd(rmul(rmul(-K.e2, radd(W2, K.zeta)), lu), rmul(W1, W2)), rmul(K.eta2, W1));
-                red[0] += -K.e2 * lu * (W1 + K.zeta * u) + (T)0.5 * W1 * W1 - K.eta2 * W;
-            }
-            s[skew(x)] = o;
+            s[skew(x)] = pointwise_elem<T, MODE>(kp, K, z, red);
         }
     }
-    const bool has_red = MODE == RM_SAV || MODE == RM_SAV_DIRECT || MODE == RM_ENERGY ||
-                         (MODE == RM_F && (kp.flags & FCH_FL_ENERGY));
+    constexpr bool has_red = MODE == RM_SAV || MODE == RM_SAV_DIRECT || MODE == RM_ENERGY;
     if (has_red) {
         block_partials<1>(red, kp.part, red_scratch);
-        if (kp.tail_op >= 0) pass_tail(kp);
+        if constexpr (row_tail_op(MODE) >= 0) pass_tail<row_tail_op(MODE)>(kp);
     }
     if (MODE == RM_C2R_STORE || MODE == RM_ENERGY) return;
 

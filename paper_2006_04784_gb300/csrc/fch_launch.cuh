@@ -34,46 +34,15 @@ inline cudaError_t set_smem(pass_fn f, int bytes, int floor_bytes, int &cur)
     return e;
 }
 
-// compile-time grid sizes: 512, 1024, 2048 (with FCH_ONLY_1024: 1024 only, which
-// keeps the double-float translation units small); others use the generic kernel
-template <typename T, int M> pass_fn col_fn(int logN)
+// the passes built for a grid size (fch_reg.cu): tile 0, N = 64 ... 2048, where the
+// twiddle tables are at hand (the radix-4 one: contexts and plans, not fch_fft_r2c_noalloc,
+// whose single-precision passes need the radix-8 one only)
+template <typename T> bool reg_applies(const fch_kparams &kp, int tile)
 {
-    switch (logN) {
-#ifndef FCH_ONLY_1024
-    case 9: return fch::col_pass<T, M, 9>;
-    case 11: return fch::col_pass<T, M, 11>;
-#endif
-    case 10: return fch::col_pass<T, M, 10>;
-    }
-    return fch::col_pass<T, M, 0>;
+    return tile == 0 && kp.logN >= 6 && kp.logN <= 11 && (sizeof(T) == 4 || kp.tw4);
 }
 
-// the slot of the kernel launched for a grid of 2^logN at the default tiles: logN
-// where a compile-time kernel is built in this translation unit, else 0 (the
-// generic kernel), so that one kernel has one shared-memory limit record
-inline int kernel_slot(int logN)
-{
-#ifndef FCH_ONLY_1024
-    if (logN == 9 || logN == 11) return logN;
-#endif
-    return logN == 10 ? 10 : 0;
-}
-
-template <typename T, int M> pass_fn row_fn(int logN)
-{
-    switch (logN) {
-#ifndef FCH_ONLY_1024
-    case 9: return fch::row_pass<T, M, 9>;
-    case 11: return fch::row_pass<T, M, 11>;
-#endif
-    case 10: return fch::row_pass<T, M, 10>;
-    }
-    return fch::row_pass<T, M, 0>;
-}
-
-// single precision at N = 1024: the warp-transform passes (one warp per sequence)
-template <typename T> constexpr bool warp_path() { return sizeof(T) == 4; }
-
+// single precision at N = 1024: the warp-transform columns (tile -2)
 template <int M> cudaError_t launch_col_w(const fch_kparams &kp, cudaStream_t s)
 {
     static int attr = 0;
@@ -84,29 +53,11 @@ template <int M> cudaError_t launch_col_w(const fch_kparams &kp, cudaStream_t s)
     return launch_pass(f, dim3(256, pair_grid(kp)), dim3(128), smem, s, kp);
 }
 
-template <int M> cudaError_t launch_row_w(const fch_kparams &kp, cudaStream_t s)
-{
-    return launch_pass(fch::row_pass_w<M>, dim3(1024, pair_grid(kp)), dim3(32), 0, s, kp);
-}
-
-// Tiles (fch_kparams::tile_col, tile_row): 0 takes the two-block-cluster column pass
-// for double and double-float at N = 1024, the warp-level row pass for single
-// precision at N = 1024, else the compile-time kernel of the grid size where one is
-// built, else the generic kernel; -1 the same without the clusters and the warp-level
-// rows; -2 (columns, single precision at N = 1024) the warp-level column pass; > 0 the
-// generic kernel with that many column pairs (rows) per block. The generic column
-// kernel reads P from kp.P, which the caller sets.
-// N = 1024, double and double-float: the column pass as clusters of two blocks
-template <typename T, int M> cudaError_t launch_col_cl(const fch_kparams &kp, cudaStream_t s)
-{
-    static int attr = 0;
-    const int smem = fch::skewed_len(1024) * (int)sizeof(typename fch::CT<T>::t);
-    pass_fn f = fch::col_pass_cl<T, M>;
-    cudaError_t e = set_smem(f, smem, 0, attr);
-    if (e != cudaSuccess) return e;
-    return launch_pass(f, dim3(1024, pair_grid(kp)), dim3(128), smem, s, kp);
-}
-
+// Tiles (fch_kparams::tile_col, tile_row): 0 takes the passes built for the grid size
+// (fch_reg.cu) where there are some, else the generic kernel; -1 the generic kernel at the
+// default geometry; -2 (columns, single precision at N = 1024) the warp-level column pass;
+// > 0 the generic kernel with that many column pairs (rows) per block; <= -3 the same at
+// four points a thread. The generic column kernel reads P from kp.P, which the caller sets.
 // N = 1024, single precision, the column passes of standalone transform plans (which
 // carry an error word): the persistent TMA-staged kernel, as many blocks as are
 // resident at once; the inverse needs 16-byte aligned half spectra (bulk copies)
@@ -150,14 +101,19 @@ template <int M> cudaError_t launch_col_t(const fch_kparams &kp, cudaStream_t s)
     return cudaErrorInvalidValue;
 }
 
+// whether a launch is a column pass of a single-precision plan at N = 1024: TMA-staged, or,
+// for half spectra off the bulk copies' alignment, the generic kernel, which computes the
+// same bit for bit
+template <typename T> bool plan_cols_1024(const fch_kparams &kp)
+{
+    return sizeof(T) == 4 && kp.err && kp.N == 1024;
+}
+
 template <typename T, int M> cudaError_t launch_col(const fch_kparams &kp, cudaStream_t s)
 {
     if constexpr (sizeof(T) == 4) {
         if (col_t_applies<M>(kp)) return launch_col_t<M>(kp, s);
-    }
-    if (warp_path<T>() && kp.N == 1024 && kp.tw2 && kp.tile_col == -2) return launch_col_w<M>(kp, s);
-    if constexpr (sizeof(T) == 8) {
-        if (kp.N == 1024 && kp.tile_col == 0) return launch_col_cl<T, M>(kp, s);
+        if (kp.N == 1024 && kp.tw2 && kp.tile_col == -2) return launch_col_w<M>(kp, s);
     }
     if (kp.tile_col <= -3) {
         // the generic kernel at four points a thread: needs the radix-4 twiddle table
@@ -165,40 +121,38 @@ template <typename T, int M> cudaError_t launch_col(const fch_kparams &kp, cudaS
         if (!kp.tw4) return cudaErrorInvalidValue;
         static int attr4 = 0;
         const fch_geom g = fch_geometry_tiled(kp.N, sizeof(T) == 4, 0, kp.tile_col);
-        pass_fn f = fch::col_pass<T, M, 0, 4>;
+        pass_fn f = fch::col_pass<T, M, 4>;
         cudaError_t e = set_smem(f, g.col_smem, 0, attr4);
         if (e != cudaSuccess) return e;
         return launch_pass(f, dim3(g.col_blocks, pair_grid(kp)), dim3(g.col_threads), g.col_smem, s, kp);
     }
-    static int attr[12] = {};
-    // the warp-level tile without its table (a context made with fft_path = 1) is -1
-    const int tc = kp.tile_col == -2 ? -1 : kp.tile_col;
+    static int attr = 0;
+    // the default tile without kernels built for the size, and the warp-level tile without
+    // its table (a context made with fft_path = 1), are -1
+    const int tc = kp.tile_col == -2 || kp.tile_col == 0 ? -1 : kp.tile_col;
     const fch_geom g = fch_geometry_tiled(kp.N, sizeof(T) == 4, 0, tc);
-    const int li = tc <= 0 ? kernel_slot(kp.logN) : 0;
-    pass_fn f = col_fn<T, M>(li);
-    cudaError_t e = set_smem(f, g.col_smem, fch_geometry(FCH_MAX_N, sizeof(T) == 4).col_smem, attr[li]);
+    pass_fn f = fch::col_pass<T, M, 8>;
+    cudaError_t e = set_smem(f, g.col_smem, fch_geometry(FCH_MAX_N, sizeof(T) == 4).col_smem, attr);
     if (e != cudaSuccess) return e;
     return launch_pass(f, dim3(g.col_blocks, pair_grid(kp)), dim3(g.col_threads), g.col_smem, s, kp);
 }
 
 template <typename T, int M> cudaError_t launch_row(const fch_kparams &kp, cudaStream_t s)
 {
-    if (warp_path<T>() && kp.N == 1024 && kp.tw2 && kp.tile_row == 0) return launch_row_w<M>(kp, s);
     if (kp.tile_row <= -3) {
         // the generic kernel at four points a thread (radix-4 twiddle table: contexts only)
         if (!kp.tw4) return cudaErrorInvalidValue;
         static int attr4 = 0;
         const fch_geom g = fch_geometry_tiled(kp.N, sizeof(T) == 4, kp.tile_row, 0);
-        pass_fn f = fch::row_pass<T, M, 0, 4>;
+        pass_fn f = fch::row_pass<T, M, 4>;
         cudaError_t e = set_smem(f, g.row_smem, 0, attr4);
         if (e != cudaSuccess) return e;
         return launch_pass(f, dim3(g.row_blocks, pair_grid(kp)), dim3(g.row_threads), g.row_smem, s, kp);
     }
-    static int attr[12] = {};
+    static int attr = 0;
     const fch_geom g = fch_geometry_tiled(kp.N, sizeof(T) == 4, kp.tile_row, 0);
-    const int li = kp.tile_row <= 0 ? kernel_slot(kp.logN) : 0;
-    pass_fn f = row_fn<T, M>(li);
-    cudaError_t e = set_smem(f, g.row_smem, fch_geometry(FCH_MAX_N, sizeof(T) == 4).row_smem, attr[li]);
+    pass_fn f = fch::row_pass<T, M, 8>;
+    cudaError_t e = set_smem(f, g.row_smem, fch_geometry(FCH_MAX_N, sizeof(T) == 4).row_smem, attr);
     if (e != cudaSuccess) return e;
     return launch_pass(f, dim3(g.row_blocks, pair_grid(kp)), dim3(g.row_threads), g.row_smem, s, kp);
 }
@@ -208,9 +162,22 @@ template <typename T, int M> cudaError_t launch_row(const fch_kparams &kp, cudaS
 #define FCH_CAT2(a, b) a##b
 #define FCH_CAT(a, b) FCH_CAT2(a, b)
 
+#define FCH_CAT3(a, b, c) a##b##_##c
+#define FCH_REG(a, b, c) FCH_CAT3(a, b, c)
+
 #ifndef FCH_NO_COL
 cudaError_t FCH_CAT(fch_launch_col_, FCH_SUFFIX)(int mode, const fch_kparams &kp, cudaStream_t s)
 {
+    if (reg_applies<FCH_T>(kp, kp.tile_col) && !plan_cols_1024<FCH_T>(kp)) {
+        switch (kp.logN) {
+        case 6: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 6)(mode, kp, s);
+        case 7: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 7)(mode, kp, s);
+        case 8: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 8)(mode, kp, s);
+        case 9: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 9)(mode, kp, s);
+        case 10: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 10)(mode, kp, s);
+        case 11: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 11)(mode, kp, s);
+        }
+    }
     switch (mode) {
     case CM_FWD_STORE: return launch_col<FCH_T, CM_FWD_STORE>(kp, s);
     case CM_INV_LOAD: return launch_col<FCH_T, CM_INV_LOAD>(kp, s);
@@ -231,6 +198,16 @@ cudaError_t FCH_CAT(fch_launch_col_, FCH_SUFFIX)(int mode, const fch_kparams &kp
 #ifndef FCH_NO_ROW
 cudaError_t FCH_CAT(fch_launch_row_, FCH_SUFFIX)(int mode, const fch_kparams &kp, cudaStream_t s)
 {
+    if (reg_applies<FCH_T>(kp, kp.tile_row)) {
+        switch (kp.logN) {
+        case 6: return FCH_REG(fch_reg_row_, FCH_SUFFIX, 6)(mode, kp, s);
+        case 7: return FCH_REG(fch_reg_row_, FCH_SUFFIX, 7)(mode, kp, s);
+        case 8: return FCH_REG(fch_reg_row_, FCH_SUFFIX, 8)(mode, kp, s);
+        case 9: return FCH_REG(fch_reg_row_, FCH_SUFFIX, 9)(mode, kp, s);
+        case 10: return FCH_REG(fch_reg_row_, FCH_SUFFIX, 10)(mode, kp, s);
+        case 11: return FCH_REG(fch_reg_row_, FCH_SUFFIX, 11)(mode, kp, s);
+        }
+    }
     switch (mode) {
     case RM_R2C_LOAD: return launch_row<FCH_T, RM_R2C_LOAD>(kp, s);
     case RM_C2R_STORE: return launch_row<FCH_T, RM_C2R_STORE>(kp, s);

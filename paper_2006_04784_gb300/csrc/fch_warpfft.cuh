@@ -1,14 +1,11 @@
-// fch_warpfft.cuh -- single-precision passes for N = 1024 built on a warp-level
-// transform: one warp owns one length-1024 sequence, 32 elements per lane.
+// fch_warpfft.cuh -- the single-precision column pass for N = 1024 built on a warp-level
+// transform (tile_col -2): one warp owns one length-1024 sequence, 32 elements per lane.
 //
 // With n = n1 + 32 n2 and k = k2 + 32 k1,
 //   X[k2 + 32 k1] = sum_{n1} W32^{n1 k1} W1024^{n1 k2} sum_{n2} W32^{n2 k2} x[n1 + 32 n2],
 // so lane n1 transforms its 32 elements x[n1 + 32 n2] in registers, multiplies by
 // W1024^{n1 k2}, the warp transposes through a padded 32 x 33 shared buffer, and
-// lane k2 transforms again, ending with X[k2 + 32 k1] in register k1. The output
-// layout of an inverse transform (lane = x mod 32, register = x / 32) is the input
-// layout of a forward one, so the pointwise stage of a row pass runs on registers
-// between the two transforms. Only __syncwarp is needed inside a transform.
+// lane k2 transforms again, ending with X[k2 + 32 k1] in register k1. Only __syncwarp is needed inside a transform.
 #pragma once
 #include "fch_kernels.cuh"
 
@@ -87,165 +84,6 @@ __device__ __forceinline__ void warp_fft1024(float2 *v, float2 *buf, const float
     RegFFT<32, DIR>::run(v);
 }
 
-// pointwise stage of a row pass on (u, Lap u); returns the pair to transform forward
-template <int MODE>
-__device__ __forceinline__ float2 pointwise(const fch_kparams &kp, const fch_consts<float> &K, float u,
-                                            float lu, float *red)
-{
-    float W, W1, W2;
-    well<float>(K, u, W, W1, W2,
-                MODE == RM_SAV || MODE == RM_SAV_DIRECT || MODE == RM_ENERGY ||
-                    (MODE == RM_F && (kp.flags & FCH_FL_ENERGY)));
-    float2 o = mk<float2>(0.f, 0.f);
-    if (MODE == RM_NIMEX || MODE == RM_NIMEX_DIRECT) {
-        o.x = K.e2 * (K.am - W2 + K.eta1) * lu + W2 * W1 - K.am2 * u - K.eta2 * W1;
-        o.y = K.am * u - W1;
-    } else if (MODE == RM_F || MODE == RM_ENERGY) {
-        const float w = K.e2 * lu - W1;
-        o.x = W1;
-        o.y = -W2 * w - K.eta2 * W1 + K.e2 * K.eta1 * lu;
-        if (MODE == RM_ENERGY || (kp.flags & FCH_FL_ENERGY))
-            red[0] += 0.5f * w * w - K.eta2 * W + 0.5f * K.e2 * K.eta1 * u * lu;
-    } else if (MODE == RM_SAV || MODE == RM_SAV_DIRECT) {
-        o.x = W1 + K.zeta * u;
-        o.y = -K.e2 * (W2 + K.zeta) * lu + W1 * W2 - K.eta2 * W1;
-        red[0] += -K.e2 * lu * (W1 + K.zeta * u) + 0.5f * W1 * W1 - K.eta2 * W;
-    }
-    return o;
-}
-
-// row pass, N = 1024, single precision: one warp (= one block) per row
-template <int MODE>
-// (the standalone transforms' row passes, launched over many field pairs, are built
-// for sixteen resident warps an SM: at most 128 registers a thread)
-__global__ void __launch_bounds__(32, (MODE == RM_R2C_LOAD || MODE == RM_C2R_STORE) ? 16 : 1)
-row_pass_w(const fch_kparams kp)
-{
-    typedef float2 C;
-    pdl_begin();
-    if (pass_skipped(kp)) return;
-    constexpr int N = 1024;
-    __shared__ __align__(16) C buf[33 * 32];
-    __shared__ double red_scratch[FCH_NRED * 32];
-    const int lane = threadIdx.x, y = blockIdx.x;
-    if (kp.nfft && blockIdx.x == 0 && lane == 0)
-        atomicAdd(kp.nfft, (MODE == RM_R2C_LOAD || MODE == RM_C2R_STORE || MODE == RM_ENERGY) ? 2ull : 4ull);
-    const C *tw2 = (const C *)kp.tw2;
-    const bool f64io = kp.flags & FCH_FL_F64IO;
-    C *row = pair_Z<C>(kp, N) + (long)y * N;
-    C v[32];
-    if (MODE == RM_NIMEX_DIRECT || MODE == RM_SAV_DIRECT) {
-        // (u*, Lap u*) pointwise from the stored real-space slots (eq. Richardson)
-        const fch_ctrl *cs = kp.ctrl;
-        const C *Rn = (const C *)kp.Rs[cs->iu_n] + (long)y * N;
-        const C *Rm = (const C *)kp.Rs[cs->iu_m] + (long)y * N;
-        const float g = cs->cof.gam;
-        const bool plain = (kp.flags & FCH_FL_GAMMA0) || g == 0.f;
-#pragma unroll
-        for (int n2 = 0; n2 < 32; n2++) {
-            const C zn = __ldg(Rn + lane + 32 * n2);
-            v[n2] = plain ? zn : cadd(zn, cscale(csub(zn, __ldg(Rm + lane + 32 * n2)), g));
-        }
-    } else if (MODE == RM_R2C_LOAD && !f64io && kp.in1) {
-        // two float fields (the common case, without a branch per element)
-        const float *a = (const float *)pair_in(kp.in0, kp) + (long)y * N + lane;
-        const float *b = (const float *)pair_in(kp.in1, kp) + (long)y * N + lane;
-#pragma unroll
-        for (int n2 = 0; n2 < 32; n2++) v[n2] = mk<C>(__ldcs(a + 32 * n2), __ldcs(b + 32 * n2));
-    } else if (MODE == RM_R2C_LOAD) {
-        const void *in0 = pair_in(kp.in0, kp), *in1 = pair_in(kp.in1, kp);
-#pragma unroll
-        for (int n2 = 0; n2 < 32; n2++) {
-            const long g = (long)y * N + lane + 32 * n2;
-            float a, b = 0.f;
-            if (f64io) {
-                a = (float)((const double *)in0)[g];
-                if (in1) b = (float)((const double *)in1)[g];
-            } else {
-                a = ((const float *)in0)[g];
-                if (in1) b = ((const float *)in1)[g];
-            }
-            v[n2] = mk<C>(a, b);
-        }
-    } else {
-        // pairs (kx, N-kx) of the pair-layout row into natural order, 16 per lane
-#pragma unroll
-        for (int j = 0; j < 16; j++) {
-            const int p = lane + 32 * j;
-            const float4 z = __ldcg((const float4 *)(row + 2 * p));
-            buf[p] = mk<C>(z.x, z.y);
-            buf[p ? N - p : N / 2] = mk<C>(z.z, z.w);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int n2 = 0; n2 < 32; n2++) v[n2] = buf[lane + 32 * n2];
-        warp_fft1024<+1>(v, buf, tw2, lane);
-    }
-
-    float red[FCH_NRED] = {0.f, 0.f, 0.f, 0.f};
-    C *store = nullptr;
-    if (MODE == RM_F && (kp.flags & FCH_FL_STORE_REAL)) {
-        const fch_ctrl *cs = kp.ctrl;
-        const int slot = kp.src == FCH_SRC_UNEW ? cs->iu_new : (kp.src == 5 ? cs->iu_m : cs->iu_n);
-        store = (C *)kp.Rs[slot] + (long)y * N;
-    }
-    if (MODE == RM_C2R_STORE && !f64io && kp.out0 && kp.out1) {
-        // two float fields (the common case, without a branch per element)
-        float *o0 = (float *)pair_out(kp.out0, kp) + (long)y * N + lane;
-        float *o1 = (float *)pair_out(kp.out1, kp) + (long)y * N + lane;
-#pragma unroll
-        for (int k1 = 0; k1 < 32; k1++) {
-            __stcs(o0 + 32 * k1, v[k1].x);
-            __stcs(o1 + 32 * k1, v[k1].y);
-        }
-        return;
-    }
-    if (MODE == RM_F && store) {
-#pragma unroll
-        for (int k1 = 0; k1 < 32; k1++) store[lane + 32 * k1] = v[k1];
-    }
-    if (MODE != RM_R2C_LOAD) {
-        const fch_consts<float> &K = kp.cf;
-#pragma unroll
-        for (int k1 = 0; k1 < 32; k1++) {
-            const int x = lane + 32 * k1;
-            const float u = v[k1].x, lu = v[k1].y;
-            if (MODE == RM_C2R_STORE) {
-                const long g = (long)y * N + x;
-                void *out0 = pair_out(kp.out0, kp), *out1 = pair_out(kp.out1, kp);
-                if (f64io) {
-                    if (out0) ((double *)out0)[g] = (double)u;
-                    if (out1) ((double *)out1)[g] = (double)lu;
-                } else {
-                    if (out0) ((float *)out0)[g] = u;
-                    if (out1) ((float *)out1)[g] = lu;
-                }
-                continue;
-            }
-            v[k1] = pointwise<MODE>(kp, K, u, lu, red);
-        }
-    }
-    const bool has_red = MODE == RM_SAV || MODE == RM_SAV_DIRECT || MODE == RM_ENERGY ||
-                         (MODE == RM_F && (kp.flags & FCH_FL_ENERGY));
-    if (has_red) {
-        block_partials<1>(red, kp.part, red_scratch);
-        if (kp.tail_op >= 0) pass_tail(kp);
-    }
-    if (MODE == RM_C2R_STORE || MODE == RM_ENERGY) return;
-
-    warp_fft1024<-1>(v, buf, tw2, lane);
-    __syncwarp();
-#pragma unroll
-    for (int k1 = 0; k1 < 32; k1++) buf[lane + 32 * k1] = v[k1];
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 16; j++) {
-        const int p = lane + 32 * j;
-        const C z0 = buf[p], z1 = buf[p ? N - p : N / 2];
-        __stcg((float4 *)(row + 2 * p), make_float4(z0.x, z0.y, z1.x, z1.y));
-    }
-}
-
 // column pass, N = 1024, single precision: P = 2 column pairs (4 columns) per
 // block, one warp per column; the tile rows are padded to 5 elements so a warp
 // reading one column of consecutive rows hits distinct banks.
@@ -271,28 +109,9 @@ __global__ void __launch_bounds__(128) col_pass_w(const fch_kparams kp)
                          (MODE == CM_F_FINISH && (kp.flags & FCH_FL_AM3));
     C *Z = pair_Z<C>(kp, N);
 
-    fch_coef<float> co = fch_coef<float>();
-    ColBufs<C> bf = ColBufs<C>();
-    bf.i0 = (const C *)pair_in(kp.in0, kp);
-    bf.i1 = (const C *)pair_in(kp.in1, kp);
-    bf.o0 = (C *)pair_out(kp.out0, kp);
-    bf.o1 = (C *)pair_out(kp.out1, kp);
-    if (kp.ctrl) {
-        const fch_ctrl *cs = kp.ctrl;
-        co = load_coef<float>(cs);
-        bf.Un = (const C *)kp.U[cs->iu_n];
-        bf.Um = (const C *)kp.U[cs->iu_m];
-        bf.Unew = (C *)kp.U[cs->iu_new];
-        bf.Fn = (const C *)kp.F[cs->if_n];
-        bf.Fm = (const C *)kp.F[cs->if_m];
-        switch (kp.src) {
-        case FCH_SRC_UN: bf.src = bf.Un; bf.dst = (C *)kp.F[cs->if_n]; break;
-        case 5: bf.src = bf.Um; bf.dst = (C *)kp.F[cs->if_m]; break;
-        case FCH_SRC_UNEW: bf.src = bf.Unew; bf.dst = (C *)kp.F[cs->if_new]; break;
-        case FCH_SRC_V: bf.src = (const C *)kp.Vb; bf.dst = nullptr; break;
-        default: bf.src = (const C *)kp.in0; bf.dst = (C *)kp.out0; break;
-        }
-    }
+    fch_coef<float> co;
+    ColBufs<C> bf;
+    load_colbufs<float>(kp, co, bf);
 
     if (TR::FWD) {
         // 4096 tile elements, 32 per thread, in 4 batches of 8 loads in flight
@@ -387,7 +206,7 @@ __global__ void __launch_bounds__(128) col_pass_w(const fch_kparams kp)
     }
     if (has_red) {
         block_partials<2>(red, kp.part, red_scratch);
-        if (kp.tail_op >= 0) pass_tail(kp);
+        if constexpr (col_tail_op(MODE) >= 0) pass_tail<col_tail_op(MODE)>(kp);
     }
     if (inv) {
         __syncthreads();
