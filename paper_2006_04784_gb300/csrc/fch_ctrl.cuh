@@ -23,29 +23,27 @@ __device__ __forceinline__ void pdl_begin()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Double-precision reciprocal and sixth root from single-precision seeds and
-// Newton steps (two steps take a 1e-7 seed to full double precision). This
-// GPU's double pipe is slow and the controller runs on one thread, so the
-// short dependent chains matter.
+// Double-precision reciprocal and sixth root: one step of third order from a
+// single-precision seed (relative error e < 2^-21: the step leaves e^3, below double
+// rounding). The controller is a chain of dependent operations on a slow double pipe, and
+// a third-order step is three of them where two Newton steps are four (the root: nine
+// where two Newton steps and the powers are sixteen).
 __device__ inline double rcp_nr(double a)
 {
-    double r = (double)(1.0f / (float)a);
-    r = r * (2.0 - a * r);
-    r = r * (2.0 - a * r);
-    return r;
+    const double r = (double)(1.0f / (float)a), e = fma(-a, r, 1.0);
+    return fma(r, fma(e, e, e), r); // 1/a = r / (1 - e) = r (1 + e + e^2 + ...)
 }
 
-// x^(1/6) for x in [1e-30, 1e30]: z = x^(-1/6) by Newton on z^-6 = x, then x z^5
+// x^(1/6) for x in [1e-30, 1e30]: z = x^(-1/6) from a seed, with d = 1 - x z^6 the root is
+// z (1 - d)^(-1/6) = z (1 + d/6 + 7 d^2/72 + ...); then x z^5
 __device__ inline double root6_nr(double x)
 {
-    double z = (double)powf((float)x, -1.0f / 6.0f);
-#pragma unroll
-    for (int i = 0; i < 2; i++) {
-        const double z2 = z * z, z6 = z2 * z2 * z2;
-        z = z * (7.0 - x * z6) * (1.0 / 6.0);
-    }
-    const double z2 = z * z;
-    return x * z2 * z2 * z;
+    const double z = (double)powf((float)x, -1.0f / 6.0f);
+    const double z2 = z * z, z4 = z2 * z2;
+    const double d = fma(-x, z4 * z2, 1.0);
+    const double y = fma(z * d, fma(d, 7.0 / 72.0, 1.0 / 6.0), z);
+    const double y2 = y * y;
+    return (x * y) * (y2 * y2);
 }
 
 // one control operation; returns false when the run stopped (done or failure). The
@@ -54,53 +52,7 @@ __device__ inline double root6_nr(double x)
 template <int OP>
 __device__ __forceinline__ bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, double S0, double S1, double arg0)
 {
-    if constexpr (OP == OP_INIT_TRIAL) {
-        double k1;
-        if (arg0 > 0) {
-            k1 = arg0; // fixed step
-        } else {
-            const double rem = c->t_final - c->t;
-            if (rem <= 1e-12 * fmax(1.0, fabs(c->t_final))) {
-                c->done = 1;
-                return false;
-            }
-            k1 = fmin(c->ktrial, rem); // the run ends exactly at t_final
-        }
-        c->k1 = k1;
-        if (c->kn <= 0) { // backward-Euler start: k_{n-1} -> infinity in eq. (BDF2Coef)
-            const double r1 = rcp_nr(k1);
-            c->a = r1;
-            c->b = -r1;
-            c->c = 0.0;
-            c->gam = 0.0;
-        } else {
-            // eq. (BDF2Coef) and the eq. (Predictor) weights from three independent
-            // reciprocals (1/(1+gam) = k_n/(k_{n+1}+k_n)), so their latencies overlap
-            const double kn = c->kn;
-            const double r1 = rcp_nr(k1), rn = rcp_nr(kn), rs = rcp_nr(k1 + kn);
-            c->a = r1 + rs;
-            c->b = -r1 - rn;
-            c->c = rn - rs;
-            const double g = k1 * rn;
-            c->gam = g;
-            const double k6 = k1 * (1.0 / 6.0), ig = kn * rs; // 1/(1+g)
-            c->w1 = k6 * (3.0 + 2.0 * g) * ig;
-            c->w2 = k6 * (3.0 + g);
-            c->w3 = -k6 * g * g * ig;
-        }
-        // PSD search step: Table SearchSize row, linear in k, clamped (slopes precomputed)
-        if (c->lam_k[0] < 0 || k1 <= c->lam_k[0]) {
-            c->lam = c->lam_tab[0];
-        } else if (k1 >= c->lam_k[9]) {
-            c->lam = c->lam_tab[9];
-        } else {
-            int j = 0;
-            while (j < 8 && k1 > c->lam_k[j + 1]) j++;
-            c->lam = c->lam_tab[j] + (k1 - c->lam_k[j]) * c->lam_slope[j];
-        }
-        c->psd_conv = 0;
-        c->psd_iter = 0;
-    } else if constexpr (OP == OP_SAV_E1) {
+    if constexpr (OP == OP_SAV_E1) {
         const double e1 = kp.h2 * S0;
         const double v = e1 + kp.D0;
         if (!isfinite(v) || v <= 0) {
@@ -200,6 +152,69 @@ __device__ __forceinline__ bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, doub
     return !c->done;
 }
 
+// The set-up of a trial of size arg0 (fixed step) or, where arg0 <= 0, of the next adaptive
+// trial: by one warp. Lane 0 has run whatever came before; the lanes compute the same
+// coefficients, and ten of them look the PSD search step up at once.
+__device__ __forceinline__ void ctrl_init_trial(fch_ctrl *c, double arg0, int lane)
+{
+    double k1;
+    if (arg0 > 0) {
+        k1 = arg0; // fixed step
+    } else {
+        const double rem = c->t_final - c->t;
+        if (rem <= 1e-12 * fmax(1.0, fabs(c->t_final))) {
+            __syncwarp();
+            c->done = 1;
+            return;
+        }
+        k1 = fmin(c->ktrial, rem); // the run ends exactly at t_final
+    }
+    const double kn = c->kn;
+    double a, b, cc, g, w1 = c->w1, w2 = c->w2, w3 = c->w3;
+    if (kn <= 0) { // backward-Euler start: k_{n-1} -> infinity in eq. (BDF2Coef)
+        a = rcp_nr(k1);
+        b = -a;
+        cc = 0.0;
+        g = 0.0;
+    } else {
+        // eq. (BDF2Coef) and the eq. (Predictor) weights from three independent
+        // reciprocals (1/(1+gam) = k_n/(k_{n+1}+k_n)), so their latencies overlap
+        const double r1 = rcp_nr(k1), rn = rcp_nr(kn), rs = rcp_nr(k1 + kn);
+        a = r1 + rs;
+        b = -r1 - rn;
+        cc = rn - rs;
+        g = k1 * rn;
+        const double k6 = k1 * (1.0 / 6.0), ig = kn * rs; // 1/(1+g)
+        w1 = k6 * (3.0 + 2.0 * g) * ig;
+        w2 = k6 * (3.0 + g);
+        w3 = -k6 * g * g * ig;
+    }
+    // PSD search step: Table SearchSize row, linear in k, clamped (slopes precomputed)
+    const unsigned above = __ballot_sync(0xffffffffu, lane < 10 && k1 > c->lam_k[lane < 10 ? lane : 0]);
+    const int j = c->lam_k[0] < 0 ? -1 : __popc(above) - 1; // last knot below k1
+    double lam;
+    if (j < 0)
+        lam = c->lam_tab[0];
+    else if (k1 >= c->lam_k[9])
+        lam = c->lam_tab[9];
+    else
+        lam = c->lam_tab[j] + (k1 - c->lam_k[j]) * c->lam_slope[j];
+    __syncwarp(); // every lane has read the old values
+    if (lane == 0) {
+        c->k1 = k1;
+        c->a = a;
+        c->b = b;
+        c->c = cc;
+        c->gam = g;
+        c->w1 = w1;
+        c->w2 = w2;
+        c->w3 = w3;
+        c->lam = lam;
+        c->psd_conv = 0;
+        c->psd_iter = 0;
+    }
+}
+
 // Float, double and double-float mirrors of the per-trial coefficients read by
 // the passes, lane i of the calling warp converting coefficient i: conversions run
 // on the double pipe, where one warp instruction costs the same for eleven lanes as
@@ -220,55 +235,77 @@ __device__ inline void sync_coef_lanes(fch_ctrl *c, int lane)
 }
 
 
-// The whole control step by one block (any multiple of 32 threads up to 1024):
-// the control block is staged through shared memory with coalesced copies, the
-// first na partials of slots 0 and 1 are summed in a fixed order (per-thread
-// strided sums, warp shuffles, then thread 0 over the warp sums), thread 0 runs
-// the operation, and the block writes the control block back.
+// block sums an operation reads: slots 0 and 1, slot 0, or none
+template <int OP> constexpr int ctrl_slots()
+{
+    return OP == OP_DECIDE_INIT || OP == OP_SAV_R || OP == OP_PSD_CHECK ? 2 : OP == OP_SAV_E1 || OP == OP_ENERGY ? 1 : 0;
+}
+
+// The whole control step by one block (any multiple of 32 threads up to 1024): the control
+// block is staged through shared memory with coalesced copies, the first na partials of
+// the slots the operation reads are summed in a fixed order, warp 0 runs the operation, and
+// the block writes the control block back. What it costs is double-precision instructions
+// (one warp instruction holds the pipe 16 cycles whatever its lanes do) and their chains:
+// both slots are reduced in the two halves of a warp at once, and the warp sums by a second
+// shuffle tree.
 template <int OP> __device__ __forceinline__ void ctrl_block(const fch_kparams &kp, int na, double arg0)
 {
+    constexpr int slots = ctrl_slots<OP>();
     __shared__ double sh[2][32];
     __shared__ fch_ctrl cs;
     const int nw = (int)(sizeof(fch_ctrl) / 8);
-    const int nthr = blockDim.x;
+    const int nthr = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < nw; i += nthr) ((long long *)&cs)[i] = ((const long long *)kp.ctrl)[i];
     // the partial sums load while the control block arrives (discarded if it says done)
     double s0 = 0, s1 = 0;
-    for (int i = threadIdx.x; i < na; i += nthr) {
-        s0 += kp.part[i];
-        s1 += kp.part[FCH_MAXBLK + i];
+    if (slots > 0) {
+        for (int i = threadIdx.x; i < na; i += 4 * nthr) {
+            double v0[4], v1[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const int j = i + k * nthr;
+                v0[k] = j < na ? kp.part[j] : 0.0;
+                v1[k] = slots > 1 && j < na ? kp.part[FCH_MAXBLK + j] : 0.0;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (i + k * nthr >= na) break;
+                s0 += v0[k];
+                if (slots > 1) s1 += v1[k];
+            }
+        }
+        // lanes 0-15 go on with slot 0, lanes 16-31 with slot 1
+        double v = lane < 16 ? s0 : s1;
+        v += __shfl_xor_sync(0xffffffffu, lane < 16 ? s1 : s0, 16);
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, 16);
+        if ((lane & 15) == 0) sh[lane >> 4][warp] = v;
     }
     __syncthreads();
     if (cs.done && !(kp.flags & FCH_FL_NOSKIP)) return;
     if (OP == OP_PSD_CHECK && cs.psd_conv) return;
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_down_sync(0xffffffffu, s0, o);
-        s1 += __shfl_down_sync(0xffffffffu, s1, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = s0;
-        sh[1][threadIdx.x >> 5] = s1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         double S0 = 0, S1 = 0;
-        for (int w = 0; w < (nthr >> 5); w++) {
-            S0 += sh[0][w];
-            S1 += sh[1][w];
+        if (slots > 0) {
+            const int w = nthr >> 5, l = lane & 15, h = lane >> 4;
+            double v = l < w ? sh[h][l] : 0.0;
+            if (w > 16) v += l + 16 < w ? sh[h][l + 16] : 0.0;
+            for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, 16);
+            S0 = __shfl_sync(0xffffffffu, v, 0);
+            S1 = __shfl_sync(0xffffffffu, v, 16);
         }
         // the combined operations: the decision (adaptive) or the acceptance of a fixed
         // step, then the set-up of the next trial (adaptive: -1; fixed: arg0 = dt)
-        if constexpr (OP == OP_DECIDE_INIT) {
-            if (ctrl_op<OP_DECIDE>(&cs, kp, S0, S1, arg0)) ctrl_op<OP_INIT_TRIAL>(&cs, kp, S0, S1, -1.0);
-        } else if constexpr (OP == OP_ACCEPT_INIT) {
-            if (ctrl_op<OP_ACCEPT>(&cs, kp, S0, S1, 0.0)) ctrl_op<OP_INIT_TRIAL>(&cs, kp, S0, S1, arg0);
-        } else {
-            ctrl_op<OP>(&cs, kp, S0, S1, arg0);
+        constexpr int FIRST = OP == OP_DECIDE_INIT ? OP_DECIDE : OP == OP_ACCEPT_INIT ? OP_ACCEPT : OP;
+        bool go = true;
+        if (FIRST != OP_INIT_TRIAL) {
+            if (lane == 0) go = ctrl_op<FIRST>(&cs, kp, S0, S1, OP == OP_ACCEPT_INIT ? 0.0 : arg0);
+            go = __shfl_sync(0xffffffffu, go, 0);
         }
-    }
-    if (threadIdx.x < 32) {
         __syncwarp();
-        sync_coef_lanes(&cs, threadIdx.x);
+        if ((OP == OP_INIT_TRIAL || OP == OP_DECIDE_INIT || OP == OP_ACCEPT_INIT) && go)
+            ctrl_init_trial(&cs, OP == OP_DECIDE_INIT ? -1.0 : arg0, lane);
+        __syncwarp();
+        sync_coef_lanes(&cs, lane);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nw; i += nthr) ((long long *)kp.ctrl)[i] = ((const long long *)&cs)[i];
