@@ -491,6 +491,7 @@ static void fill_consts(fch_consts<T> &k, const fch_params &p, double kf, double
     k.bm = (T)p.b_minus;
     k.bp = (T)p.b_plus;
     k.eps = (T)p.eps;
+    k.ieps = (T)(1.0 / p.eps);
     k.q = (T)p.q;
     k.qeps = (T)(p.q * p.eps);
     k.qoe = (T)(p.q / p.eps);
@@ -2434,6 +2435,26 @@ extern "C" int fch_debug_twiddles(int n, int lp, double *out)
     if (!pow2_in_range(n) || (lp != 2 && lp != 3) || !out) return 1;
     make_twiddles(n, out, lp);
     return 0;
+}
+
+__global__ void fch_debug_dfl_exp_kernel(const double *x, double *ex, double *em, long cnt)
+{
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= cnt) return;
+    ex[i] = (double)fch::exp(fch::df(x[i]));
+    em[i] = (double)fch::expm1(fch::df(x[i]));
+}
+
+// test hook: the double-float exp and expm1 on cnt device doubles (rounded to
+// double-float first); 0 or a status
+extern "C" int fch_debug_dfl_exp(const double *x, double *ex, double *em, long cnt, void *stream)
+{
+    if (!x || !ex || !em || cnt < 1) return FCH_EINVAL;
+    cudaStream_t s = (cudaStream_t)stream;
+    fch_debug_dfl_exp_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(x, ex, em, cnt);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e == cudaSuccess ? FCH_OK : FCH_ECUDA;
 }
 
 // which trials and fixed steps of a context replay a captured graph (tests):

@@ -11,8 +11,8 @@
 // Addition sums the high parts with TwoSum and the low parts with one rounding
 // (error bounded relative to the operands); multiplication adds the cross terms to
 // the exact product of the high parts; division refines a float quotient with two
-// correction terms, the reciprocal takes one Newton step. Transcendental functions
-// (used only by the q > 0 well and the ETD phi functions) go through double.
+// correction terms, the reciprocal takes one Newton step. exp and expm1 (the q > 0 well and the ETD phi
+// functions) are table-driven on the FP32 pipe.
 // Compile without fast-math: the transformations rely on IEEE rounding of each step.
 #pragma once
 #include <math.h>
@@ -238,7 +238,91 @@ __device__ __forceinline__ df copysign(df a, df s)
     s = renorm_exact(s);
     return (a.hi < 0.f) != (s.hi < 0.f) ? -a : a;
 }
-__device__ __forceinline__ df exp(df a) { return df(::exp((double)a)); }
-__device__ __forceinline__ df expm1(df a) { return df(::expm1((double)a)); }
+
+// exp and expm1 on the FP32 pipe, table-driven (P. T. P. Tang, "Table-driven implementation
+// of the exponential function in IEEE floating-point arithmetic", 1989): a = n ln2/32 + r,
+// |r| <= ln2/64; e^a = 2^(n/32) (1 + p), p = e^r - 1 by the series (terms from r^4/4! on in
+// single precision: they are below 2^-30), 2^(n/32) = 2^e T_j from the table. ln2/32 is split
+// in three floats: n L1 cancels against a.hi without rounding (fused multiply-add), n L2 is
+// an exact product. Relative error below 2^-47 (the format's own rounding is 2^-48); the
+// double pipe's exp costs some twenty double operations a point, 64 FP32 issue slots each.
+__device__ const float2 kExp2Tab[32] = { // 2^(j/32) = hi + lo
+    {0x1.0p+0f, 0x0.0p+0f}, {0x1.059b0ep+0f, -0x1.9d4f52p-25f}, {0x1.0b5586p+0f, 0x1.9f3122p-25f}, {0x1.11301ep+0f, -0x1.fdb496p-25f},
+    {0x1.172b84p+0f, -0x1.c15742p-27f}, {0x1.1d4874p+0f, -0x1.d2e8cap-25f}, {0x1.2387a6p+0f, 0x1.ceac48p-25f}, {0x1.29e9ep+0f, -0x1.5c0424p-25f},
+    {0x1.306fep+0f, 0x1.4636e2p-25f}, {0x1.371a74p+0f, -0x1.18aac6p-25f}, {0x1.3dea64p+0f, 0x1.824684p-25f}, {0x1.44e086p+0f, 0x1.8624b4p-30f},
+    {0x1.4bfdaep+0f, -0x1.593abcp-25f}, {0x1.5342b6p+0f, -0x1.2c561p-25f}, {0x1.5ab07ep+0f, -0x1.5bd5ecp-27f}, {0x1.6247ecp+0f, -0x1.f8b55p-25f},
+    {0x1.6a09e6p+0f, 0x1.9fcef4p-26f}, {0x1.71f75ep+0f, 0x1.1d8beep-25f}, {0x1.7a1148p+0f, -0x1.829fdp-25f}, {0x1.82589ap+0f, -0x1.accc7cp-26f},
+    {0x1.8ace54p+0f, 0x1.15506ep-27f}, {0x1.93737cp+0f, -0x1.e64744p-25f}, {0x1.9c4918p+0f, 0x1.51f848p-27f}, {0x1.a5503cp+0f, -0x1.b83b54p-25f},
+    {0x1.ae89fap+0f, -0x1.a94b14p-26f}, {0x1.b7f77p+0f, -0x1.a09438p-25f}, {0x1.c199bep+0f, -0x1.3d56b2p-27f}, {0x1.cb720ep+0f, -0x1.8837ccp-27f},
+    {0x1.d5818ep+0f, -0x1.822dbcp-27f}, {0x1.dfc974p+0f, -0x1.908c94p-25f}, {0x1.ea4afap+0f, 0x1.52486cp-27f}, {0x1.f50766p+0f, -0x1.246ebp-26f},
+};
+
+struct df_exp_parts {
+    df T, p; // 2^(j/32), e^r - 1
+    int e;   // binary exponent
+};
+__device__ __forceinline__ df_exp_parts exp_parts(df a)
+{
+    const float n = rintf(a.hi * 0x1.715476p+5f); // 32 / ln 2
+    const float r1 = fmaf(-n, 0x1.62e43p-6f, a.hi); // exact
+    const float p2 = __fmul_rn(n, 0x1.05c61p-34f), pe = fmaf(n, 0x1.05c61p-34f, -p2);
+    const df s = two_sum(p2, a.lo);
+    df r = two_sum(r1, s.hi);
+    r.lo += s.lo + fmaf(n, 0x1.950d88p-59f, pe);
+    const float q = fmaf(r.hi, fmaf(r.hi, (float)(1.0 / 720), (float)(1.0 / 120)), (float)(1.0 / 24));
+    df c = two_sum((float)(1.0 / 6), __fmul_rn(r.hi, q));
+    c.lo += (float)(1.0 / 6 - (double)(float)(1.0 / 6));
+    c = mul_lazy(c, r);
+    df h = two_sum(0.5f, c.hi);
+    h.lo += c.lo;
+    df_exp_parts o;
+    o.p = add_lazy(r, mul_lazy(mul_lazy(r, r), h)); // r + r^2 (1/2 + r (1/6 + r q))
+    const int N = (int)n;
+    const float2 t = __ldg(kExp2Tab + (N & 31));
+    o.T = df(t.x, t.y);
+    o.e = N >> 5;
+    return o;
+}
+// x 2^e for any e (two factors where 2^e is below the normal range)
+__device__ __forceinline__ df scale2(df x, int e)
+{
+    const int e1 = max(e, -126), e2 = max(e - e1, -126);
+    const float f1 = __int_as_float((e1 + 127) << 23), f2 = __int_as_float((e2 + 127) << 23);
+    return df(x.hi * f1 * f2, x.lo * f1 * f2);
+}
+__device__ __forceinline__ df exp(df a)
+{
+    if (a.hi < -200.0f) return df(0.f, 0.f); // far below the underflow, -inf too (its low word is NaN)
+    a = renorm_exact(a);
+    if (!(a.hi < 88.0f)) return df(::exp((double)a)); // near and above the overflow of a float, NaN
+    const df_exp_parts x = exp_parts(a);
+    return scale2(renorm(add_lazy(x.T, mul_lazy(x.T, x.p))), x.e);
+}
+// expm1: the series below 0.35, where e^a - 1 would cancel
+__device__ __forceinline__ df expm1(df a)
+{
+    if (a.hi < -200.0f) return df(-1.f, 0.f);
+    a = renorm_exact(a);
+    if (!(a.hi < 88.0f)) return df(::expm1((double)a));
+    if (::fabsf(a.hi) < 0.35f) {
+        // a + a^2 (1/2! + a (1/3! + ...)), terms from a^9/9! on in single precision
+        float t = (float)(1.0 / 87178291200.0);
+        t = fmaf(t, a.hi, (float)(1.0 / 6227020800.0));
+        t = fmaf(t, a.hi, (float)(1.0 / 479001600.0));
+        t = fmaf(t, a.hi, (float)(1.0 / 39916800.0));
+        t = fmaf(t, a.hi, (float)(1.0 / 3628800.0));
+        t = fmaf(t, a.hi, (float)(1.0 / 362880.0));
+        df s(t, 0.f);
+        const double c[7] = {1.0 / 40320, 1.0 / 5040, 1.0 / 720, 1.0 / 120, 1.0 / 24, 1.0 / 6, 1.0 / 2};
+#pragma unroll
+        for (int i = 0; i < 7; i++) s = add_lazy(df(c[i]), mul_lazy(s, a));
+        return renorm(add_lazy(a, mul_lazy(mul_lazy(a, a), s)));
+    }
+    const df_exp_parts x = exp_parts(a);
+    const df T = scale2(x.T, x.e);
+    df d = two_sum(T.hi, -1.0f);
+    d.lo += T.lo;
+    return renorm(add_lazy(d, mul_lazy(T, x.p)));
+}
 
 } // namespace fch

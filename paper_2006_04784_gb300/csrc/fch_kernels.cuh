@@ -23,6 +23,7 @@
 #pragma once
 #include <cooperative_groups.h>
 #include <math.h>
+#include <type_traits>
 #include "fch_ctrl.cuh"
 #include "fch_df.cuh"
 #include "fch_internal.h"
@@ -267,23 +268,21 @@ __device__ __forceinline__ void well(const fch_consts<T> &k, T u, T &W, T &W1, T
         return;
     }
     const T v = rsub(u, k.bm);
-    T A = mul_p2(rmul(v, v), (T)0.5), A1 = v, A2 = (T)1;
-    if (k.q != (T)0) {
-        const T x = v / k.eps;
-        const T e = exp(-fabs(x)); // e^{-|x|} in (0, 1]
-        const T id = recip((T)1 + e * e);
-        const T sech = mul_p2(e * id, (T)2);
-        const T th = copysign(((T)1 - e * e) * id, x);
-        A += k.qeps * ((T)1 - sech);
-        A1 += k.q * sech * th;
-        A2 += k.qoe * sech * (mul_p2(sech * sech, (T)2) - (T)1);
-    }
+    // x = v / eps: the product with 1 / eps and one correction
+    const T x0 = rmul(v, k.ieps), x = radd(x0, rmul(rsub(v, rmul(x0, k.eps)), k.ieps));
+    const T e = exp(-fabs(x)); // e^{-|x|} in (0, 1]
+    const T e2 = rmul(e, e), id = recip(radd((T)1, e2));
+    const T sech = mul_p2(rmul(e, id), (T)2);
+    const T th = copysign(rmul(rsub((T)1, e2), id), x);
+    const T A = radd(mul_p2(rmul(v, v), (T)0.5), rmul(k.qeps, rsub((T)1, sech)));
+    const T A1 = radd(v, rmul(rmul(k.q, sech), th));
+    const T A2 = radd((T)1, rmul(rmul(k.qoe, sech), rsub(mul_p2(rmul(sech, sech), (T)2), (T)1)));
     const T w = rsub(u, k.bp);
     const T B = radd(mul_p2(rmul(w, w), (T)0.5), rmul(k.g3, rsub(u, k.c3)));
     const T B1 = radd(w, k.g3);
     W = rmul(A, B);
     W1 = radd(rmul(A1, B), rmul(A, B1));
-    W2 = radd(radd(k.q != (T)0 ? rmul(A2, B) : B, mul_p2(rmul(A1, B1), (T)2)), A);
+    W2 = radd(radd(rmul(A2, B), mul_p2(rmul(A1, B1), (T)2)), A);
 }
 
 // ---------------------------------------------------------------------------
@@ -345,13 +344,14 @@ __device__ __forceinline__ bool pass_skipped(const fch_kparams &kp)
 
 // ---------------------------------------------------------------------------
 // ETD phi functions in precision T: phi1 = (e^z - 1)/z, phi2 = (e^z - 1 - z)/z^2.
-// Below a threshold (1e-2 in double, 0.1 in float, where the direct forms lose
-// digits to cancellation) the Taylor series sum_j z^j/(j+1)!, sum_j z^j/(j+2)!
-// in Horner form, j < 10; the direct forms above.
+// Below a threshold (1e-2 in double, 0.1 in float and double-float, where the direct forms
+// lose digits to cancellation) the Taylor series sum_j z^j/(j+1)!, sum_j z^j/(j+2)!
+// in Horner form, j < 10; the direct forms above (double-float: one reciprocal).
 template <typename T> __device__ __forceinline__ void etd_phi(T z, T &ez, T &p1, T &p2)
 {
+    constexpr bool dfl = std::is_same<T, df>::value;
     ez = exp(z);
-    const T thr = sizeof(T) == 8 ? (T)1e-2 : (T)0.1;
+    const T thr = std::is_same<T, double>::value ? (T)1e-2 : (T)0.1;
     if (fabs(z) < thr) {
         // inverse factorials 1/1! .. 1/11!
         const T f[11] = {(T)1.0, (T)(1.0 / 2), (T)(1.0 / 6), (T)(1.0 / 24), (T)(1.0 / 120),
@@ -360,15 +360,21 @@ template <typename T> __device__ __forceinline__ void etd_phi(T z, T &ez, T &p1,
         T a = f[9], b = f[10];
 #pragma unroll
         for (int j = 8; j >= 0; j--) {
-            a = a * z + f[j];
-            b = b * z + f[j + 1];
+            a = radd(rmul(a, z), f[j]);
+            b = radd(rmul(b, z), f[j + 1]);
         }
         p1 = a;
         p2 = b;
     } else {
         const T em = expm1(z);
-        p1 = em / z;
-        p2 = (em - z) / (z * z);
+        if constexpr (dfl) {
+            const T iz = recip(z);
+            p1 = rmul(em, iz);
+            p2 = rmul(rmul(rsub(em, z), iz), iz);
+        } else {
+            p1 = em / z;
+            p2 = (em - z) / (z * z);
+        }
     }
 }
 
