@@ -108,6 +108,7 @@ enum {
     FCH_FL_F64IO = 64,     // explicit real-space io in float64 (else the pass precision)
     FCH_FL_STORE_REAL = 256, // F row pass: also store (u, Lap u) into the real-space slot of src
     FCH_FL_GAMMA0 = 512,     // direct row passes: use u^n itself (gamma = 0, the ETD first stage)
+    FCH_FL_PACK_USTAR = 4,   // solve passes: pack u* of the next fixed step (same dt) instead
     FCH_FL_USTAR_V = 1024    // SAV p/q pass: u* is the caller's field in Vb, not eq. (Richardson)
 };
 

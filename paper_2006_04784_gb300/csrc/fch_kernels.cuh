@@ -454,6 +454,28 @@ template <typename T, typename C> __device__ __forceinline__ C mean_mode(const f
     return cadd(un, cscale(csub(un, um), co.c * recip(co.a)));
 }
 
+// u^n + gam (u^n - u^{n-1}), eq. (Richardson)
+template <typename T, typename C> __device__ __forceinline__ C extrapolated(C un, C um, T gam)
+{
+    return cadd(un, cscale(csub(un, um), gam));
+}
+
+// u^{n+1} = v of a solve into the trial slot; what the pass packs for the inverse columns:
+// nothing (false), v itself (for F(v)), or the next fixed step's u* (of the value as stored,
+// with this step's ratio: the step sizes are the same)
+template <typename T, typename C>
+__device__ __forceinline__ bool store_solution(const fch_kparams &kp, const fch_coef<T> &co, const ColBufs<C> &bf,
+                                               long idx, C &v)
+{
+    const C s = lnorm(v);
+    bf.Unew[idx] = s;
+    if (kp.flags & FCH_FL_PACK_USTAR) {
+        v = extrapolated(s, ldg(bf.Un + idx), co.gam);
+        return true;
+    }
+    return kp.flags & FCH_FL_PACK_F;
+}
+
 template <typename T, int MODE>
 __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_consts<T> &K,
                                           const fch_coef<T> &co, const ColBufs<typename CT<T>::t> &bf,
@@ -484,7 +506,7 @@ __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_const
     if (MODE == CM_START) {
         if (kp.src == 4) { // u* = u^n + gam (u^n - u^{n-1}), eq. (Richardson); gam = 0 at the start
             const C un = ldg(bf.Un + idx);
-            v = co.gam != (T)0 ? cadd(un, cscale(csub(un, ldg(bf.Um + idx)), co.gam)) : un;
+            v = co.gam != (T)0 ? extrapolated(un, ldg(bf.Um + idx), co.gam) : un;
             if (kp.flags & 128) ((C *)kp.Vb)[idx] = v; // PSD: v_0 = u*, eq. (recurrence)
         } else {
             v = bf.src[idx];
@@ -501,8 +523,7 @@ __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_const
                 bsub(lscale(ldg(bf.Un + idx), -co.b), badd(lscale(ldg(bf.Um + idx), co.c), lscale(Nh, k2)));
             v = lscale(rhs, recip(radd(co.a, rmul(k2, sk))));
         }
-        bf.Unew[idx] = lnorm(v);
-        pack = kp.flags & FCH_FL_PACK_F;
+        pack = store_solution(kp, co, bf, idx, v);
     } else if (MODE == CM_F_FINISH) {
         // mu^ = eps^4 |k|^4 u^ + eps^2 |k|^2 W'^ + (rest)^ ; F^ = -|k|^2 mu^ (eq. sFCH)
         const C u = ldg(bf.src + idx);
@@ -551,8 +572,7 @@ __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_const
         return;
     } else if (MODE == CM_SAV_COMBINE) {
         v = badd(((const C *)kp.Pb)[idx], lscale(((const C *)kp.Qb)[idx], co.r_new));
-        bf.Unew[idx] = lnorm(v);
-        pack = kp.flags & FCH_FL_PACK_F;
+        pack = store_solution(kp, co, bf, idx, v);
     } else if (MODE == CM_PSD_ITER) {
         // R = mu(v) + (a v + b u^n + c u^{n-1}) / |k|^2,  d = -R / (s + a/|k|^2)  (k != 0),
         // v <- v + lambda d, eqs. (residual), (recurrence)
@@ -592,8 +612,10 @@ __device__ __forceinline__ void spec_elem(const fch_kparams &kp, const fch_const
             const C ut = bf.Unew[idx];
             const C N1 = badd(lscale(Nim, -k2), lscale(ut, lin));
             v = badd(ut, lscale(bsub(N1, Nb[idx]), rmul(co.k1, p2)));
-            bf.Unew[idx] = lnorm(v);
-            pack = kp.flags & FCH_FL_PACK_F;
+            const C s = lnorm(v);
+            bf.Unew[idx] = s;
+            if (kp.flags & FCH_FL_PACK_USTAR) v = s; // the next step starts at u^{n+1} itself
+            pack = kp.flags & (FCH_FL_PACK_F | FCH_FL_PACK_USTAR);
         }
     }
     if (pack) {
@@ -677,7 +699,7 @@ template <typename T, int MODE, int PPT = 8> __global__ void __launch_bounds__(1
     const int c = threadIdx.x % nc, t = threadIdx.x / nc;
     const int p0 = blockIdx.x * P;
     const fch_consts<T> &K = consts<T>(kp);
-    const bool inv = TR::INV_ALWAYS || (TR::INV_OPT && (kp.flags & FCH_FL_PACK_F));
+    const bool inv = TR::INV_ALWAYS || (TR::INV_OPT && (kp.flags & (FCH_FL_PACK_F | FCH_FL_PACK_USTAR)));
     const bool has_red = MODE == CM_SAV_PQ || MODE == CM_PSD_ITER ||
                          (MODE == CM_F_FINISH && (kp.flags & FCH_FL_AM3));
     C *Z = pair_Z<C>(kp, N);

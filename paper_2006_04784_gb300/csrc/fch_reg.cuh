@@ -303,7 +303,7 @@ __device__ __forceinline__ void col_body_r(const fch_kparams &kp)
     __shared__ double red_scratch[FCH_NRED * 32];
     const C *tw = (const C *)(PPT == 8 ? kp.tw : kp.tw4);
     const fch_consts<T> &K = consts<T>(kp);
-    const bool inv = TR::INV_ALWAYS || (TR::INV_OPT && (kp.flags & FCH_FL_PACK_F));
+    const bool inv = TR::INV_ALWAYS || (TR::INV_OPT && (kp.flags & (FCH_FL_PACK_F | FCH_FL_PACK_USTAR)));
     const bool has_red = MODE == CM_SAV_PQ || MODE == CM_PSD_ITER ||
                          (MODE == CM_F_FINISH && (kp.flags & FCH_FL_AM3));
     // this thread's column: slot cc of the block's columns (slot c of pair p), point t + TPS m

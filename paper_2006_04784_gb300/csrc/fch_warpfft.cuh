@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(128) col_pass_w(const fch_kparams kp)
     const int p0 = blockIdx.x * P;
     const fch_consts<float> &K = kp.cf;
     const C *tw2 = (const C *)kp.tw2;
-    const bool inv = TR::INV_ALWAYS || (TR::INV_OPT && (kp.flags & FCH_FL_PACK_F));
+    const bool inv = TR::INV_ALWAYS || (TR::INV_OPT && (kp.flags & (FCH_FL_PACK_F | FCH_FL_PACK_USTAR)));
     const bool has_red = MODE == CM_SAV_PQ || MODE == CM_PSD_ITER ||
                          (MODE == CM_F_FINISH && (kp.flags & FCH_FL_AM3));
     C *Z = pair_Z<C>(kp, N);

@@ -87,3 +87,21 @@ def test_mean_mode_is_kept_to_the_last_bit(prec, scheme):
         for dt in (1e-4, 3e-4, 1e-4, 7e-5):
             ctx.step(scheme, dt)
         assert ctx.mass() == m0
+
+
+@pytest.mark.parametrize("n", [16, 128, 1024])
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("scheme", ["imex", "sav", "etd"])
+def test_fused_fixed_steps_equal_single_steps(n, prec, scheme):
+    # from the second step of a run on, the solve packs the next step's u*: the same bits as
+    # steps of their own, whatever the length of the run and what went before it
+    u0 = I.circle_bilayer(n, noise=1e-2)
+    p = fch.params_default(0.0, prec=prec)
+    with fch.Context(n, p) as a, fch.Context(n, p) as b:
+        a.set_state(u0)
+        b.set_state(u0)
+        for m, dt in ((1, 2e-6), (2, 1e-6), (3, 1e-6), (4, 3e-6), (6, 3e-6)):
+            for _ in range(m):
+                a.step(scheme, dt)
+            b.run_fixed(scheme, dt, m)
+            assert np.array_equal(a.get_state(), b.get_state()), (m, dt)
