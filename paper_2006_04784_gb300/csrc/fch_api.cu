@@ -912,10 +912,15 @@ extern "C" fch_status fch_get_state_device(fch_ctx *ctx, void *u_dev, int dtype)
 // the converged iterate
 static const int kPsdChunk = 4;
 
-static fch_status psd_chunk_eager(fch_ctx *ctx)
+// pdl: programmatic launch behind the chunk's first pass (in the body of a while node, whose
+// first node it must not reach across; 256^2 FP32X2, 24 PSD trials 2725 -> 2619 us). Chunks
+// of three, four and six iterations time alike, of one or two the loop's launches cost
+// more (2866, 2666), of eight the skipped passes do (2662).
+static fch_status psd_chunk_eager(fch_ctx *ctx, int pdl = -1)
 {
     for (int i = 0; i < kPsdChunk; i++) {
         TRY(row(ctx, RM_F, FCH_FL_PSDSKIP));
+        if (i == 0 && pdl > 0) ctx->kp.pdl = pdl;
         TRY(colt(ctx, CM_PSD_ITER, 0, FCH_FL_PSDSKIP, OP_PSD_CHECK));
     }
     return FCH_OK;
@@ -1019,7 +1024,8 @@ static fch_status psd_loop_captured(fch_ctx *ctx)
     const int pdl = ctx->kp.pdl;
     ctx->stream = ctx->bstream;
     ctx->kp.pdl = 0;
-    fch_status s = psd_chunk_eager(ctx);
+    fch_status s = psd_chunk_eager(ctx, pdl);
+    ctx->kp.pdl = 0;
     if (s == FCH_OK) {
         fch_psd_loop_kernel<<<1, 1, 0, ctx->stream>>>(h, ctx->dctrl, count, 0, limit);
         if (cudaGetLastError() != cudaSuccess) s = FCH_ECUDA;
