@@ -2333,6 +2333,8 @@ extern "C" fch_status fch_fft_plan_destroy(fch_fft_plan *pl)
     return FCH_OK;
 }
 
+const void *fch_fft_plan_twiddles(const fch_fft_plan *pl) { return pl->tw; }
+
 extern "C" fch_status fch_fft_plan_status(fch_fft_plan *pl)
 {
     if (!pl) return FCH_EINVAL;

@@ -30,6 +30,7 @@
 #include <string.h>
 
 #include "../../include/fch.h"
+#include "fch_fnomodes.cuh"
 #include "fch_internal.h"
 #include "fch_tc.cuh"
 #include "fch_tmap.h"
@@ -37,6 +38,7 @@
 namespace {
 
 constexpr int kMaxW2 = 128;  // hidden channels of the projection
+constexpr int kMaxQ1 = 2048; // its first layer's weights, W2 W
 
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float x)
@@ -138,30 +140,9 @@ __global__ void fno_to_bf16(const float *__restrict__ w, __nv_bfloat16 *__restri
     if (t < cnt) out[t] = __float2bfloat16_rn(w[t]);
 }
 
-// h0[b][c][p] = sum_i P[c][i] a[b][i][p] + bP[c] (the weights staged in shared memory)
-template <typename WT>
-__global__ void fno_lift(const float *__restrict__ a, const WT *__restrict__ P, const WT *__restrict__ bP,
-                         float *__restrict__ h, int B, int n2, int W, int cin)
-{
-    __shared__ float ps[32 * 4], bs[32];
-    for (int i = threadIdx.x; i < W * cin; i += blockDim.x) ps[i] = wld(P, i);
-    for (int i = threadIdx.x; i < W; i += blockDim.x) bs[i] = wld(bP, i);
-    __syncthreads();
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)B * n2) return;
-    const int b = (int)(t / n2), p = (int)(t - (long)b * n2);
-    float in[4];
-    for (int i = 0; i < cin; i++) in[i] = a[((long)b * cin + i) * n2 + p];
-    for (int c = 0; c < W; c++) {
-        float acc = bs[c];
-        for (int i = 0; i < cin; i++) acc += ps[c * cin + i] * in[i];
-        h[((long)b * W + c) * n2 + p] = acc;
-    }
-}
-
-// the same with the channel counts fixed at compile time (the tensor-core forward
-// pass): loops unrolled, each output channel one multiply-add chain and one store at a
-// running pointer
+// h0[b][c][p] = sum_i P[c][i] a[b][i][p] + bP[c]: the channel counts fixed at compile time,
+// loops unrolled, each output channel one multiply-add chain and one store at a running
+// pointer
 template <typename WT, int W, int CIN>
 __global__ void __launch_bounds__(256) fno_lift_t(const float *__restrict__ a, const WT *__restrict__ P,
                                                   const WT *__restrict__ bP, float *__restrict__ h, long pts, int n2)
@@ -188,54 +169,95 @@ __global__ void __launch_bounds__(256) fno_lift_t(const float *__restrict__ a, c
 }
 
 // z[b][c][p] = sum_j Wl[c][j] h[b][j][p] + bl[c] + s[b][c][p];  out = act(z)
-// (W, the channel count, is a compile-time constant so the per-point channel
-// vectors stay in registers)
+// (W, the channel count, is a compile-time constant so the per-point channel vectors stay
+// in registers). A thread takes two neighbouring points: each 16-byte read of four weights
+// from shared memory feeds eight multiply-adds, where one point and scalar reads made the
+// kernel wait on shared memory (one read a multiply-add; 128^2, batch 8, W = 32: 26 us for
+// 67 MB).
 template <int W, typename WT = float>
-__global__ void fno_pointwise(const float *__restrict__ h, const float *__restrict__ s,
-                              const WT *__restrict__ Wl, const WT *__restrict__ bl, float *__restrict__ z,
-                              float *__restrict__ out, int B, int n2, int act)
+__global__ void __launch_bounds__(128) fno_pointwise(const float *__restrict__ h, const float *__restrict__ s,
+                                                     const WT *__restrict__ Wl, const WT *__restrict__ bl,
+                                                     float *__restrict__ z, float *__restrict__ out, int B, int n2,
+                                                     int act)
 {
-    __shared__ float ws[W * W];
+    __shared__ __align__(16) float ws[W * W];
     __shared__ float bs[W];
     for (int i = threadIdx.x; i < W * W; i += blockDim.x) ws[i] = wld(Wl, i);
     for (int i = threadIdx.x; i < W; i += blockDim.x) bs[i] = wld(bl, i);
     __syncthreads();
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long t = 2 * ((long)blockIdx.x * blockDim.x + threadIdx.x);
     if (t >= (long)B * n2) return;
     const int b = (int)(t / n2), p = (int)(t - (long)b * n2);
-    float in[W];
+    const long o0 = (long)b * W * n2 + p;
+    float2 in[W];
 #pragma unroll
-    for (int j = 0; j < W; j++) in[j] = h[((long)b * W + j) * n2 + p];
+    for (int j = 0; j < W; j++) in[j] = *(const float2 *)(h + o0 + (long)j * n2);
+#pragma unroll 2
     for (int c = 0; c < W; c++) {
-        const long o = ((long)b * W + c) * n2 + p;
-        float acc = bs[c] + s[o];
+        const long o = o0 + (long)c * n2;
+        const float2 sv = *(const float2 *)(s + o);
+        float2 acc = make_float2(bs[c] + sv.x, bs[c] + sv.y);
 #pragma unroll
-        for (int j = 0; j < W; j++) acc += ws[c * W + j] * in[j];
-        z[o] = acc;
-        out[o] = act ? gelu(acc) : acc;
+        for (int j = 0; j < W; j += 4) {
+            const float4 w = *(const float4 *)(ws + c * W + j);
+            acc.x = fmaf(w.x, in[j].x, acc.x);
+            acc.y = fmaf(w.x, in[j].y, acc.y);
+            acc.x = fmaf(w.y, in[j + 1].x, acc.x);
+            acc.y = fmaf(w.y, in[j + 1].y, acc.y);
+            acc.x = fmaf(w.z, in[j + 2].x, acc.x);
+            acc.y = fmaf(w.z, in[j + 2].y, acc.y);
+            acc.x = fmaf(w.w, in[j + 3].x, acc.x);
+            acc.y = fmaf(w.w, in[j + 3].y, acc.y);
+        }
+        *(float2 *)(z + o) = acc;
+        *(float2 *)(out + o) = act ? make_float2(gelu(acc.x), gelu(acc.y)) : acc;
     }
 }
 
-// y[b][p] = bQ2 + sum_d Q2[d] GELU(bQ1[d] + sum_c Q1[d][c] h[b][c][p])
+// y[b][p] = bQ2 + sum_d Q2[d] GELU(bQ1[d] + sum_c Q1[d][c] h[b][c][p]); two points a thread
+// and the weights in shared memory, as fno_pointwise (read from global memory one weight a
+// multiply-add it took 65 us for 131072 points, W = 32, W2 = 64)
 template <int W, typename WT = float>
-__global__ void fno_project(const float *__restrict__ h, const WT *__restrict__ Q1, const WT *__restrict__ bQ1,
-                            const WT *__restrict__ Q2, const WT *__restrict__ bQ2, float *__restrict__ y,
-                            int B, int n2, int W2)
+__global__ void __launch_bounds__(128) fno_project(const float *__restrict__ h, const WT *__restrict__ Q1,
+                                                   const WT *__restrict__ bQ1, const WT *__restrict__ Q2,
+                                                   const WT *__restrict__ bQ2, float *__restrict__ y, int B, int n2,
+                                                   int W2)
 {
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ __align__(16) float ws[kMaxQ1];
+    __shared__ float bs[kMaxW2], qs[kMaxW2];
+    for (int i = threadIdx.x; i < W2 * W; i += blockDim.x) ws[i] = wld(Q1, i);
+    for (int i = threadIdx.x; i < W2; i += blockDim.x) {
+        bs[i] = wld(bQ1, i);
+        qs[i] = wld(Q2, i);
+    }
+    __syncthreads();
+    const long t = 2 * ((long)blockIdx.x * blockDim.x + threadIdx.x);
     if (t >= (long)B * n2) return;
     const int b = (int)(t / n2), p = (int)(t - (long)b * n2);
-    float in[W];
+    float2 in[W];
 #pragma unroll
-    for (int c = 0; c < W; c++) in[c] = h[((long)b * W + c) * n2 + p];
-    float acc = wld(bQ2, 0);
+    for (int c = 0; c < W; c++) in[c] = *(const float2 *)(h + ((long)b * W + c) * n2 + p);
+    const float b2 = wld(bQ2, 0);
+    float2 acc = make_float2(b2, b2);
     for (int d = 0; d < W2; d++) {
-        float zq = wld(bQ1, d);
+        float2 zq = make_float2(bs[d], bs[d]);
 #pragma unroll
-        for (int c = 0; c < W; c++) zq += wld(Q1, d * W + c) * in[c];
-        acc += wld(Q2, d) * gelu(zq);
+        for (int c = 0; c < W; c += 4) {
+            const float4 w = *(const float4 *)(ws + d * W + c);
+            zq.x = fmaf(w.x, in[c].x, zq.x);
+            zq.y = fmaf(w.x, in[c].y, zq.y);
+            zq.x = fmaf(w.y, in[c + 1].x, zq.x);
+            zq.y = fmaf(w.y, in[c + 1].y, zq.y);
+            zq.x = fmaf(w.z, in[c + 2].x, zq.x);
+            zq.y = fmaf(w.z, in[c + 2].y, zq.y);
+            zq.x = fmaf(w.w, in[c + 3].x, zq.x);
+            zq.y = fmaf(w.w, in[c + 3].y, zq.y);
+        }
+        acc.x = fmaf(qs[d], gelu(zq.x), acc.x);
+        acc.y = fmaf(qs[d], gelu(zq.y), acc.y);
     }
-    y[(long)b * n2 + p] = acc;
+    y[t] = acc.x;
+    y[t + 1] = acc.y;
 }
 
 // Backward of the projection and the loss mean((y - target)^2): per point dy, the
@@ -248,6 +270,14 @@ __global__ void fno_project_bwd(const float *__restrict__ h, const float *__rest
                                 float *__restrict__ q, float *__restrict__ dzq, float *__restrict__ dh,
                                 float *__restrict__ sq, int B, int n2, int W2, float scale)
 {
+    __shared__ __align__(16) float ws[kMaxQ1];
+    __shared__ float bs[kMaxW2], qs[kMaxW2];
+    for (int i = threadIdx.x; i < W2 * W; i += blockDim.x) ws[i] = Q1[i];
+    for (int i = threadIdx.x; i < W2; i += blockDim.x) {
+        bs[i] = bQ1[i];
+        qs[i] = Q2[i];
+    }
+    __syncthreads();
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long)B * n2) return;
     const int b = (int)(t / n2), p = (int)(t - (long)b * n2);
@@ -262,15 +292,27 @@ __global__ void fno_project_bwd(const float *__restrict__ h, const float *__rest
     dy[t] = d;
     sq[t] = r * r;
     for (int k = 0; k < W2; k++) {
-        float zq = bQ1[k];
+        float4 w[W / 4];
+        float zq = bs[k];
 #pragma unroll
-        for (int c = 0; c < W; c++) zq += Q1[k * W + c] * in[c];
+        for (int c = 0; c < W; c += 4) {
+            w[c / 4] = *(const float4 *)(ws + k * W + c);
+            zq = fmaf(w[c / 4].x, in[c], zq);
+            zq = fmaf(w[c / 4].y, in[c + 1], zq);
+            zq = fmaf(w[c / 4].z, in[c + 2], zq);
+            zq = fmaf(w[c / 4].w, in[c + 3], zq);
+        }
         const long o = ((long)b * W2 + k) * n2 + p;
         q[o] = gelu(zq);
-        const float dz = d * Q2[k] * gelu_grad(zq);
+        const float dz = d * qs[k] * gelu_grad(zq);
         dzq[o] = dz;
 #pragma unroll
-        for (int c = 0; c < W; c++) g[c] += Q1[k * W + c] * dz;
+        for (int c = 0; c < W; c += 4) {
+            g[c] = fmaf(w[c / 4].x, dz, g[c]);
+            g[c + 1] = fmaf(w[c / 4].y, dz, g[c + 1]);
+            g[c + 2] = fmaf(w[c / 4].z, dz, g[c + 2]);
+            g[c + 3] = fmaf(w[c / 4].w, dz, g[c + 3]);
+        }
     }
 #pragma unroll
     for (int c = 0; c < W; c++) dh[((long)b * W + c) * n2 + p] = g[c];
@@ -282,7 +324,7 @@ __global__ void fno_pointwise_bwd(const float *__restrict__ dout, const float *_
                                   const float *__restrict__ Wl, float *__restrict__ dz, float *__restrict__ dh,
                                   int B, int n2, int act)
 {
-    __shared__ float ws[W * W];
+    __shared__ __align__(16) float ws[W * W];
     for (int i = threadIdx.x; i < W * W; i += blockDim.x) ws[i] = Wl[i];
     __syncthreads();
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -931,6 +973,68 @@ __global__ void fno_dX(const float2 *__restrict__ dY, const float2 *__restrict__
     }
 }
 
+// The products over the channels at one retained mode (block m) on mode-major spectra
+// [m][b W + c]: Y[b][o] = sum_i R[o][i] X[b][i]. The weights pass through shared memory, rows
+// padded by one (lanes read consecutive o).
+template <typename WT>
+__global__ void __launch_bounds__(256) fno_mode_mix(const float2 *__restrict__ X, const WT *__restrict__ R,
+                                                    float2 *__restrict__ Y, int BW, int W)
+{
+    extern __shared__ __align__(16) float2 mm_smem[];
+    float2 *r = mm_smem, *x = mm_smem + W * (W + 1);
+    const long m = blockIdx.x;
+    for (int e = threadIdx.x; e < W * W; e += 256) r[e / W * (W + 1) + e % W] = wld2(R, m * W * W + e);
+    for (int e = threadIdx.x; e < BW; e += 256) x[e] = X[m * BW + e];
+    __syncthreads();
+    for (int e = threadIdx.x; e < BW; e += 256) {
+        const float2 *ro = r + e % W * (W + 1), *xb = x + e / W * W;
+        float re = 0.f, im = 0.f;
+        for (int i = 0; i < W; i++) {
+            const float2 w = ro[i], v = xb[i];
+            re += w.x * v.x - w.y * v.y;
+            im += w.x * v.y + w.y * v.x;
+        }
+        Y[m * BW + e] = make_float2(re, im);
+    }
+}
+
+// Backward at one mode: dR[o][i] = sum_b dY[b][o] conj X[b][i] and
+// Z[b][i] = sum_o conj(R[o][i]) dY[b][o].
+__global__ void __launch_bounds__(256) fno_mode_bwd(const float2 *__restrict__ dY, const float2 *__restrict__ X,
+                                                    const float2 *__restrict__ R, float2 *__restrict__ dR,
+                                                    float2 *__restrict__ Z, int BW, int W)
+{
+    extern __shared__ __align__(16) float2 mm_smem[];
+    float2 *r = mm_smem, *x = r + W * W, *d = x + BW;
+    const long m = blockIdx.x;
+    for (int e = threadIdx.x; e < W * W; e += 256) r[e] = R[m * W * W + e];
+    for (int e = threadIdx.x; e < BW; e += 256) {
+        x[e] = X[m * BW + e];
+        d[e] = dY[m * BW + e];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < W * W; e += 256) {
+        const int o = e / W, i = e % W;
+        float re = 0.f, im = 0.f;
+        for (int b = 0; b < BW; b += W) {
+            const float2 u = d[b + o], v = x[b + i];
+            re += u.x * v.x + u.y * v.y;
+            im += u.y * v.x - u.x * v.y;
+        }
+        dR[m * W * W + e] = make_float2(re, im);
+    }
+    for (int e = threadIdx.x; e < BW; e += 256) {
+        const int i = e % W, b = e - i;
+        float re = 0.f, im = 0.f;
+        for (int o = 0; o < W; o++) {
+            const float2 w = r[o * W + i], u = d[b + o];
+            re += w.x * u.x + w.y * u.y;
+            im += w.x * u.y - w.y * u.x;
+        }
+        Z[m * BW + e] = make_float2(re, im);
+    }
+}
+
 __global__ void fno_add(float *__restrict__ a, const float *__restrict__ b, long cnt)
 {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -940,20 +1044,21 @@ __global__ void fno_add(float *__restrict__ a, const float *__restrict__ b, long
 // Weight-gradient partials of a dense layer: G[a][c] = sum over points of A(a, pt) Bm(c, pt)
 // and the bias row sums of A, with A(a, (b, p)) = A[(b na + a) n2 + p] (Bm alike). A block
 // takes the 32 x 32 outputs (32 blockIdx.y, 32 blockIdx.z) over its share of the points,
-// staged 32 at a time in shared memory (rows padded to 36 floats: the 16-byte reads of eight
+// staged 64 at a time in shared memory (rows padded to 68 floats: the 16-byte reads of eight
 // lanes fall on distinct banks); a thread owns 4 x 4 outputs of one quarter of the points,
 // 64 fused multiply-adds per eight 16-byte reads, and the quarters are summed at the end.
 // Block k writes part[k][off + a nb + c] and part[k][off + na nb + a].
 // The kernel before gave a thread 1-8 outputs with one multiply-add per two scalar reads, and
 // the sums of 1024 partials ran in one to eight blocks: at 128^2, batch 8, 32 channels, 1.17 ms
 // of partials and 0.85 ms of sums a training step.
-constexpr int kWgPad = 36;
+constexpr int kWgPts = 64, kWgPad = kWgPts + 4;
 __global__ void __launch_bounds__(256) fno_wgrad_part(const float *__restrict__ A, int na,
                                                       const float *__restrict__ Bm, int nb, int n2, long npts,
                                                       int chunk, float *__restrict__ part, long stride, long off)
 {
-    __shared__ __align__(16) float sm[2 * 32 * kWgPad + 16];
-    __shared__ float acc_sm[4][32 * 33];
+    __shared__ __align__(16) float sm[2 * 32 * kWgPad]; // then the quarters' sums [4][32 * 33]
+    static_assert(2 * 32 * kWgPad >= 4 * 32 * 33, "the sums fit the stage");
+    float(*acc_sm)[32 * 33] = (float(*)[32 * 33])sm;
     float *sa = sm, *sb = sm + 32 * kWgPad;
     const int tid = threadIdx.x, kg = tid >> 6, ta = (tid >> 3) & 7, tc = tid & 7;
     const int a0 = blockIdx.y * 32, c0 = blockIdx.z * 32;
@@ -967,25 +1072,33 @@ __global__ void __launch_bounds__(256) fno_wgrad_part(const float *__restrict__ 
         for (int j = 0; j < 4; j++) acc[i][j] = 0.f;
     }
     const long p0 = (long)blockIdx.x * chunk, p1 = min(p0 + chunk, npts);
-    // chunks of 32 points lie within one sample (n2 is a multiple of 32)
+    // a stage's points lie within one sample (n2 is a multiple of 256)
     const bool vec = !((uintptr_t)Bm & 15); // the network's input is the caller's array
-    auto fetch = [&](long q, float4 &fa, float4 &fb) {
+    auto fetch = [&](long q, float4 *fa, float4 *fb) {
         const long b = q / n2, p = q - b * n2 + lk;
-        fa = la ? *(const float4 *)(A + (b * na + a0 + lr) * n2 + p) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float *B = Bm + (b * nb + c0 + lr) * n2 + p;
-        fb = !lb ? make_float4(0.f, 0.f, 0.f, 0.f) : vec ? *(const float4 *)B : make_float4(B[0], B[1], B[2], B[3]);
-    };
-    float4 fa, fb;
-    if (p0 < p1) fetch(p0, fa, fb);
-    for (long q = p0; q < p1; q += 32) {
-        __syncthreads();
-        *(float4 *)(sa + lr * kWgPad + lk) = fa;
-        *(float4 *)(sb + lr * kWgPad + lk) = fb;
-        __syncthreads();
-        if (q + 32 < p1) fetch(q + 32, fa, fb);
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float *pa = A + (b * na + a0 + lr) * n2 + p, *pb = Bm + (b * nb + c0 + lr) * n2 + p;
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            const int k = kg * 8 + h * 4;
+            const float *w = pb + 32 * h;
+            fa[h] = la ? *(const float4 *)(pa + 32 * h) : zero;
+            fb[h] = !lb ? zero : vec ? *(const float4 *)w : make_float4(w[0], w[1], w[2], w[3]);
+        }
+    };
+    float4 fa[2], fb[2];
+    if (p0 < p1) fetch(p0, fa, fb);
+    for (long q = p0; q < p1; q += kWgPts) {
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            *(float4 *)(sa + lr * kWgPad + lk + 32 * h) = fa[h];
+            *(float4 *)(sb + lr * kWgPad + lk + 32 * h) = fb[h];
+        }
+        __syncthreads();
+        if (q + kWgPts < p1) fetch(q + kWgPts, fa, fb);
+#pragma unroll
+        for (int h = 0; h < kWgPts / 16; h++) {
+            const int k = kg * (kWgPts / 4) + h * 4;
             float4 va[4], vb[4];
 #pragma unroll
             for (int i = 0; i < 4; i++) {
@@ -1006,6 +1119,7 @@ __global__ void __launch_bounds__(256) fno_wgrad_part(const float *__restrict__ 
             }
         }
     }
+    __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; i++) {
 #pragma unroll
@@ -1100,10 +1214,11 @@ struct fch_fno {
     fch_fft_plan *plan;
     float *h;     // (L + 1) x [B][W][n^2]
     float *z;     // L x [B][W][n^2]
-    float2 *X;    // L x [B W][(n/2+1) n]
-    float2 *Ysp;  // [B W][(n/2+1) n], zero outside the retained modes
-    float2 *Fd;   // [B W][(n/2+1) n]
-    float2 *dY;   // [B][W][K]
+    // spectra: up to 256^2 the retained modes only, mode-major (fch_fnomodes.cuh): X L x
+    // [K][B W], Ysp and dY [K][B W]; on larger grids (or M > 32) X L x [B W][(n/2+1) n], Ysp
+    // and Fd [B W][(n/2+1) n] (Ysp zero outside the retained modes), dY [B][W][K]
+    bool modes;
+    float2 *X, *Ysp, *Fd, *dY;
     float *s;     // [B][W][n^2]
     float *dh, *dz, *tmp; // [B][W][n^2]
     float *q, *dzq;       // [B][W2][n^2]
@@ -1148,16 +1263,67 @@ size_t offset_of(const fch_fno *f, int what, int l)
 }
 
 // blocks the points of a weight gradient are split over (two an SM of the 152 at the most,
-// whole runs of 32 points), and the partial sums of all layers in one block's row
+// whole stages), and the partial sums of all layers in one block's row
 int wgrad_blocks(long npts, int &chunk)
 {
-    const long runs = npts / 32, per = (runs + 303) / 304;
-    chunk = (int)(per * 32);
+    const long runs = npts / kWgPts, per = (runs + 303) / 304;
+    chunk = (int)(per * kWgPts);
     return (int)((runs + per - 1) / per);
 }
 size_t wgrad_stride(const fch_fno *f)
 {
     return (size_t)f->W * f->cin + f->W + (size_t)f->L * (f->W * f->W + f->W) + (size_t)f->W2 * f->W + 2 * f->W2 + 1;
+}
+
+// whether the spectral branch runs on the retained modes inside a block: grids whose rows and
+// kept columns fit an SM's shared memory twice, and channel vectors of a mode that fit the
+// products' 48 KB
+bool modes_fit(const fch_fno *f, int B, int n)
+{
+    return n >= 32 && n <= 256 && f->M <= 32 && (size_t)B * f->W <= 2048;
+}
+
+template <int LOGN>
+cudaError_t field_modes_t(fch_fno *f, const float *h, float2 *out, float s0, float s1, int herm)
+{
+    typedef fch::FnoModes<LOGN> G;
+    cudaError_t e = cudaFuncSetAttribute(fch::fno_field_modes<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         G::smem(32));
+    if (e != cudaSuccess) return e;
+    fch::fno_field_modes<LOGN><<<f->B * f->W, G::threads, G::smem(f->M), f->stream>>>(
+        h, out, (const float2 *)fch_fft_plan_twiddles(f->plan), f->M, s0, s1, herm);
+    return cudaGetLastError();
+}
+cudaError_t field_modes(fch_fno *f, const float *h, float2 *out, float s0, float s1, int herm)
+{
+    switch (f->n) {
+    case 32: return field_modes_t<5>(f, h, out, s0, s1, herm);
+    case 64: return field_modes_t<6>(f, h, out, s0, s1, herm);
+    case 128: return field_modes_t<7>(f, h, out, s0, s1, herm);
+    case 256: return field_modes_t<8>(f, h, out, s0, s1, herm);
+    }
+    return cudaErrorInvalidValue;
+}
+template <int LOGN>
+cudaError_t modes_field_t(fch_fno *f, const float2 *Y, const float *base, float *out, float s0, float s1)
+{
+    typedef fch::FnoModes<LOGN> G;
+    cudaError_t e = cudaFuncSetAttribute(fch::fno_modes_field<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         G::smem(32));
+    if (e != cudaSuccess) return e;
+    fch::fno_modes_field<LOGN><<<f->B * f->W, G::threads, G::smem(f->M), f->stream>>>(
+        Y, base, out, (const float2 *)fch_fft_plan_twiddles(f->plan), f->M, s0, s1);
+    return cudaGetLastError();
+}
+cudaError_t modes_field(fch_fno *f, const float2 *Y, const float *base, float *out, float s0, float s1)
+{
+    switch (f->n) {
+    case 32: return modes_field_t<5>(f, Y, base, out, s0, s1);
+    case 64: return modes_field_t<6>(f, Y, base, out, s0, s1);
+    case 128: return modes_field_t<7>(f, Y, base, out, s0, s1);
+    case 256: return modes_field_t<8>(f, Y, base, out, s0, s1);
+    }
+    return cudaErrorInvalidValue;
 }
 
 void free_buffers(fch_fno *f)
@@ -1185,9 +1351,11 @@ fch_status ensure_buffers(fch_fno *f, int B, int n)
     };
     al((void **)&f->h, (f->L + 1) * fld * 4);
     al((void **)&f->z, f->L * fld * 4);
-    al((void **)&f->X, (size_t)f->L * B * f->W * S * 8);
-    al((void **)&f->Ysp, (size_t)B * f->W * S * 8);
-    al((void **)&f->Fd, (size_t)B * f->W * S * 8);
+    f->modes = modes_fit(f, B, n);
+    const size_t spec = (size_t)B * f->W * (f->modes ? (size_t)f->K : S) * 8;
+    al((void **)&f->X, f->L * spec);
+    al((void **)&f->Ysp, spec);
+    if (!f->modes) al((void **)&f->Fd, spec);
     al((void **)&f->dY, (size_t)B * f->W * f->K * 8);
     al((void **)&f->s, fld * 4);
     al((void **)&f->dh, fld * 4);
@@ -1201,7 +1369,7 @@ fch_status ensure_buffers(fch_fno *f, int B, int n)
     int chunk;
     al((void **)&f->part, (size_t)wgrad_blocks((long)B * n2, chunk) * wgrad_stride(f) * 4);
     al((void **)&f->lpart, kLossBlocks * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemsetAsync(f->Ysp, 0, (size_t)B * f->W * S * 8, f->stream);
+    if (e == cudaSuccess && !f->modes) e = cudaMemsetAsync(f->Ysp, 0, spec, f->stream);
     if (e != cudaSuccess) {
         snprintf(f->err, sizeof(f->err), "fch_fno: %s", cudaGetErrorString(e));
         free_buffers(f);
@@ -1259,7 +1427,7 @@ cudaStream_t fch_fno_stream_of(const fch_fno *f) { return f->stream; }
 extern "C" fch_status fch_fno_create(int width, int layers, int modes, int proj, void *stream, fch_fno **out)
 {
     if (!out || (width != 8 && width != 16 && width != 32) || layers < 1 || layers > 16 || modes < 1 ||
-        proj < 1 || proj > kMaxW2 || proj * width > 8 * 256) {
+        proj < 1 || proj > kMaxW2 || proj * width > kMaxQ1) {
         fch_set_thread_error("fch_fno_create: invalid argument");
         return FCH_EINVAL;
     }
@@ -1348,6 +1516,13 @@ extern "C" fch_status fch_fno_get_grads(fch_fno *f, float *host, size_t cnt)
     return copy_vec(f, f ? f->grads : nullptr, nullptr, host, cnt);
 }
 
+static fch_status spec_error(fch_fno *f, cudaError_t e)
+{
+    snprintf(f->err, sizeof(f->err), "fch_fno (spectral branch): %s", cudaGetErrorString(e));
+    fch_set_thread_error(f->err);
+    return FCH_ECUDA;
+}
+
 // the forward pass with weights P of type WT (FP32 parameters or their bfloat16 copy)
 template <typename WT>
 static fch_status forward_impl(fch_fno *f, int batch, int n, const float *a, float *y, const WT *P)
@@ -1358,20 +1533,39 @@ static fch_status forward_impl(fch_fno *f, int batch, int n, const float *a, flo
     const long pts = (long)batch * n2;
     const size_t fld = (size_t)batch * W * n2, S = (size_t)(n / 2 + 1) * n;
     cudaStream_t s = f->stream;
-    fno_lift<WT><<<grid(pts, 256), 256, 0, s>>>(a, P + offset_of(f, 0, 0), P + offset_of(f, 1, 0), f->h, batch, n2,
-                                                W, f->cin);
+    {
+        const WT *P0 = P + offset_of(f, 0, 0), *P1 = P + offset_of(f, 1, 0);
+        if (W == 8)
+            fno_lift_t<WT, 8, 2><<<grid(pts, 256), 256, 0, s>>>(a, P0, P1, f->h, pts, n2);
+        else if (W == 16)
+            fno_lift_t<WT, 16, 2><<<grid(pts, 256), 256, 0, s>>>(a, P0, P1, f->h, pts, n2);
+        else
+            fno_lift_t<WT, 32, 2><<<grid(pts, 256), 256, 0, s>>>(a, P0, P1, f->h, pts, n2);
+    }
     for (int l = 0; l < f->L; l++) {
         float *hin = f->h + l * fld, *hout = f->h + (l + 1) * fld;
-        float2 *X = f->X + (size_t)l * batch * W * S;
-        if ((st = fch_fft_r2c(f->plan, hin, X, batch * W)) != FCH_OK) return st;
-        const int items = f->M + (f->M - 1) * (2 * f->M - 1);
-        fno_mix<WT><<<grid((long)batch * W * items, 256), 256, 0, s>>>(X, P + offset_of(f, 4, l), f->Ysp, batch, W,
-                                                                      f->M, n);
-        if ((st = fch_fft_c2r(f->plan, f->Ysp, f->s, batch * W)) != FCH_OK) return st;
-        WDISPATCH_T(W, fno_pointwise, WT, grid(pts, 128), 128, s, hin, f->s, P + offset_of(f, 2, l),
+        const WT *R = P + offset_of(f, 4, l);
+        if (f->modes) {
+            float2 *X = f->X + (size_t)l * batch * W * f->K;
+            const int BW = batch * W, smem = (W * (W + 1) + BW) * 8;
+            cudaError_t e = field_modes(f, hin, X, 1.f, 1.f, 0);
+            if (e == cudaSuccess) {
+                fno_mode_mix<WT><<<f->K, 256, smem, s>>>(X, R, f->Ysp, BW, W);
+                const float inv = 1.0f / ((float)n * (float)n);
+                e = modes_field(f, f->Ysp, nullptr, f->s, inv, inv);
+            }
+            if (e != cudaSuccess) return spec_error(f, e);
+        } else {
+            float2 *X = f->X + (size_t)l * batch * W * S;
+            if ((st = fch_fft_r2c(f->plan, hin, X, batch * W)) != FCH_OK) return st;
+            const int items = f->M + (f->M - 1) * (2 * f->M - 1);
+            fno_mix<WT><<<grid((long)batch * W * items, 256), 256, 0, s>>>(X, R, f->Ysp, batch, W, f->M, n);
+            if ((st = fch_fft_c2r(f->plan, f->Ysp, f->s, batch * W)) != FCH_OK) return st;
+        }
+        WDISPATCH_T(W, fno_pointwise, WT, grid(pts, 256), 128, s, hin, f->s, P + offset_of(f, 2, l),
                     P + offset_of(f, 3, l), f->z + l * fld, hout, batch, n2, l < f->L - 1);
     }
-    WDISPATCH_T(W, fno_project, WT, grid(pts, 128), 128, s, f->h + f->L * fld, P + offset_of(f, 5, 0),
+    WDISPATCH_T(W, fno_project, WT, grid(pts, 256), 128, s, f->h + f->L * fld, P + offset_of(f, 5, 0),
                 P + offset_of(f, 6, 0), P + offset_of(f, 7, 0), P + offset_of(f, 8, 0), y, batch, n2, f->W2);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -1435,13 +1629,10 @@ static fch_status forward_tc(fch_fno *f, int batch, int n, const float *a, float
     {
         const WT *P0 = P + offset_of(f, 0, 0), *P1 = P + offset_of(f, 1, 0);
         const unsigned gl = grid(pts, 256);
-        switch (f->cin * 64 + W) {
-        case 1 * 64 + 16: fno_lift_t<WT, 16, 1><<<gl, 256, 0, s>>>(a, P0, P1, f->h, pts, n2); break;
-        case 2 * 64 + 16: fno_lift_t<WT, 16, 2><<<gl, 256, 0, s>>>(a, P0, P1, f->h, pts, n2); break;
-        case 1 * 64 + 32: fno_lift_t<WT, 32, 1><<<gl, 256, 0, s>>>(a, P0, P1, f->h, pts, n2); break;
-        case 2 * 64 + 32: fno_lift_t<WT, 32, 2><<<gl, 256, 0, s>>>(a, P0, P1, f->h, pts, n2); break;
-        default: fno_lift<WT><<<gl, 256, 0, s>>>(a, P0, P1, f->h, batch, n2, W, f->cin);
-        }
+        if (W == 16)
+            fno_lift_t<WT, 16, 2><<<gl, 256, 0, s>>>(a, P0, P1, f->h, pts, n2);
+        else
+            fno_lift_t<WT, 32, 2><<<gl, 256, 0, s>>>(a, P0, P1, f->h, pts, n2);
     }
     for (int l = 0; l < f->L; l++) {
         float *hin = f->h + l * fld, *hout = f->h + (l + 1) * fld;
@@ -1561,6 +1752,20 @@ extern "C" fch_status fch_fno_backward(fch_fno *f, const float *target, double *
         e = wgrad(f, f->dz, W, hin, W, lP + l * lW); // W_l, b_l
         if (e != cudaSuccess) break;
         // spectral branch
+        if (f->modes) {
+            const int BW = B * W;
+            const float inv = 1.0f / ((float)n * (float)n);
+            // dY = H(w(kx)/n^2 R2C(dz)); dR and the modes of the input gradient; dh = tmp +
+            // C2R(n^2 v(kx) modes)
+            e = field_modes(f, f->dz, f->dY, inv, 2.f * inv, 1);
+            if (e == cudaSuccess) {
+                fno_mode_bwd<<<f->K, 256, (W * W + 2 * BW) * 8, s>>>(f->dY, f->X + (size_t)l * BW * f->K, R,
+                                                                    (float2 *)(G + offset_of(f, 4, l)), f->Ysp, BW, W);
+                e = modes_field(f, f->Ysp, f->tmp, f->dh, 1.f, 0.5f);
+            }
+            if (e != cudaSuccess) break;
+            continue;
+        }
         if (fch_fft_r2c(f->plan, f->dz, f->Fd, B * W) != FCH_OK) return FCH_ECUDA;
         const int K = f->K;
         fno_dY<<<grid((long)B * W * K, 256), 256, 0, s>>>(f->Fd, f->dY, B, W, f->M, n);

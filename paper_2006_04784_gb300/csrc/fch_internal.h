@@ -201,6 +201,10 @@ void fch_pdl_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, dim3 grid,
 cudaError_t fch_launch_ctrl(int op, const fch_kparams &kp, int nblk_a, int nblk_b, double arg0,
                             cudaStream_t s);
 
+// the radix-8 stage twiddles a plan keeps on the device (n complex elements of its precision)
+struct fch_fft_plan;
+const void *fch_fft_plan_twiddles(const fch_fft_plan *pl);
+
 // sets the per-thread message returned by fch_last_cuda_error(NULL)
 void fch_set_thread_error(const char *msg);
 
