@@ -142,10 +142,12 @@ __global__ void fno_to_bf16(const float *__restrict__ w, __nv_bfloat16 *__restri
 
 // h0[b][c][p] = sum_i P[c][i] a[b][i][p] + bP[c]: the channel counts fixed at compile time,
 // loops unrolled, each output channel one multiply-add chain and one store at a running
-// pointer
-template <typename WT, int W, int CIN>
+// pointer (bf16 output: the tensor-core pass, whose kernels read h rounded to bf16)
+__device__ __forceinline__ void put(float *p, float v) { *p = v; }
+__device__ __forceinline__ void put(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
+template <typename WT, int W, int CIN, typename HT = float>
 __global__ void __launch_bounds__(256) fno_lift_t(const float *__restrict__ a, const WT *__restrict__ P,
-                                                  const WT *__restrict__ bP, float *__restrict__ h, long pts, int n2)
+                                                  const WT *__restrict__ bP, HT *__restrict__ h, long pts, int n2)
 {
     __shared__ float ps[W * CIN], bs[W];
     for (int i = threadIdx.x; i < W * CIN; i += blockDim.x) ps[i] = wld(P, i);
@@ -157,13 +159,13 @@ __global__ void __launch_bounds__(256) fno_lift_t(const float *__restrict__ a, c
     float in[CIN];
 #pragma unroll
     for (int i = 0; i < CIN; i++) in[i] = __ldcs(a + (b * CIN + i) * n2 + p);
-    float *hp = h + b * W * n2 + p;
+    HT *hp = h + b * W * n2 + p;
 #pragma unroll
     for (int c = 0; c < W; c++) {
         float acc = bs[c];
 #pragma unroll
         for (int i = 0; i < CIN; i++) acc = fmaf(ps[c * CIN + i], in[i], acc);
-        *hp = acc;
+        put(hp, acc);
         hp += n2;
     }
 }
@@ -406,8 +408,10 @@ constexpr int kTcRows = 128, kTcLBO = 144, kTcSBO = 8 * kTcLBO, kTcNB = 32;
 constexpr uint64_t kTcBound = 1000000000ull; // ns an mbarrier wait lasts before a kernel gives up
 
 // Bt[j][x] (bf16): cos(2 pi j x / n) for j < 16, -sin(2 pi (j - 16) x / n) for j >= 16;
-// tw[kx][x] (float2): (cos, sin)(2 pi kx x / n), kx < 16
-__global__ void fno_dft_tables(__nv_bfloat16 *__restrict__ Bt, float2 *__restrict__ tw, int n)
+// tw[kx][x] (float2): (cos, sin)(2 pi kx x / n), kx < 16; At[j][x] (may be null): tw rounded
+// to bf16, cos for j < 16, sin for j >= 16
+__global__ void fno_dft_tables(__nv_bfloat16 *__restrict__ Bt, float2 *__restrict__ tw,
+                               __nv_bfloat16 *__restrict__ At, int n)
 {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 16L * n) return;
@@ -417,40 +421,41 @@ __global__ void fno_dft_tables(__nv_bfloat16 *__restrict__ Bt, float2 *__restric
     Bt[(long)kx * n + x] = __double2bfloat16(cs);
     Bt[(long)(16 + kx) * n + x] = __double2bfloat16(-sn);
     tw[(long)kx * n + x] = make_float2((float)cs, (float)sn);
+    if (At) {
+        At[(long)kx * n + x] = __float2bfloat16_rn((float)cs);
+        At[(long)(16 + kx) * n + x] = __float2bfloat16_rn((float)sn);
+    }
 }
 
-// X[r][kx] = (D[r][kx], D[r][16 + kx]) with D = bf16(h) Bt^T over K = n: one CTA of 128
-// threads per 128 rows, K in chunks of 32. A chunk of the FP32 rows arrives as one 2D
-// tile of a tensor map over h (the TMA engine: 128 rows x 32 floats, two chunks ahead,
-// completion counted in bytes on the stage's `full` mbarrier; rows beyond R read as
-// zero); the threads round it to bfloat16 into the core-matrix layout of the stage's A
-// tile (see fch_tc.cuh) and copy the table's chunk; thread 0 issues two K = 16 MMAs
-// into a 128 x 32 FP32 accumulator in tensor memory and commits them to the stage's
-// `mma` mbarrier, which guards the stage's tiles. A wait that runs out of time (1 s) sets
-// *err; the CTA then stops, waits (bounded) for the loads and MMAs it issued, frees its
-// tensor memory and returns.
-constexpr int kDftKc = 32;                                  // K of a chunk (two K = 16 MMAs)
-// 160 bytes between K cores: a half warp's 8-byte stores (two rows x four cores x two
-// halves, one 128-byte wavefront) then fall on 16 distinct bank pairs, and a quarter
-// warp's 16-byte stores of the table (two rows x four cores) on 8 distinct bank quads
-constexpr int kDftLBO = 160;
-constexpr int kDftSBO = (kDftKc / 8) * kDftLBO;             // 8-row groups of four K cores
-constexpr int kRawBytes = kTcRows * kDftKc * 4;             // one tile of FP32 rows (16 KB)
-constexpr int kAtBytes = (kTcRows / 8) * kDftSBO, kBtBytes = (kTcNB / 8) * kDftSBO;
+// X[r][kx] = (D[r][kx], D[r][16 + kx]) with D = h Bt^T over K = n, h the bf16 activations:
+// one CTA of 128 threads per 128 rows, K in chunks of 64 (128 bytes a row). A chunk of the
+// rows and of the table arrive as tiles of two tensor maps with the 128-byte swizzle, the
+// layout the tensor core reads, kDftStages chunks ahead; thread 0 alone starts the copies
+// and issues four K = 16 MMAs a chunk into a 128 x 32 FP32 accumulator in tensor memory; a
+// chunk's `full` mbarrier counts its bytes, its `mma` mbarrier the MMAs that free the
+// stage. Rows past R read as zero. A wait that runs out of time (1 s) sets *err; the CTA
+// then stops, waits (bounded) for the copies and MMAs it issued, frees its tensor memory
+// and returns.
+// Bound by reading h. With h in FP32 every CTA's threads rounded each chunk through shared
+// memory: 134 MB at 1024^2, 32 channels, 38.5 us; the values are the same, rounded once by
+// the kernel that writes them.
+constexpr int kDftKc = 64;                                  // K of a chunk (four K = 16 MMAs)
+constexpr int kDftStages = 4;
+constexpr int kDftABytes = kTcRows * kDftKc * 2, kDftBBytes = kTcNB * kDftKc * 2; // 16 KB, 4 KB
 // the stages, then the mbarriers and the tensor-memory address, and 1 KB of slack to
 // align the tiles to 1024 bytes
-constexpr int kRowdftSmem = 2 * kRawBytes + 2 * kAtBytes + 2 * kBtBytes + 64 + 1024;
+constexpr int kRowdftSmem = kDftStages * (kDftABytes + kDftBBytes) + 128 + 1024;
 
-__global__ void __launch_bounds__(128) fno_rowdft_tc(const __grid_constant__ CUtensorMap tmap,
-                                                     const __nv_bfloat16 *__restrict__ Bt, float2 *__restrict__ X,
-                                                     int R, int n, int *err)
+__global__ void __launch_bounds__(128) fno_rowdft_tc(const __grid_constant__ CUtensorMap amap,
+                                                     const __grid_constant__ CUtensorMap bmap,
+                                                     float2 *__restrict__ X, int R, int n, int *err)
 {
     extern __shared__ unsigned char dsm_raw[];
-    // the TMA destination wants an aligned tile: the window's start rounded up to 1024 B
-    unsigned char *dsm = dsm_raw + ((1024u - (fch::tc::smem_u32(dsm_raw) & 1023u)) & 1023u);
-    unsigned char *raw = dsm, *sA = dsm + 2 * kRawBytes, *sB = sA + 2 * kAtBytes;
-    uint64_t *full = reinterpret_cast<uint64_t *>(sB + 2 * kBtBytes), *mmab = full + 2;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mmab + 2);
+    // swizzled tiles want 1024-byte alignment: the window's start rounded up
+    unsigned char *sA = dsm_raw + ((1024u - (fch::tc::smem_u32(dsm_raw) & 1023u)) & 1023u);
+    unsigned char *sB = sA + kDftStages * kDftABytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(sB + kDftStages * kDftBBytes), *mmab = full + kDftStages;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(mmab + kDftStages);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long row0 = (long)blockIdx.x * kTcRows;
     const int nch = n / kDftKc;
@@ -459,7 +464,7 @@ __global__ void __launch_bounds__(128) fno_rowdft_tc(const __grid_constant__ CUt
         fch::tc::tmem_relinquish();
     }
     if (tid == 0) {
-        for (int i = 0; i < 2; i++) {
+        for (int i = 0; i < kDftStages; i++) {
             fch::tc::mbar_init(&full[i], 1);
             fch::tc::mbar_init(&mmab[i], 1);
         }
@@ -469,66 +474,49 @@ __global__ void __launch_bounds__(128) fno_rowdft_tc(const __grid_constant__ CUt
     __syncthreads();
     fch::tc::fence_after_sync();
     const uint32_t tmem = *tslot;
-    auto fetch = [&](int c) { // thread 0
-        fch::tc::mbar_expect_tx(&full[c & 1], kRawBytes);
-        fch::tc::tma_load_2d(raw + (c & 1) * kRawBytes, &tmap, c * kDftKc, (int)row0, &full[c & 1]);
-    };
-    if (tid == 0)
-        for (int c = 0; c < 2 && c < nch; c++) fetch(c);
-    constexpr uint32_t idesc = fch::tc::idesc_bf16_f32(kTcRows, kTcNB);
     bool ok = true;
-    int fetched = nch < 2 ? nch : 2, issued = 0;
-    for (int c = 0; c < nch; c++) {
-        const int st = c & 1;
-        ok = fch::tc::mbar_wait(&full[st], (uint32_t)((c >> 1) & 1), kTcBound);
-        if (ok && c >= 2) ok = fch::tc::mbar_wait(&mmab[st], (uint32_t)(((c >> 1) - 1) & 1), kTcBound);
-        if (!__syncthreads_and(ok)) break;
-        // raw -> A: 16 bytes (4 floats) a thread and step, a warp reading four whole rows
-        const unsigned char *rs = raw + st * kRawBytes;
-        unsigned char *a = sA + st * kAtBytes;
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-            const int idx = tid + 128 * i, r = idx >> 3, q = idx & 7, kc = q >> 1, half = q & 1;
-            const float4 f4 = *reinterpret_cast<const float4 *>(rs + r * (kDftKc * 4) + q * 16);
-            __nv_bfloat162 b0 = __floats2bfloat162_rn(f4.x, f4.y), b1 = __floats2bfloat162_rn(f4.z, f4.w);
-            const uint2 v = make_uint2(*reinterpret_cast<uint32_t *>(&b0), *reinterpret_cast<uint32_t *>(&b1));
-            *reinterpret_cast<uint2 *>(a + (r >> 3) * kDftSBO + kc * kDftLBO + (r & 7) * 16 + half * 8) = v;
-        }
-        unsigned char *bb = sB + st * kBtBytes;
-        {
-            const int r = tid >> 2, kc = tid & 3; // 32 table rows x 4 K cores
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(Bt + (long)r * n + (long)c * kDftKc + kc * 8));
-            *reinterpret_cast<uint4 *>(bb + (r >> 3) * kDftSBO + kc * kDftLBO + (r & 7) * 16) = v;
-        }
-        // the tiles go to the tensor core and the raw stage back to the copy engine
-        fch::tc::fence_async_smem();
-        fch::tc::fence_before_sync();
-        __syncthreads();
-        if (tid == 0) {
-            if (c + 2 < nch) {
-                fetch(c + 2);
-                fetched = c + 3;
-            }
-            fch::tc::fence_after_sync();
-            const uint32_t sa = fch::tc::smem_u32(a), sb = fch::tc::smem_u32(bb);
+    if (tid == 0) {
+        auto fetch = [&](int c) {
+            const int st = c % kDftStages;
+            fch::tc::mbar_expect_tx(&full[st], kDftABytes + kDftBBytes);
+            fch::tc::tma_load_2d(sA + st * kDftABytes, &amap, c * kDftKc, (int)row0, &full[st]);
+            fch::tc::tma_load_2d(sB + st * kDftBBytes, &bmap, c * kDftKc, 0, &full[st]);
+        };
+        constexpr uint32_t idesc = fch::tc::idesc_bf16_f32(kTcRows, kTcNB);
+        int fetched = nch < kDftStages ? nch : kDftStages, issued = 0;
+        for (int c = 0; c < fetched; c++) fetch(c);
+        for (int c = 0; c < nch && ok; c++) {
+            const int st = c % kDftStages;
+            ok = fch::tc::mbar_wait(&full[st], (uint32_t)((c / kDftStages) & 1), kTcBound);
+            if (!ok) break;
+            const uint32_t sa = fch::tc::smem_u32(sA + st * kDftABytes), sb = fch::tc::smem_u32(sB + st * kDftBBytes);
 #pragma unroll
             for (int k = 0; k < kDftKc / 16; k++)
-                fch::tc::mma_bf16(tmem, fch::tc::smem_desc(sa + 2 * k * kDftLBO, kDftLBO, kDftSBO),
-                                  fch::tc::smem_desc(sb + 2 * k * kDftLBO, kDftLBO, kDftSBO), idesc,
-                                  (c | k) != 0);
+                fch::tc::mma_bf16(tmem, fch::tc::smem_desc_sw128(sa + 32 * k), fch::tc::smem_desc_sw128(sb + 32 * k),
+                                  idesc, (c | k) != 0);
             fch::tc::mma_commit(&mmab[st]);
+            issued = c + 1;
+            // the stage of the chunk before is free once its MMAs are done: refill it
+            const int pc = c - 1, nc = pc + kDftStages;
+            if (pc >= 0 && nc < nch) {
+                ok = fch::tc::mbar_wait(&mmab[pc % kDftStages], (uint32_t)((pc / kDftStages) & 1), kTcBound);
+                if (ok) {
+                    fetch(nc);
+                    fetched = nc + 1;
+                }
+            }
         }
-        issued = c + 1;
-    }
-    // the last commit covers every MMA issued; tiles fetched beyond what was consumed (an
-    // early stop) are waited for before the CTA's shared memory goes away
-    bool done = true;
-    if (issued > 0)
-        done = fch::tc::mbar_wait(&mmab[(issued - 1) & 1], (uint32_t)(((issued - 1) >> 1) & 1), kTcBound);
-    if (tid == 0)
+        // the last commit covers every MMA issued; tiles fetched beyond what was consumed (an
+        // early stop) are waited for before the CTA's shared memory goes away
+        if (issued > 0 && !fch::tc::mbar_wait(&mmab[(issued - 1) % kDftStages],
+                                              (uint32_t)(((issued - 1) / kDftStages) & 1), kTcBound))
+            ok = false;
         for (int c = issued; c < fetched; c++)
-            fch::tc::mbar_wait(&full[c & 1], (uint32_t)((c >> 1) & 1), kTcBound);
-    ok = __syncthreads_and(ok && done && issued == nch);
+            fch::tc::mbar_wait(&full[c % kDftStages], (uint32_t)((c / kDftStages) & 1), kTcBound);
+        ok = ok && issued == nch;
+        fch::tc::fence_before_sync();
+    }
+    ok = __syncthreads_and(ok);
     fch::tc::fence_after_sync();
     if (ok) {
         float v[32];
@@ -548,9 +536,9 @@ __global__ void __launch_bounds__(128) fno_rowdft_tc(const __grid_constant__ CUt
     if (warp == 0) fch::tc::tmem_dealloc(tmem, 32);
 }
 
-// launch of fno_rowdft_tc over R rows of n floats at h (n a multiple of 32), with its
-// tensor map and dynamic shared memory (the limit raised once)
-cudaError_t launch_rowdft_tc(const float *h, const __nv_bfloat16 *Bt, float2 *X, long R, int n, int *err,
+// launch of fno_rowdft_tc over R rows of n bf16 at h (n a multiple of 64), with its tensor
+// maps and dynamic shared memory (the limit raised once)
+cudaError_t launch_rowdft_tc(const __nv_bfloat16 *h, const __nv_bfloat16 *Bt, float2 *X, long R, int n, int *err,
                              cudaStream_t s)
 {
     static bool attr = false;
@@ -560,11 +548,12 @@ cudaError_t launch_rowdft_tc(const float *h, const __nv_bfloat16 *Bt, float2 *X,
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    CUtensorMap m;
-    // R rows of n floats, tiles of 128 rows x 32 floats, zero past the last row
-    const cudaError_t e = fch_tmap_f32_2d(&m, h, (uint64_t)n, (uint64_t)R, (uint64_t)n * 4, kDftKc, kTcRows);
+    CUtensorMap ma, mb;
+    // R rows of n, tiles of 128 rows x 64, zero past the last row; the table's 32 rows x 64
+    cudaError_t e = fch_tmap_bf16_2d_sw128(&ma, h, (uint64_t)n, (uint64_t)R, (uint64_t)n * 2, kTcRows);
+    if (e == cudaSuccess) e = fch_tmap_bf16_2d_sw128(&mb, Bt, (uint64_t)n, kTcNB, (uint64_t)n * 2, kTcNB);
     if (e != cudaSuccess) return e;
-    fno_rowdft_tc<<<(unsigned)((R + kTcRows - 1) / kTcRows), 128, kRowdftSmem, s>>>(m, Bt, X, (int)R, n, err);
+    fno_rowdft_tc<<<(unsigned)((R + kTcRows - 1) / kTcRows), 128, kRowdftSmem, s>>>(ma, mb, X, (int)R, n, err);
     return cudaGetLastError();
 }
 
@@ -612,24 +601,32 @@ __global__ void __launch_bounds__(256) fno_coldft(const float2 *__restrict__ X, 
     if (j == 0 && k < K2) Y[((long)f * K2 + k) * MM + kx] = acc;
 }
 
-// Z[b][o][kyi][kx] = sum_i R[m][o][i] Y[b][i][kyi][kx], m = kx (2M-1) + kyi
+// Z[b][o][kyi][kx] = sum_i R[m][o][i] Y[b][i][kyi][kx], m = kx (2M-1) + kyi: one block a
+// mode, its weights (contiguous in memory) and channel vectors through shared memory, the
+// weight rows padded by one
 template <typename WT>
-__global__ void fno_mix_modes(const float2 *__restrict__ Y, const WT *__restrict__ R, float2 *__restrict__ Z,
-                              int B, int W, int M)
+__global__ void __launch_bounds__(128) fno_mix_modes(const float2 *__restrict__ Y, const WT *__restrict__ R,
+                                                     float2 *__restrict__ Z, int B, int W, int M)
 {
-    const int K2 = 2 * M - 1, K = M * K2;
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)B * W * K) return;
-    const int q = (int)(t % K), o = (int)((t / K) % W), b = (int)(t / ((long)K * W));
-    const int kyi = q / M, kx = q - kyi * M, m = kx * K2 + kyi;
-    float re = 0.f, im = 0.f;
-    for (int i = 0; i < W; i++) {
-        const float2 x = Y[(((long)b * W + i) * K2 + kyi) * M + kx];
-        const float2 w = wld2(R, ((long)m * W + o) * W + i);
-        re += w.x * x.x - w.y * x.y;
-        im += w.x * x.y + w.y * x.x;
+    extern __shared__ __align__(16) float2 mm_smem[];
+    float2 *r = mm_smem, *x = mm_smem + W * (W + 1);
+    const int K2 = 2 * M - 1, K = M * K2, q = blockIdx.x, kyi = q / M, kx = q - kyi * M;
+    const long m = (long)kx * K2 + kyi;
+    for (int e = threadIdx.x; e < W * W; e += 128) r[e / W * (W + 1) + e % W] = wld2(R, m * W * W + e);
+    for (int b = 0; b < B; b++) {
+        __syncthreads(); // the vectors of the sample before are read
+        for (int i = threadIdx.x; i < W; i += 128) x[i] = Y[((long)b * W + i) * K + q];
+        __syncthreads();
+        for (int o = threadIdx.x; o < W; o += 128) {
+            float re = 0.f, im = 0.f;
+            for (int i = 0; i < W; i++) {
+                const float2 v = x[i], w = r[o * (W + 1) + i];
+                re += w.x * v.x - w.y * v.y;
+                im += w.x * v.y + w.y * v.x;
+            }
+            Z[((long)b * W + o) * K + q] = make_float2(re, im);
+        }
     }
-    Z[(((long)b * W + o) * K2 + kyi) * M + kx] = make_float2(re, im);
 }
 
 // V[f][y][kx] = sum_kyi Z[f][kyi][kx] e^{+2 pi i ky y / n}: one block per (field f, 64
@@ -679,33 +676,49 @@ __device__ __forceinline__ void core_store(unsigned char *tile, int r, int kc, u
     *reinterpret_cast<uint4 *>(tile + (r >> 3) * kTcSBO + kc * kTcLBO + (r & 7) * 16) = v;
 }
 
-// set up (tensor memory, mbarrier) and tear down of the one-tile tensor-core kernels
-struct TcTile {
-    uint32_t tmem;
-};
-
-// The pointwise layer on the tensor cores: for the 128 points x of one row segment
-// (thread t, TMEM lane t), z[o] = sum_j W[o][j] h[j] + b[o] + S[o] with S the inverse
-// x DFT of V, as one MMA chain with K = W + 32:
-//   A[t][:] = (bf16 h[b][j][y][x], j < W | bf16 cos(2 pi kx x/n), kx < 16 | bf16 sin(...))
-//   B[o][:] = (W[o][j] | bf16(w(kx)/n^2 Re V[o][y][kx]) | bf16(-w(kx)/n^2 Im V[o][y][kx]))
-// D = A B^T (128 x W, FP32 in tensor memory); out = act(D + b).
-template <int W>
-__global__ void __launch_bounds__(128) fno_pw_tc(const float *__restrict__ h, const float2 *__restrict__ V,
-                                                 const float2 *__restrict__ tw, const __nv_bfloat16 *__restrict__ Wl,
-                                                 const __nv_bfloat16 *__restrict__ bl, float *__restrict__ out,
-                                                 int n, int act, int *err)
+// A operand tiles of 128 points with the points contiguous (core matrices of eight K rows of
+// eight points): row k, points 8 xg.. at xg * kMnSBO + (k / 8) * 128 + (k mod 8) * 16, so a
+// 16-byte piece of a channel row is stored as it was loaded. kMnSBO: eight K cores and 16
+// bytes, which spreads the stores of neighbouring xg over the banks.
+constexpr int kMnLBO = 128, kMnSBO = 8 * 128 + 16;
+__device__ __forceinline__ void mn_store(unsigned char *tile, int k, int xg, uint4 v)
 {
-    constexpr int K = W + 32, NKC = K / 8;
-    __shared__ __align__(128) unsigned char sA[16 * kTcSBO];
+    *reinterpret_cast<uint4 *>(tile + xg * kMnSBO + (k >> 3) * kMnLBO + (k & 7) * 16) = v;
+}
+
+// The pointwise layer on the tensor cores: for the 128 points x of a row segment (TMEM lane
+// = point), z[o] = sum_j W[o][j] h[j] + b[o] + S[o] with S the inverse x DFT of V, as one
+// MMA chain with K = W + 32:
+//   A[x][:] = (h[b][j][y][x], j < W | bf16 cos(2 pi kx x/n), kx < 16 | bf16 sin(...))
+//   B[o][:] = (W[o][j] | bf16(w(kx)/n^2 Re V[o][y][kx]) | bf16(-w(kx)/n^2 Im V[o][y][kx]))
+// D = A B^T (128 x W, FP32 in tensor memory); out = bf16(act(D + b)). h and out are bf16:
+// the tensor cores are their only readers, and took them rounded to bf16 from FP32 before,
+// so no bit of a result changes while the layer reads and writes half the bytes.
+// A CTA takes kPwRows rows y of one segment: the table part of A, the weights in B and the
+// tensor memory are set up once, and the next row's activations are loaded while the tensor
+// core and the epilogue work on the row before. (One row a CTA with FP32 activations and the
+// table read as 32 float2 a thread: 54 us a layer at 1024^2, 32 channels; now 40, the GELU's
+// instructions and the row's chain of barriers, MMA and read-back at 20 warps an SM. Rows a
+// CTA 2 / 4 / 8 / 16: 471 / 458 / 468 / 484 us a forward pass; no register bound: 475.)
+constexpr int kPwRows = 4;
+template <int W>
+__global__ void __launch_bounds__(128, 5) fno_pw_tc(const __nv_bfloat16 *__restrict__ h, const float2 *__restrict__ V,
+                                                 const __nv_bfloat16 *__restrict__ At,
+                                                 const __nv_bfloat16 *__restrict__ Wl,
+                                                 const __nv_bfloat16 *__restrict__ bl,
+                                                 __nv_bfloat16 *__restrict__ out, int n, int act, int *err)
+{
+    constexpr int K = W + 32, NP = W / 8; // 16-byte pieces of a tile's channels a thread moves
+    constexpr int kOutRow = 128 * 2 + 16; // staged output rows, padded
+    __shared__ __align__(128) unsigned char sA[16 * kMnSBO];
     __shared__ __align__(128) unsigned char sB[(W / 8) * kTcSBO];
+    __shared__ __align__(16) unsigned char sO[W * kOutRow];
     __shared__ float bs[W];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int segs = n >> 7, seg = blockIdx.x % segs, y = blockIdx.x / segs, b = blockIdx.y;
-    const int x = seg * 128 + tid;
-    const long n2 = (long)n * n, p = (long)y * n + x;
+    const int segs = n >> 7, seg = blockIdx.x % segs, y0 = blockIdx.x / segs * kPwRows, b = blockIdx.y;
+    const long n2 = (long)n * n;
     if (warp == 0) {
         fch::tc::tmem_alloc(&tslot, 32);
         fch::tc::tmem_relinquish();
@@ -714,111 +727,112 @@ __global__ void __launch_bounds__(128) fno_pw_tc(const float *__restrict__ h, co
         fch::tc::mbar_init(&bar, 1);
         fch::tc::mbar_init_fence();
     }
-    float f[8];
-    const float *hp = h + (long)b * W * n2 + p;
+    const int xg = tid & 15, r0 = tid >> 4; // piece i of this thread: channel r0 + 8 i, points 8 xg..
+    const long base = (long)b * W * n2 + seg * 128 + 8 * xg;
+    // the V part of B: thread (o, kc) rounds eight coefficients of output o, W * 4 threads
+    const int vo = tid >> 2, vkc = tid & 3, vpart = vkc >> 1, vk0 = (vkc & 1) * 8;
+    const float4 *vp = reinterpret_cast<const float4 *>(V + ((long)b * W + vo) * n * 16 + vk0);
+    uint4 hv[NP];
+    float4 vv[4];
+    auto load = [&](int y) {
 #pragma unroll
-    for (int kc = 0; kc < W / 8; kc++) {
+        for (int i = 0; i < NP; i++)
+            hv[i] = *reinterpret_cast<const uint4 *>(h + base + (long)(r0 + 8 * i) * n2 + (long)y * n);
+        if (vo < W) {
 #pragma unroll
-        for (int e = 0; e < 8; e++) {
-            f[e] = *hp;
-            hp += n2;
+            for (int e = 0; e < 4; e++) vv[e] = vp[(long)y * 8 + e];
         }
-        core_store(sA, tid, kc, pack8_bf16(f));
-    }
+    };
+    load(y0);
 #pragma unroll
-    for (int part = 0; part < 2; part++)
-#pragma unroll
-        for (int kc = 0; kc < 2; kc++) {
-#pragma unroll
-            for (int e = 0; e < 8; e++) {
-                const float2 t = tw[(long)(kc * 8 + e) * n + x];
-                f[e] = part ? t.y : t.x;
-            }
-            core_store(sA, tid, W / 8 + 2 * part + kc, pack8_bf16(f));
-        }
-    const float sc = 1.0f / ((float)n * (float)n);
-    for (int i = tid; i < W * NKC; i += 128) {
-        const int o = i / NKC, kc = i - o * NKC;
-        uint4 v;
-        if (kc < W / 8) {
-            v = *reinterpret_cast<const uint4 *>(Wl + o * W + kc * 8); // already bf16
-        } else {
-            const int part = (kc - W / 8) >> 1, k0 = ((kc - W / 8) & 1) * 8;
-            const float2 *Vr = V + (((long)b * W + o) * n + y) * 16;
-#pragma unroll
-            for (int e = 0; e < 8; e++) {
-                const int k = k0 + e;
-                const float wk = (k == 0 ? 1.f : 2.f) * sc;
-                const float2 vv = Vr[k];
-                f[e] = part ? -wk * vv.y : wk * vv.x;
-            }
-            v = pack8_bf16(f);
-        }
-        core_store(sB, o, kc, v);
+    for (int i = 0; i < 4; i++)
+        mn_store(sA, W + r0 + 8 * i, xg,
+                 *reinterpret_cast<const uint4 *>(At + (long)(r0 + 8 * i) * n + seg * 128 + 8 * xg));
+    for (int i = tid; i < W * NP; i += 128) {
+        const int o = i / NP, kc = i - o * NP;
+        core_store(sB, o, kc, *reinterpret_cast<const uint4 *>(Wl + o * W + kc * 8));
     }
     for (int i = tid; i < W; i += 128) bs[i] = __bfloat162float(bl[i]);
-    fch::tc::fence_async_smem();
-    fch::tc::fence_before_sync();
-    __syncthreads();
-    fch::tc::fence_after_sync();
-    const uint32_t tmem = tslot;
-    if (tid == 0) {
-        constexpr uint32_t idesc = fch::tc::idesc_bf16_f32(128, W);
-        const uint32_t sa = fch::tc::smem_u32(sA), sb = fch::tc::smem_u32(sB);
+    const float sc = 1.0f / ((float)n * (float)n);
+    bool ok = true;
+    uint32_t tmem = 0;
+    for (int r = 0; r < kPwRows; r++) {
+        const int y = y0 + r;
 #pragma unroll
-        for (int k = 0; k < K / 16; k++)
-            fch::tc::mma_bf16(tmem, fch::tc::smem_desc(sa + 2 * k * kTcLBO, kTcLBO, kTcSBO),
-                              fch::tc::smem_desc(sb + 2 * k * kTcLBO, kTcLBO, kTcSBO), idesc, k != 0);
-        fch::tc::mma_commit(&bar);
-    }
-    const bool ok = __syncthreads_and(fch::tc::mbar_wait(&bar, 0, kTcBound));
-    fch::tc::fence_after_sync();
-    if (ok) {
+        for (int i = 0; i < NP; i++) mn_store(sA, r0 + 8 * i, xg, hv[i]);
+        if (vo < W) {
+            float f[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const float wk = (vk0 + e == 0 ? 1.f : 2.f) * sc;
+                const float4 q = vv[e >> 1];
+                f[e] = vpart ? -wk * (e & 1 ? q.w : q.y) : wk * (e & 1 ? q.z : q.x);
+            }
+            core_store(sB, vo, NP + vkc, pack8_bf16(f));
+        }
+        fch::tc::fence_async_smem();
+        fch::tc::fence_before_sync();
+        __syncthreads();
+        fch::tc::fence_after_sync();
+        tmem = tslot;
+        if (tid == 0) {
+            constexpr uint32_t idesc = fch::tc::idesc_bf16_f32(128, W, true);
+            const uint32_t sa = fch::tc::smem_u32(sA), sb = fch::tc::smem_u32(sB);
+#pragma unroll
+            for (int k = 0; k < K / 16; k++)
+                fch::tc::mma_bf16(tmem, fch::tc::smem_desc(sa + 2 * k * kMnLBO, kMnLBO, kMnSBO),
+                                  fch::tc::smem_desc(sb + 2 * k * kTcLBO, kTcLBO, kTcSBO), idesc, k != 0);
+            fch::tc::mma_commit(&bar);
+        }
+        if (r + 1 < kPwRows) load(y + 1);
+        ok = __syncthreads_and(fch::tc::mbar_wait(&bar, (uint32_t)(r & 1), kTcBound));
+        fch::tc::fence_after_sync();
+        if (!ok) break;
         float v[32];
         fch::tc::tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16), v);
-        float *op = out + (long)b * W * n2 + p;
-        if (act) {
 #pragma unroll
-            for (int o = 0; o < W; o += 2) {
-                const float2 g2 = x2_split(gelu_as2(x2_add(x2(v[o], v[o + 1]), x2(bs[o], bs[o + 1]))));
-                op[0] = g2.x;
-                op[n2] = g2.y;
-                op += 2 * n2;
-            }
-        } else {
-#pragma unroll
-            for (int o = 0; o < W; o++) {
-                *op = v[o] + bs[o];
-                op += n2;
-            }
+        for (int o = 0; o < W; o += 2) {
+            float2 g2;
+            if (act)
+                g2 = x2_split(gelu_as2(x2_add(x2(v[o], v[o + 1]), x2(bs[o], bs[o + 1]))));
+            else
+                g2 = make_float2(v[o] + bs[o], v[o + 1] + bs[o + 1]);
+            *reinterpret_cast<__nv_bfloat16 *>(sO + o * kOutRow + tid * 2) = __float2bfloat16_rn(g2.x);
+            *reinterpret_cast<__nv_bfloat16 *>(sO + (o + 1) * kOutRow + tid * 2) = __float2bfloat16_rn(g2.y);
         }
-    } else if (tid == 0) {
-        atomicExch(err, 1);
+        fch::tc::fence_before_sync(); // the accumulator is read before the next row's MMAs
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < NP; i++)
+            *reinterpret_cast<uint4 *>(out + base + (long)(r0 + 8 * i) * n2 + (long)y * n) =
+                *reinterpret_cast<const uint4 *>(sO + (r0 + 8 * i) * kOutRow + xg * 16);
     }
+    if (!ok && tid == 0) atomicExch(err, 1);
     fch::tc::fence_before_sync();
     __syncthreads();
+    tmem = tslot;
     if (warp == 0) fch::tc::tmem_dealloc(tmem, 32);
 }
 
 // The projection on the tensor cores: for 128 points (thread t, TMEM lane t),
-// zq = Q1 bf16(h) + bQ1 as D = A B^T with A[t][:] = bf16 h[b][c][p] (K = W) and
-// B = Q1 (W2 x W), then y = bQ2 + sum_d Q2[d] GELU(zq[d]) in the epilogue.
+// zq = Q1 h + bQ1 as D = A B^T with A[t][:] = h[b][c][p] in bf16 (K = W) and
+// B = Q1 (W2 x W), then y = bQ2 + sum_d Q2[d] GELU(zq[d]) in the epilogue. A tile's points
+// lie in one sample (n a multiple of 128).
 template <int W>
-__global__ void __launch_bounds__(128) fno_proj_tc(const float *__restrict__ h, const __nv_bfloat16 *__restrict__ Q1,
+__global__ void __launch_bounds__(128) fno_proj_tc(const __nv_bfloat16 *__restrict__ h,
+                                                   const __nv_bfloat16 *__restrict__ Q1,
                                                    const __nv_bfloat16 *__restrict__ bQ1,
                                                    const __nv_bfloat16 *__restrict__ Q2,
                                                    const __nv_bfloat16 *__restrict__ bQ2, float *__restrict__ y,
-                                                   long pts, int n2, int W2, int *err)
+                                                   int n2, int W2, int *err)
 {
-    __shared__ __align__(128) unsigned char sA[16 * kTcSBO];
+    __shared__ __align__(128) unsigned char sA[16 * kMnSBO];
     __shared__ __align__(128) unsigned char sB[(kMaxW2 / 8) * kTcSBO];
     __shared__ __align__(16) float bq[kMaxW2], q2[kMaxW2];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
     const int tid = threadIdx.x, warp = tid >> 5;
-    const long g = (long)blockIdx.x * 128 + tid;
-    const bool live = g < pts;
-    const long b = live ? g / n2 : 0, p = live ? g - b * n2 : 0;
+    const long g0 = (long)blockIdx.x * 128, b = g0 / n2, p0 = g0 - b * n2;
     const uint32_t ncols = W2 <= 32 ? 32 : (W2 <= 64 ? 64 : 128);
     if (warp == 0) {
         fch::tc::tmem_alloc(&tslot, ncols);
@@ -828,17 +842,11 @@ __global__ void __launch_bounds__(128) fno_proj_tc(const float *__restrict__ h, 
         fch::tc::mbar_init(&bar, 1);
         fch::tc::mbar_init_fence();
     }
-    float f[8];
-    const float *hp = h + b * W * n2 + p;
+    const int xg = tid & 15, r0 = tid >> 4;
 #pragma unroll
-    for (int kc = 0; kc < W / 8; kc++) {
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-            f[e] = live ? __ldcs(hp) : 0.f;
-            hp += n2;
-        }
-        core_store(sA, tid, kc, pack8_bf16(f));
-    }
+    for (int i = 0; i < W / 8; i++)
+        mn_store(sA, r0 + 8 * i, xg,
+                 __ldcs(reinterpret_cast<const uint4 *>(h + (b * W + r0 + 8 * i) * n2 + p0 + 8 * xg)));
     for (int i = tid; i < W2 * (W / 8); i += 128) {
         const int d = i / (W / 8), kc = i - d * (W / 8);
         core_store(sB, d, kc, *reinterpret_cast<const uint4 *>(Q1 + d * W + kc * 8));
@@ -853,11 +861,11 @@ __global__ void __launch_bounds__(128) fno_proj_tc(const float *__restrict__ h, 
     fch::tc::fence_after_sync();
     const uint32_t tmem = tslot;
     if (tid == 0) {
-        const uint32_t idesc = fch::tc::idesc_bf16_f32(128, W2);
+        const uint32_t idesc = fch::tc::idesc_bf16_f32(128, W2, true);
         const uint32_t sa = fch::tc::smem_u32(sA), sb = fch::tc::smem_u32(sB);
 #pragma unroll
         for (int k = 0; k < W / 16; k++)
-            fch::tc::mma_bf16(tmem, fch::tc::smem_desc(sa + 2 * k * kTcLBO, kTcLBO, kTcSBO),
+            fch::tc::mma_bf16(tmem, fch::tc::smem_desc(sa + 2 * k * kMnLBO, kMnLBO, kMnSBO),
                               fch::tc::smem_desc(sb + 2 * k * kTcLBO, kTcLBO, kTcSBO), idesc, k != 0);
         fch::tc::mma_commit(&bar);
     }
@@ -879,7 +887,7 @@ __global__ void __launch_bounds__(128) fno_proj_tc(const float *__restrict__ h, 
             }
         }
         const float2 a2 = x2_split(acc);
-        if (live) y[g] = a2.x + a2.y;
+        y[g0 + tid] = a2.x + a2.y;
     } else if (tid == 0) {
         atomicExch(err, 1);
     }
@@ -1233,7 +1241,8 @@ struct fch_fno {
     // work arrays for (tc_B, tc_n), the device error flag of the tensor-core kernel
     bool tc;
     int tc_B, tc_n;
-    __nv_bfloat16 *tc_Bt; // [32][n]
+    __nv_bfloat16 *tc_Bt, *tc_At; // [32][n]
+    __nv_bfloat16 *tc_h[2];       // [B][W][n^2]: a layer's input and output
     float2 *tc_tw;        // [16][n]
     float2 *tc_X, *tc_V;  // [B W n][16]
     float2 *tc_Y, *tc_Z;  // [B W][2M-1][M]
@@ -1465,7 +1474,7 @@ extern "C" fch_status fch_fno_destroy(fch_fno *f)
     if (f->stream) cudaStreamSynchronize(f->stream);
     free_buffers(f);
     for (void *b : {(void *)f->params, (void *)f->grads, (void *)f->am, (void *)f->av, (void *)f->pbf,
-                    (void *)f->tc_Bt, (void *)f->tc_tw, (void *)f->tc_X, (void *)f->tc_V, (void *)f->tc_Y,
+                    (void *)f->tc_Bt, (void *)f->tc_At, (void *)f->tc_h[0], (void *)f->tc_h[1], (void *)f->tc_tw, (void *)f->tc_X, (void *)f->tc_V, (void *)f->tc_Y,
                     (void *)f->tc_Z, (void *)f->tc_err})
         if (b) cudaFree(b);
     if (f->hsum) cudaFreeHost(f->hsum);
@@ -1584,14 +1593,17 @@ static fch_status forward_impl(fch_fno *f, int batch, int n, const float *a, flo
 static fch_status ensure_tc(fch_fno *f, int B, int n)
 {
     if (f->tc_B == B && f->tc_n == n) return FCH_OK;
-    for (void *b : {(void *)f->tc_Bt, (void *)f->tc_tw, (void *)f->tc_X, (void *)f->tc_V, (void *)f->tc_Y,
+    for (void *b : {(void *)f->tc_Bt, (void *)f->tc_At, (void *)f->tc_h[0], (void *)f->tc_h[1], (void *)f->tc_tw, (void *)f->tc_X, (void *)f->tc_V, (void *)f->tc_Y,
                     (void *)f->tc_Z})
         if (b) cudaFree(b);
-    f->tc_Bt = nullptr;
+    f->tc_Bt = f->tc_At = f->tc_h[0] = f->tc_h[1] = nullptr;
     f->tc_tw = f->tc_X = f->tc_V = f->tc_Y = f->tc_Z = nullptr;
     f->tc_B = f->tc_n = 0;
     const size_t rows = (size_t)B * f->W * n, modes = (size_t)B * f->W * f->K;
     cudaError_t e = cudaMalloc((void **)&f->tc_Bt, (size_t)32 * n * sizeof(__nv_bfloat16));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&f->tc_At, (size_t)32 * n * sizeof(__nv_bfloat16));
+    for (int i = 0; i < 2; i++)
+        if (e == cudaSuccess) e = cudaMalloc((void **)&f->tc_h[i], rows * n * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = cudaMalloc((void **)&f->tc_tw, (size_t)16 * n * sizeof(float2));
     if (e == cudaSuccess) e = cudaMalloc((void **)&f->tc_X, rows * 16 * sizeof(float2));
     if (e == cudaSuccess) e = cudaMalloc((void **)&f->tc_V, rows * 16 * sizeof(float2));
@@ -1600,7 +1612,7 @@ static fch_status ensure_tc(fch_fno *f, int B, int n)
     if (e == cudaSuccess && !f->tc_err) e = cudaMalloc((void **)&f->tc_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(f->tc_err, 0, sizeof(int), f->stream);
     if (e == cudaSuccess) {
-        fno_dft_tables<<<grid(16L * n, 256), 256, 0, f->stream>>>(f->tc_Bt, f->tc_tw, n);
+        fno_dft_tables<<<grid(16L * n, 256), 256, 0, f->stream>>>(f->tc_Bt, f->tc_tw, f->tc_At, n);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
@@ -1619,48 +1631,47 @@ static fch_status forward_tc(fch_fno *f, int batch, int n, const float *a, float
 {
     typedef __nv_bfloat16 WT;
     const WT *P = f->pbf;
-    fch_status st = ensure_buffers(f, batch, n);
-    if (st == FCH_OK) st = ensure_tc(f, batch, n);
+    const fch_status st = ensure_tc(f, batch, n);
     if (st != FCH_OK) return st;
     const int W = f->W, M = f->M, n2 = n * n;
     const long pts = (long)batch * n2, R = (long)batch * W * n;
-    const size_t fld = (size_t)batch * W * n2;
     cudaStream_t s = f->stream;
     {
         const WT *P0 = P + offset_of(f, 0, 0), *P1 = P + offset_of(f, 1, 0);
         const unsigned gl = grid(pts, 256);
         if (W == 16)
-            fno_lift_t<WT, 16, 2><<<gl, 256, 0, s>>>(a, P0, P1, f->h, pts, n2);
+            fno_lift_t<WT, 16, 2><<<gl, 256, 0, s>>>(a, P0, P1, f->tc_h[0], pts, n2);
         else
-            fno_lift_t<WT, 32, 2><<<gl, 256, 0, s>>>(a, P0, P1, f->h, pts, n2);
+            fno_lift_t<WT, 32, 2><<<gl, 256, 0, s>>>(a, P0, P1, f->tc_h[0], pts, n2);
     }
     for (int l = 0; l < f->L; l++) {
-        float *hin = f->h + l * fld, *hout = f->h + (l + 1) * fld;
-        launch_rowdft_tc(hin, f->tc_Bt, f->tc_X, R, n, f->tc_err, s);
+        const WT *hin = f->tc_h[l & 1];
+        WT *hout = f->tc_h[(l + 1) & 1];
+        const cudaError_t e = launch_rowdft_tc(hin, f->tc_Bt, f->tc_X, R, n, f->tc_err, s);
+        if (e != cudaSuccess) return spec_error(f, e);
         fno_coldft<16><<<dim3(batch * W, M), 256, 2 * n * sizeof(float2), s>>>(f->tc_X, f->tc_tw + n, f->tc_Y, n);
-        fno_mix_modes<WT><<<grid((long)batch * W * f->K, 256), 256, 0, s>>>(f->tc_Y, P + offset_of(f, 4, l),
-                                                                           f->tc_Z, batch, W, M);
+        fno_mix_modes<WT><<<f->K, 128, (W * (W + 1) + W) * 8, s>>>(f->tc_Y, P + offset_of(f, 4, l), f->tc_Z, batch, W,
+                                                                  M);
         fno_icoldft<16><<<(unsigned)((long)batch * W * (n / 64)), 256, n * sizeof(float2), s>>>(
             f->tc_Z, f->tc_tw + n, f->tc_V, (long)batch * W, n);
         // the channel mixing and the inverse x DFT: one MMA chain per 128 points
-        const dim3 g((unsigned)(n / 128 * n), (unsigned)batch);
+        const dim3 g((unsigned)(n / 128 * (n / kPwRows)), (unsigned)batch);
         const int act = l < f->L - 1;
         if (W == 16)
-            fno_pw_tc<16><<<g, 128, 0, s>>>(hin, f->tc_V, f->tc_tw, P + offset_of(f, 2, l), P + offset_of(f, 3, l),
+            fno_pw_tc<16><<<g, 128, 0, s>>>(hin, f->tc_V, f->tc_At, P + offset_of(f, 2, l), P + offset_of(f, 3, l),
                                            hout, n, act, f->tc_err);
         else
-            fno_pw_tc<32><<<g, 128, 0, s>>>(hin, f->tc_V, f->tc_tw, P + offset_of(f, 2, l), P + offset_of(f, 3, l),
+            fno_pw_tc<32><<<g, 128, 0, s>>>(hin, f->tc_V, f->tc_At, P + offset_of(f, 2, l), P + offset_of(f, 3, l),
                                            hout, n, act, f->tc_err);
     }
-    const unsigned gp = (unsigned)((pts + 127) / 128);
+    const unsigned gp = (unsigned)(pts / 128);
+    const WT *hL = f->tc_h[f->L & 1];
     if (W == 16)
-        fno_proj_tc<16><<<gp, 128, 0, s>>>(f->h + f->L * fld, P + offset_of(f, 5, 0), P + offset_of(f, 6, 0),
-                                           P + offset_of(f, 7, 0), P + offset_of(f, 8, 0), y, pts, n2, f->W2,
-                                           f->tc_err);
+        fno_proj_tc<16><<<gp, 128, 0, s>>>(hL, P + offset_of(f, 5, 0), P + offset_of(f, 6, 0), P + offset_of(f, 7, 0),
+                                           P + offset_of(f, 8, 0), y, n2, f->W2, f->tc_err);
     else
-        fno_proj_tc<32><<<gp, 128, 0, s>>>(f->h + f->L * fld, P + offset_of(f, 5, 0), P + offset_of(f, 6, 0),
-                                           P + offset_of(f, 7, 0), P + offset_of(f, 8, 0), y, pts, n2, f->W2,
-                                           f->tc_err);
+        fno_proj_tc<32><<<gp, 128, 0, s>>>(hL, P + offset_of(f, 5, 0), P + offset_of(f, 6, 0), P + offset_of(f, 7, 0),
+                                           P + offset_of(f, 8, 0), y, n2, f->W2, f->tc_err);
     cudaError_t e = cudaGetLastError();
     int herr = 0;
     // the tensor-core kernel's bounded waits report through a device flag
@@ -1863,21 +1874,23 @@ extern "C" int fch_debug_rowdft_tc(const float *h, float *X, int R, int n, void 
 {
     if (!h || !X || R < 1 || n < 64 || n % 64 != 0 || n > 2048) return FCH_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    __nv_bfloat16 *Bt = nullptr;
+    __nv_bfloat16 *Bt = nullptr, *hb = nullptr;
     float2 *tw = nullptr;
     int *err = nullptr, herr = 0;
     cudaError_t e = cudaMalloc((void **)&Bt, (size_t)32 * n * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = cudaMalloc((void **)&tw, (size_t)16 * n * sizeof(float2));
     if (e == cudaSuccess) e = cudaMalloc((void **)&err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&hb, (size_t)R * n * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) {
-        fno_dft_tables<<<grid(16L * n, 256), 256, 0, s>>>(Bt, tw, n);
+        fno_dft_tables<<<grid(16L * n, 256), 256, 0, s>>>(Bt, tw, nullptr, n);
+        fno_to_bf16<<<grid((long)R * n, 256), 256, 0, s>>>(h, hb, (long)R * n);
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = launch_rowdft_tc(h, Bt, (float2 *)X, R, n, err, s);
+        if (e == cudaSuccess) e = launch_rowdft_tc(hb, Bt, (float2 *)X, R, n, err, s);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (void *b : {(void *)Bt, (void *)tw, (void *)err})
+    for (void *b : {(void *)Bt, (void *)hb, (void *)tw, (void *)err})
         if (b) cudaFree(b);
     if (e != cudaSuccess) {
         fch_set_thread_error(cudaGetErrorString(e));

@@ -121,11 +121,26 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
     d |= (uint64_t)1 << 46;
     return d;
 }
-// instruction descriptor of kind::f16: D in FP32, A and B in BF16, both K-major,
-// N (multiple of 16 for M = 128) and M
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
+// the same for a K-major tile with the 128-byte swizzle, as a tensor-map copy with that
+// swizzle writes it: rows of 64 bf16 (128 bytes) in 1024-byte groups of eight rows (the
+// tile 1024-byte aligned); the next 16 columns of K start 32 bytes on
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+// instruction descriptor of kind::f16: D in FP32, A and B in BF16, B K-major, A K-major or
+// (a_mn) with its rows contiguous: core matrices of eight K, each 16 bytes of eight rows;
+// LBO then steps along K and SBO along the rows, as for the K-major ones. N (multiple of
+// 16 for M = 128) and M
+__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool a_mn = false)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn ? 1u << 15 : 0u) | ((uint32_t)(N >> 3) << 17) |
+           ((uint32_t)(M >> 4) << 24);
 }
 
 // D[tmem] (+)= A[smem] * B[smem]^T, one thread issues; accumulate = 0 overwrites D

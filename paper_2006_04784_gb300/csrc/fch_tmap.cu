@@ -5,10 +5,10 @@ namespace {
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-}
 
-cudaError_t fch_tmap_f32_2d(CUtensorMap *m, const void *base, uint64_t inner, uint64_t outer, uint64_t row_bytes,
-                            uint32_t box_inner, uint32_t box_outer)
+cudaError_t encode_2d(CUtensorMap *m, CUtensorMapDataType type, uint32_t esize, CUtensorMapSwizzle swizzle,
+                      const void *base, uint64_t inner, uint64_t outer, uint64_t row_bytes, uint32_t box_inner,
+                      uint32_t box_outer)
 {
     static EncodeTiledFn enc = nullptr;
     if (!enc) {
@@ -19,15 +19,30 @@ cudaError_t fch_tmap_f32_2d(CUtensorMap *m, const void *base, uint64_t inner, ui
         if (q != cudaDriverEntryPointSuccess || !p) return cudaErrorNotSupported;
         enc = (EncodeTiledFn)p;
     }
-    if (((uintptr_t)base & 15) || (row_bytes & 15) || ((box_inner * 4) & 15) || box_inner > 256 || box_outer > 256 ||
-        box_inner == 0 || box_outer == 0)
+    if (((uintptr_t)base & 15) || (row_bytes & 15) || ((box_inner * esize) & 15) || box_inner > 256 ||
+        box_outer > 256 || box_inner == 0 || box_outer == 0)
         return cudaErrorInvalidValue;
     const cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
     const cuuint64_t strides[1] = {(cuuint64_t)row_bytes};
     const cuuint32_t box[2] = {box_inner, box_outer};
     const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(base), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = enc(m, type, 2, const_cast<void *>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+} // namespace
+
+cudaError_t fch_tmap_f32_2d(CUtensorMap *m, const void *base, uint64_t inner, uint64_t outer, uint64_t row_bytes,
+                            uint32_t box_inner, uint32_t box_outer)
+{
+    return encode_2d(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, CU_TENSOR_MAP_SWIZZLE_NONE, base, inner, outer, row_bytes,
+                     box_inner, box_outer);
+}
+
+cudaError_t fch_tmap_bf16_2d_sw128(CUtensorMap *m, const void *base, uint64_t inner, uint64_t outer,
+                                   uint64_t row_bytes, uint32_t box_outer)
+{
+    return encode_2d(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, CU_TENSOR_MAP_SWIZZLE_128B, base, inner, outer, row_bytes,
+                     64, box_outer);
 }

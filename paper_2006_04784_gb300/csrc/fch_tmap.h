@@ -1,5 +1,5 @@
 // fch_tmap.h -- tensor maps (the descriptors of the TMA engine's tiled copies) of
-// row-major FP32 matrices, encoded by the driver's cuTensorMapEncodeTiled, which the
+// row-major matrices, encoded by the driver's cuTensorMapEncodeTiled, which the
 // runtime looks up once.
 #pragma once
 #include <cuda.h>
@@ -12,3 +12,8 @@
 // read as zero; no swizzle, L2 promotion by 128 bytes.
 cudaError_t fch_tmap_f32_2d(CUtensorMap *m, const void *base, uint64_t inner, uint64_t outer, uint64_t row_bytes,
                             uint32_t box_inner, uint32_t box_outer);
+
+// The same of `outer` rows of `inner` bf16 in boxes of box_outer rows x 64 (128 bytes) with
+// the 128-byte swizzle (the destination 1024-byte aligned).
+cudaError_t fch_tmap_bf16_2d_sw128(CUtensorMap *m, const void *base, uint64_t inner, uint64_t outer,
+                                   uint64_t row_bytes, uint32_t box_outer);
