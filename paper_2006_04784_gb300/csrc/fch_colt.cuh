@@ -2,65 +2,39 @@
 // N = 1024 with their input staged by the TMA engine.
 //
 // A tile is P = 2 column pairs: four columns, 32 bytes of every row of the
-// pair-layout work array Z. 512 threads transform its four columns in shared memory
-// as col_pass does (radix-8, 8, 8, 2 Stockham stages over the skewed tile; thread
-// (c, t) = (tid mod 4, tid / 4) works on column c). Blocks are persistent: block b
-// takes tiles b, b + B, b + 2B, ... of all the launch's field pairs (tile g: pair
-// g / 256, column pairs 2 (g mod 256) and the next), and the next tile's input lands
-// in a 32 KB stage while the current tile is transformed:
+// pair-layout work array Z. 512 threads: thread (c, t) = (tid mod 4, tid / 4) holds the
+// points t + 128 m of column c at both ends of the transform, as the passes built for a
+// size do (fch_reg.cuh: column N - kx in its conjugate, inverses as conj, forward, conj).
+// Blocks are persistent: block b takes tiles b, b + B, b + 2B, ... of all the launch's field
+// pairs (tile g: pair g / 256, column pairs 2 (g mod 256) and the next), and the next tile's
+// input lands in a 32 KB stage while the current tile is transformed:
 //  - forward (R2C): four 2D tensor-map boxes of Z (256 rows x 8 floats each,
-//    cp.async.bulk.tensor) fill the stage densely, row n at 32 n bytes. The first
-//    radix-8 stage reads it there (rows t + 128 r of column c: a warp reads 256
-//    contiguous bytes) and writes the skewed tile, after which the stage is free;
-//  - inverse (C2R): the rows kx of the two half spectra (8 KB each, cp.async.bulk)
-//    of the tile's two column pairs; the first radix-8 stage forms its inputs from
-//    them there (the spectral stage folded into it) and writes the skewed tile. The
-//    tile of pair 0 (kx = 0 and N/2 need four rows) reads its spectra from global
-//    memory and takes the separate spectral stage.
-// The forward spectral stage gives each thread rows ky and -ky of the tile, read as
-// whole 32-byte rows, and the four work items that touch only them.
+//    cp.async.bulk.tensor) fill the stage densely, row n at 32 n bytes; a warp's reads of
+//    the first stage's inputs are 256 contiguous bytes;
+//  - inverse (C2R): the rows kx of the two half spectra (8 KB each, cp.async.bulk) of the
+//    tile's two column pairs; both columns of a pair read the same index, natural order.
+//    The tile of pair 0 (kx = 0 and N/2 need four rows) reads its spectra from global memory.
+// The Hermitian split of the forward pass trades one value of a work item each way between
+// lanes c = 0, 1 (2, 3) by shuffles; the inverse stores straight from the last stage, whole
+// 32-byte sectors. Shared memory carries the three exchanges between the stages only: the
+// kernel before went through it eight times a transform (MIO throttle its first stall) and
+// took 38.4 us forward, 50.1 us inverse for eight field pairs.
 // Copies complete in bytes on the block's mbarrier; a wait that runs out of time (1 s)
 // sets *kp.err, and the block stops after waiting (bounded) for the copy it started.
 #pragma once
 #include <cuda.h>
-#include "fch_kernels.cuh"
+#include "fch_reg.cuh"
 #include "fch_tc.cuh"
 
 namespace fch {
 
 constexpr int kColtThreads = 512;
 constexpr int kColtStageBytes = 4 * 1024 * 8;           // the next tile's input
-constexpr int kColtTileBytes = 4 * 1152 * 8;            // four skewed columns (skewed_len(1024) = 1152)
+constexpr int kColtSC = 1152 + 4;                       // a skewed column; the four start 4 elements apart mod 16
+constexpr int kColtTileBytes = 4 * kColtSC * 8;
 constexpr int kColtTwBytes = 1024 * 8;                  // the per-stage twiddles, loaded once a block
 constexpr int kColtSmem = kColtStageBytes + kColtTileBytes + kColtTwBytes + 16 + 128; // + mbarrier, + slack
 constexpr uint64_t kColtWaitNs = 1000000000ull;
-
-// a 32-byte row of four complex values of the tile, as two 16-byte accesses
-__device__ __forceinline__ void load_row4(const float2 *row, float2 *v)
-{
-    const float4 a = *(const float4 *)row, b = *(const float4 *)(row + 2);
-    v[0] = make_float2(a.x, a.y);
-    v[1] = make_float2(a.z, a.w);
-    v[2] = make_float2(b.x, b.y);
-    v[3] = make_float2(b.z, b.w);
-}
-__device__ __forceinline__ void store_row4(float2 *row, const float2 *v)
-{
-    *(float4 *)row = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
-    *(float4 *)(row + 2) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
-}
-
-// the Hermitian split of one work item: z0 = Z(kx, ky), z1 = Z(N - kx, -ky) give
-// A = (z0 + conj z1) / 2 and B = (z0 - conj z1) / (2i) at o0[idx], o1[idx]
-__device__ __forceinline__ void split_store(float2 z0, float2 z1, float2 *o0, float2 *o1, long idx)
-{
-    const float2 c1 = cconj(z1);
-    o0[idx] = cscale(cadd(z0, c1), 0.5f);
-    if (o1) {
-        const float2 dm = csub(z0, c1);
-        o1[idx] = mk<float2>(0.5f * dm.y, -0.5f * dm.x);
-    }
-}
 
 template <int MODE>
 __global__ void __launch_bounds__(kColtThreads, 2) col_pass_t(const fch_kparams kp,
@@ -69,23 +43,20 @@ __global__ void __launch_bounds__(kColtThreads, 2) col_pass_t(const fch_kparams 
     static_assert(MODE == CM_FWD_STORE || MODE == CM_INV_LOAD, "the standalone transform modes");
     typedef float2 C;
     constexpr bool FWD = MODE == CM_FWD_STORE;
-    constexpr int N = 1024, LOGN = 10, NC = 4, NT = kColtThreads;
+    constexpr int N = 1024, NC = 4, NT = kColtThreads, H = 4;
     pdl_begin();
     extern __shared__ unsigned char smem_raw[];
     // the TMA destination wants 128-byte alignment
     unsigned char *base = smem_raw + ((128u - (fch::tc::smem_u32(smem_raw) & 127u)) & 127u);
     C *stage = (C *)base;
     C *tile = (C *)(base + kColtStageBytes);
-    C *tws = (C *)(base + kColtStageBytes + kColtTileBytes);
+    C *tw = (C *)(base + kColtStageBytes + kColtTileBytes);
     uint64_t *bar = (uint64_t *)(base + kColtStageBytes + kColtTileBytes + kColtTwBytes);
-    const int c = threadIdx.x % NC, t = threadIdx.x / NC;
+    const int c = threadIdx.x % NC, t = threadIdx.x / NC, side = c & 1, pp = c >> 1;
     const long npairs = kp.npairs > 1 ? kp.npairs : 1;
     const long ntiles = npairs * (N / 4);
-    for (int i = threadIdx.x; i < N; i += NT) tws[i] = ldg((const C *)kp.tw + i);
-    const C *tw = tws;
-    const fch_consts<float> &K = kp.cf;
-    const fch_coef<float> co = fch_coef<float>();
-    const float inv_n2 = K.inv_n2;
+    for (int i = threadIdx.x; i < N; i += NT) tw[i] = ldg((const C *)kp.tw + i);
+    const float inv_n2 = kp.cf.inv_n2;
     const bool two = kp.in1 != nullptr; // inverse: a second half spectrum
 
     // a tile's input reaches the stage unless it is an inverse tile of pair 0
@@ -103,9 +74,9 @@ __global__ void __launch_bounds__(kColtThreads, 2) col_pass_t(const fch_kparams 
             const char *i1 = two ? (const char *)kp.in1 + pr * kp.pstride_in : nullptr;
             fch::tc::mbar_expect_tx(bar, (two ? 4 : 2) * N * 8);
 #pragma unroll
-            for (int pp = 0; pp < 2; pp++) {
-                fch::tc::bulk_g2s(stage + 2 * pp * N, i0 + (long)(p0 + pp) * N * 8, N * 8, bar);
-                if (two) fch::tc::bulk_g2s(stage + (2 * pp + 1) * N, i1 + (long)(p0 + pp) * N * 8, N * 8, bar);
+            for (int q = 0; q < 2; q++) {
+                fch::tc::bulk_g2s(stage + 2 * q * N, i0 + (long)(p0 + q) * N * 8, N * 8, bar);
+                if (two) fch::tc::bulk_g2s(stage + (2 * q + 1) * N, i1 + (long)(p0 + q) * N * 8, N * 8, bar);
             }
         }
     };
@@ -121,131 +92,102 @@ __global__ void __launch_bounds__(kColtThreads, 2) col_pass_t(const fch_kparams 
     bool ok = true;
     for (; g < ntiles; g += gridDim.x) {
         const long pr = g >> 8;
-        const int p0 = 2 * (int)(g & 255);
-        const bool st = staged(g);
-        if (st) {
+        const int p0 = 2 * (int)(g & 255), p = p0 + pp;
+        if (staged(g)) {
             ok = __syncthreads_and(fch::tc::mbar_wait(bar, phase, kColtWaitNs));
             if (!ok) break;
             phase ^= 1u;
         }
-        ColBufs<C> bf = ColBufs<C>();
-        bf.i0 = kp.in0 ? (const C *)((const char *)kp.in0 + pr * kp.pstride_in) : nullptr;
-        bf.i1 = two ? (const C *)((const char *)kp.in1 + pr * kp.pstride_in) : nullptr;
-        bf.o0 = kp.out0 ? (C *)((char *)kp.out0 + pr * kp.pstride_out) : nullptr;
-        bf.o1 = kp.out1 ? (C *)((char *)kp.out1 + pr * kp.pstride_out) : nullptr;
-        float red[FCH_NRED] = {0.f, 0.f, 0.f, 0.f};
+        C v[8];
         if (FWD) {
-            // first radix-8 stage (no twiddles) from the stage into the skewed tile
-            C v[8];
+            const unsigned m1 = side ? 0x80000000u : 0u;
 #pragma unroll
-            for (int r = 0; r < 8; r++) v[r] = stage[(t + 128 * r) * NC + c];
-            bfly8<-1>(v);
-#pragma unroll
-            for (int r = 0; r < 8; r++) tile[skew(8 * t + r) * NC + c] = v[r];
-            __syncthreads(); // stage consumed, tile written
-            if (threadIdx.x == 0) {
-                fch::tc::fence_async_smem(); // the stage's reads come before the next copy's writes
-                if (g + gridDim.x < ntiles) fetch(g + gridDim.x);
-            }
-            fft_stage<-1, 3, false, 8>(tile, N, LOGN, NC, c, tw, t, 8, 3);
-            fft_stage<-1, 3, false, 8>(tile, N, LOGN, NC, c, tw, t, 64, 6);
-            fft_stage<-1, 1, false, 8>(tile, N, LOGN, NC, c, tw, t, 512, 9);
-            // spectral stage: the Hermitian split into the two half spectra. A thread
-            // owns rows ky and -ky (both 32-byte rows of the tile, read whole) and all
-            // four work items (pair p0 + pp, row ky or -ky) that touch only them.
-            if (p0 > 0) {
-                for (int ky = threadIdx.x; ky <= (N >> 1); ky += NT) {
-                    const int mky = (N - ky) & (N - 1);
-                    C rk[4], rm[4];
-                    load_row4(tile + skew(ky) * NC, rk);
-                    load_row4(tile + skew(mky) * NC, rm);
-#pragma unroll
-                    for (int pp = 0; pp < 2; pp++) {
-                        const long base = (long)(p0 + pp) * N;
-                        // item (pp, ky): slot 0 at row ky, slot 1 at row -ky; item (pp, -ky): the other way
-                        split_store(rk[2 * pp], rm[2 * pp + 1], bf.o0, bf.o1, base + ky);
-                        if (mky != ky) split_store(rm[2 * pp], rk[2 * pp + 1], bf.o0, bf.o1, base + mky);
-                    }
-                }
-            } else {
-                // pair 0 (columns 0 and N/2) and pair 1, item by item
-#pragma unroll 1
-                for (int it = 0; it < 4; it++) {
-                    const int i = threadIdx.x + it * NT;
-                    const int pp = i / N, ky = i - pp * N;
-                    const int s0 = 2 * pp, s1 = 2 * pp + 1;
-                    if (pp > 0) {
-                        const int mky = (N - ky) & (N - 1);
-                        split_store(tile[skew(ky) * NC + s0], tile[skew(mky) * NC + s1], bf.o0, bf.o1,
-                                    (long)pp * N + ky);
-                    } else if (ky <= (N >> 1)) {
-                        pair0_item<float, MODE>(kp, K, co, bf, tile, N, NC, s0, s1, ky, false, red);
-                    }
-                }
+            for (int m = 0; m < 8; m++) {
+                v[m] = stage[(t + 128 * m) * NC + c];
+                v[m].y = flip(v[m].y, m1);
             }
         } else {
-            if (p0 > 0) {
-                // the spectral stage fused into the first radix-8 stage: thread (c, t)
-                // forms rows t + 128 r of column c straight from the staged spectra. With
-                // (C, D) the two half spectra over N^2, slot 0 (column kx) of a pair holds
-                // C + i D at (kx, ky) and slot 1 (column N - kx) conj(C) + i conj(D) taken
-                // at (kx, -ky).
-                const int pp = c >> 1;
-                const bool odd = c & 1;
-                const C *a = stage + 2 * pp * N, *b = stage + (2 * pp + 1) * N;
-                C v[8];
-#pragma unroll
-                for (int r = 0; r < 8; r++) {
-                    const int ky = t + 128 * r, kk = odd ? (N - ky) & (N - 1) : ky;
-                    const C Co = cscale(a[kk], inv_n2);
-                    const C Do = two ? cscale(b[kk], inv_n2) : mk<C>(0.f, 0.f);
-                    v[r] = odd ? mk<C>(Co.x + Do.y, Do.x - Co.y) : mk<C>(Co.x - Do.y, Co.y + Do.x);
-                }
-                bfly8<+1>(v);
-#pragma unroll
-                for (int r = 0; r < 8; r++) tile[skew(8 * t + r) * NC + c] = v[r];
-                __syncthreads(); // stage consumed, tile written
-                if (threadIdx.x == 0) {
-                    fch::tc::fence_async_smem(); // the stage's reads come before the next copy's writes
-                    if (g + gridDim.x < ntiles) fetch(g + gridDim.x);
-                }
-                fft_stage<+1, 3, false, 8>(tile, N, LOGN, NC, c, tw, t, 8, 3);
-                fft_stage<+1, 3, false, 8>(tile, N, LOGN, NC, c, tw, t, 64, 6);
-                fft_stage<+1, 1, false, 8>(tile, N, LOGN, NC, c, tw, t, 512, 9);
+            // (C, D) the two half spectra over N^2: column kx holds conj(C + i D), column
+            // N - kx C* + i D* at the same index (pair 0: column N/2 holds C + i D of -k)
+            const bool own = p0 == 0 && pp == 0;
+            const C *a, *b;
+            if (staged(g)) {
+                a = stage + 2 * pp * N;
+                b = stage + (2 * pp + 1) * N;
             } else {
-                // pair 0 (columns 0 and N/2) and pair 1, item by item from global memory
-#pragma unroll 1
-                for (int it = 0; it < 4; it++) {
-                    const int i = threadIdx.x + it * NT;
-                    const int pp = i / N, ky = i - pp * N;
-                    const int s0 = 2 * pp, s1 = 2 * pp + 1;
-                    if (pp > 0) {
-                        const int mky = (N - ky) & (N - 1);
-                        const C Co = cscale(bf.i0[(long)pp * N + ky], inv_n2);
-                        const C Do = two ? cscale(bf.i1[(long)pp * N + ky], inv_n2) : mk<C>(0.f, 0.f);
-                        tile[skew(ky) * NC + s0] = mk<C>(Co.x - Do.y, Co.y + Do.x);
-                        tile[skew(mky) * NC + s1] = mk<C>(Co.x + Do.y, Do.x - Co.y);
-                    } else if (ky <= (N >> 1)) {
-                        pair0_item<float, MODE>(kp, K, co, bf, tile, N, NC, s0, s1, ky, true, red);
-                    }
-                }
-                __syncthreads();
-                if (threadIdx.x == 0) { // the stage is idle here
-                    fch::tc::fence_async_smem();
-                    if (g + gridDim.x < ntiles) fetch(g + gridDim.x);
-                }
-                fft_smem<+1, false>(tile, N, LOGN, NC, c, tw, t);
+                const long kx = own ? (side ? N / 2 : 0) : 1;
+                a = (const C *)((const char *)kp.in0 + pr * kp.pstride_in) + kx * N;
+                b = two ? (const C *)((const char *)kp.in1 + pr * kp.pstride_in) + kx * N : a;
             }
-            // the four columns back to Z: half a 32-byte row per thread and store
-            C *Z = (C *)kp.Z + pr * N * N;
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const int i = threadIdx.x + k * NT;
-                const int n = i >> 1, h = i & 1;
-                __stcg((float4 *)(Z + (long)n * N + 2 * p0 + 2 * h), *(const float4 *)(tile + skew(n) * NC + 2 * h));
+            for (int m = 0; m < 8; m++) {
+                const int k = t + 128 * m, kk = own && side ? (N - k) & (N - 1) : k;
+                const C Co = cscale(a[kk], inv_n2);
+                const C Do = two ? cscale(b[kk], inv_n2) : mk<C>(0.f, 0.f);
+                if (!side)
+                    v[m] = mk<C>(Co.x - Do.y, -(Co.y + Do.x));
+                else if (!own)
+                    v[m] = mk<C>(Co.x + Do.y, Do.x - Co.y);
+                else
+                    v[m] = mk<C>(Co.x - Do.y, Co.y + Do.x);
             }
         }
-        __syncthreads(); // the tile is read before the next tile's first writes
+        C *buf = tile + c * kColtSC, *none = nullptr;
+        reg_stage<10, 8, 3, 0, false, false, false>(v, buf, none, (const C *)tw, t);
+        // the exchange's barriers: every thread has read the stage
+        if (threadIdx.x == 0) {
+            fch::tc::fence_async_smem(); // the stage's reads come before the next copy's writes
+            if (g + gridDim.x < ntiles) fetch(g + gridDim.x);
+        }
+        reg_stage<10, 8, 3, 1, false, false, false>(v, buf, none, (const C *)tw, t);
+        reg_stage<10, 8, 3, 2, false, false, false>(v, buf, none, (const C *)tw, t);
+        reg_stage<10, 8, 1, 3, false, false, false>(v, buf, none, (const C *)tw, t);
+        if (FWD) {
+            C *o0 = (C *)((char *)kp.out0 + pr * kp.pstride_out);
+            C *o1 = kp.out1 ? (C *)((char *)kp.out1 + pr * kp.pstride_out) : nullptr;
+            // A = (za + zb) / 2, B = (za - zb) / (2i), za = Z(kx, ky), zb = conj Z(N - kx, -ky)
+            auto split = [&](C za, C zb, long idx) {
+                o0[idx] = cscale(cadd(za, zb), 0.5f);
+                if (o1) {
+                    const C dm = csub(za, zb);
+                    o1[idx] = mk<C>(0.5f * dm.y, -0.5f * dm.x);
+                }
+            };
+            C r[H]; // the partner column's values of this thread's work items
+#pragma unroll
+            for (int i = 0; i < H; i++) {
+                const C s = side ? v[i] : v[i + H];
+                r[i] = mk<C>(__shfl_xor_sync(0xffffffffu, s.x, 1), __shfl_xor_sync(0xffffffffu, s.y, 1));
+            }
+            if (p0 == 0) { // pair 0: columns 0 and N/2 pair row k with row -k of themselves
+#pragma unroll
+                for (int m = 0; m < 8; m++) buf[skew(t + 128 * m)] = v[m];
+                __syncthreads();
+            }
+            if (p > 0) {
+#pragma unroll
+                for (int i = 0; i < H; i++) {
+                    const int ky = t + 128 * (side ? i + H : i);
+                    split(side ? r[i] : v[i], side ? v[i + H] : r[i], (long)p * N + ky);
+                }
+            } else {
+#pragma unroll
+                for (int m = 0; m < 8; m++) {
+                    const int k = t + 128 * m, km = (N - k) & (N - 1);
+                    const C zm = buf[skew(km)];
+                    split(side ? cconj(v[m]) : v[m], side ? zm : cconj(zm), side ? (long)(N / 2) * N + km : k);
+                }
+            }
+            if (p0 == 0) __syncthreads(); // the tile is read before the next tile's first writes
+        } else {
+            const unsigned m0 = side ? 0u : 0x80000000u;
+            C *Z = (C *)kp.Z + pr * N * N + 2 * p0 + c;
+#pragma unroll
+            for (int m = 0; m < 8; m++) {
+                v[m].y = flip(v[m].y, m0);
+                __stcg(Z + (long)(t + 128 * m) * N, v[m]);
+            }
+        }
     }
     if (!ok && threadIdx.x == 0) {
         // the copy this block waits for may still land: let it, then report

@@ -89,6 +89,30 @@ template <typename C> __device__ __forceinline__ C badd(C a, C b) { return mk<C>
 template <typename C> __device__ __forceinline__ C bsub(C a, C b) { return mk<C>(rsub(a.x, b.x), rsub(a.y, b.y)); }
 template <typename C> __device__ __forceinline__ C btw(C a, C w) { return cmul(a, w); }
 template <> __device__ __forceinline__ df2 btw(df2 a, df2 w) { return cmul_lazy(a, w); }
+// (single precision: which product is fused is fixed, so that every kernel's transform of
+// the same data gives the same bits)
+template <> __device__ __forceinline__ float2 btw(float2 a, float2 w)
+{
+    return make_float2(__fmaf_rn(-a.y, w.y, __fmul_rn(a.x, w.x)), __fmaf_rn(a.y, w.x, __fmul_rn(a.x, w.y)));
+}
+// p = e + s t, m = e - s t: a fused multiply-add each where there is one (float, double), in
+// double-float the product once
+template <typename C, typename R> __device__ __forceinline__ void bscaled(C e, C t, R s, C &p, C &m)
+{
+    p = mk<C>(fma(t.x, s, e.x), fma(t.y, s, e.y));
+    m = mk<C>(fma(-t.x, s, e.x), fma(-t.y, s, e.y));
+}
+template <> __device__ __forceinline__ void bscaled(float2 e, float2 t, float s, float2 &p, float2 &m)
+{
+    p = make_float2(__fmaf_rn(t.x, s, e.x), __fmaf_rn(t.y, s, e.y));
+    m = make_float2(__fmaf_rn(-t.x, s, e.x), __fmaf_rn(-t.y, s, e.y));
+}
+template <> __device__ __forceinline__ void bscaled(df2 e, df2 t, df s, df2 &p, df2 &m)
+{
+    const df2 o = mk<df2>(mul_lazy(t.x, s), mul_lazy(t.y, s));
+    p = mk<df2>(add_lazy(e.x, o.x), add_lazy(e.y, o.y));
+    m = mk<df2>(sub_lazy(e.x, o.x), sub_lazy(e.y, o.y));
+}
 template <typename C> __device__ __forceinline__ C bnorm(C a) { return a; }
 template <> __device__ __forceinline__ df2 bnorm(df2 a) { return mk<df2>(renorm(a.x), renorm(a.y)); }
 // The pointwise and spectral stages use the same unrenormalised arithmetic for
@@ -130,26 +154,24 @@ template <int DIR, typename C> __device__ __forceinline__ void bfly8(C *v)
     bfly4<DIR>(v[0], v[2], v[4], v[6]);
     bfly4<DIR>(v[1], v[3], v[5], v[7]);
     const R s = (R)0.70710678118654752440;
-    // x W8 and x W8^3 with W8 = s (1 + DIR i): two adds and two scalings each
+    // x W8 and x W8^3 with W8 = s (1 + DIR i): two adds, the scaling with the next sums
     const C a = v[3], b = v[7];
     C o1, o3;
     if (DIR < 0) {
-        o1 = mk<C>(rmul(radd(a.x, a.y), s), rmul(rsub(a.y, a.x), s));
-        o3 = mk<C>(rmul(rsub(b.y, b.x), s), -rmul(radd(b.x, b.y), s));
+        o1 = mk<C>(radd(a.x, a.y), rsub(a.y, a.x));
+        o3 = mk<C>(rsub(b.y, b.x), -radd(b.x, b.y));
     } else {
-        o1 = mk<C>(rmul(rsub(a.x, a.y), s), rmul(radd(a.x, a.y), s));
-        o3 = mk<C>(-rmul(radd(b.x, b.y), s), rmul(rsub(b.x, b.y), s));
+        o1 = mk<C>(rsub(a.x, a.y), radd(a.x, a.y));
+        o3 = mk<C>(-radd(b.x, b.y), rsub(b.x, b.y));
     }
     C o2 = rot<DIR>(v[5]);
     C e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
     v[0] = badd(e0, o0);
     v[4] = bsub(e0, o0);
-    v[1] = badd(e1, o1);
-    v[5] = bsub(e1, o1);
+    bscaled(e1, o1, s, v[1], v[5]);
     v[2] = badd(e2, o2);
     v[6] = bsub(e2, o2);
-    v[3] = badd(e3, o3);
-    v[7] = bsub(e3, o3);
+    bscaled(e3, o3, s, v[3], v[7]);
 }
 
 // Shared-memory skew: element n of a sequence is stored at n + n/8, which spreads

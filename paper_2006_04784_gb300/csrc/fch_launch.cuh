@@ -101,12 +101,15 @@ template <int M> cudaError_t launch_col_t(const fch_kparams &kp, cudaStream_t s)
     return cudaErrorInvalidValue;
 }
 
-// whether a launch is a column pass of a single-precision plan at N = 1024: TMA-staged, or,
-// for half spectra off the bulk copies' alignment, the generic kernel, which computes the
-// same bit for bit
-template <typename T> bool plan_cols_1024(const fch_kparams &kp)
+// whether a launch takes the TMA-staged columns (half spectra off the bulk copies' alignment
+// take the kernel built for the size, which computes the same bit for bit)
+template <typename T> bool cols_staged(int mode, const fch_kparams &kp)
 {
-    return sizeof(T) == 4 && kp.err && kp.N == 1024;
+    if constexpr (sizeof(T) == 4) {
+        return (mode == CM_FWD_STORE && col_t_applies<CM_FWD_STORE>(kp)) ||
+               (mode == CM_INV_LOAD && col_t_applies<CM_INV_LOAD>(kp));
+    }
+    return false;
 }
 
 template <typename T, int M> cudaError_t launch_col(const fch_kparams &kp, cudaStream_t s)
@@ -168,7 +171,7 @@ template <typename T, int M> cudaError_t launch_row(const fch_kparams &kp, cudaS
 #ifndef FCH_NO_COL
 cudaError_t FCH_CAT(fch_launch_col_, FCH_SUFFIX)(int mode, const fch_kparams &kp, cudaStream_t s)
 {
-    if (reg_applies<FCH_T>(kp, kp.tile_col) && !plan_cols_1024<FCH_T>(kp)) {
+    if (reg_applies<FCH_T>(kp, kp.tile_col) && !cols_staged<FCH_T>(mode, kp)) {
         switch (kp.logN) {
         case 6: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 6)(mode, kp, s);
         case 7: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 7)(mode, kp, s);

@@ -55,7 +55,7 @@ template <typename T, int LOGN> struct RegCfg {
     // rows: whole warps
     static constexpr int rpb = tps >= 32 ? 1 : 32 / tps;
     static constexpr int row_threads = rpb * tps;
-    static constexpr int row_minb = LOGN == 10 ? (dfl ? 4 : single ? 7 : 5) : LOGN == 11 ? 3 : LOGN == 9 ? 4 : 1;
+    static constexpr int row_minb = LOGN == 10 ? (dfl ? 4 : single ? 8 : 5) : LOGN == 11 ? 3 : LOGN == 9 ? 4 : 1;
     // columns: P pairs a block; at N = 1024 in 16-byte elements a cluster of two blocks, one
     // column each (1024 blocks fill the 152 SMs evenly where 512 leave a sixth idle)
     static constexpr bool cl = !single && LOGN == 10;
@@ -95,7 +95,8 @@ template <bool WS> __device__ __forceinline__ void seq_sync()
         __syncthreads();
 }
 
-template <int LOGN, int PPT, int LR, int S, bool DB, bool WS, typename C>
+// (TWG: the twiddles lie in global memory, read through the read-only cache; else shared)
+template <int LOGN, int PPT, int LR, int S, bool DB, bool WS, bool TWG = true, typename C>
 __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__restrict__ tw, int t)
 {
     constexpr int N = 1 << LOGN, tps = N / PPT, LP = PPT == 8 ? 3 : 2;
@@ -111,7 +112,7 @@ __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__re
         if (Ns > 1) {
             const C *tws = tw + (Ns - PPT) + (j & (Ns - 1));
 #pragma unroll
-            for (int r = 1; r < R; r++) x[r] = btw(x[r], ldg(tws + (r - 1) * Ns));
+            for (int r = 1; r < R; r++) x[r] = btw(x[r], TWG ? ldg(tws + (r - 1) * Ns) : tws[(r - 1) * Ns]);
         }
         if (LR == 3)
             bfly8<-1>(x);
