@@ -23,27 +23,35 @@ __device__ __forceinline__ void pdl_begin()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Double-precision reciprocal and sixth root: one step of third order from a
-// single-precision seed (relative error e < 2^-21: the step leaves e^3, below double
-// rounding). The controller is a chain of dependent operations on a slow double pipe, and
-// a third-order step is three of them where two Newton steps are four (the root: nine
-// where two Newton steps and the powers are sixteen).
+// What the control steps cost is double-precision instructions: on this GPU one of them
+// holds an SM's sub-partition for 64 cycles, whatever its lanes do and whether or not it
+// depends on the one before (conversions too; fmin 155, a division 365, a square root 610:
+// measured). So few of them, spread over warps of different sub-partitions where they are
+// independent, and comparisons on the bits: doubles that are not negative are ordered as
+// their bit patterns are, and so is any number against one that is not. Against chains of
+// one warp with double comparisons and two square roots a check: 24 PSD trials of 256^2 in
+// double-float 2618 -> 2534 us, 32 IMEX trials of 512^2 with the regularised well 1662 ->
+// 1605 us.
+__device__ __forceinline__ long long ord(double a) { return __double_as_longlong(a); }
+__device__ __forceinline__ double pmin(double a, double b) { return ord(a) < ord(b) ? a : b; }
+__device__ __forceinline__ double pmax(double a, double b) { return ord(a) > ord(b) ? a : b; }
+
+// Double-precision reciprocal and x^(-1/6): one step of third order from a single-precision
+// seed (relative error e < 2^-21: the step leaves e^3, below double rounding).
 __device__ inline double rcp_nr(double a)
 {
     const double r = (double)(1.0f / (float)a), e = fma(-a, r, 1.0);
     return fma(r, fma(e, e, e), r); // 1/a = r / (1 - e) = r (1 + e + e^2 + ...)
 }
 
-// x^(1/6) for x in [1e-30, 1e30]: z = x^(-1/6) from a seed, with d = 1 - x z^6 the root is
-// z (1 - d)^(-1/6) = z (1 + d/6 + 7 d^2/72 + ...); then x z^5
-__device__ inline double root6_nr(double x)
+// x in [1e-30, 1e36]: with a seed z and d = 1 - x z^6 the root is z (1 - d)^(-1/6) =
+// z (1 + d/6 + 7 d^2/72 + ...)
+__device__ inline double rroot6_nr(double x)
 {
     const double z = (double)powf((float)x, -1.0f / 6.0f);
     const double z2 = z * z, z4 = z2 * z2;
     const double d = fma(-x, z4 * z2, 1.0);
-    const double y = fma(z * d, fma(d, 7.0 / 72.0, 1.0 / 6.0), z);
-    const double y2 = y * y;
-    return (x * y) * (y2 * y2);
+    return fma(z * d, fma(d, 7.0 / 72.0, 1.0 / 6.0), z);
 }
 
 // one control operation; returns false when the run stopped (done or failure). The
@@ -55,13 +63,13 @@ __device__ __forceinline__ bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, doub
     if constexpr (OP == OP_SAV_E1) {
         const double e1 = kp.h2 * S0;
         const double v = e1 + kp.D0;
-        if (!isfinite(v) || v <= 0) {
+        if (!isfinite(v) || ord(v) <= 0) {
             c->status = FCH_ENONFINITE;
             c->done = 1;
             return false;
         }
         c->e1 = e1;
-        c->inv_sqrt_e1 = 1.0 / sqrt(v);
+        c->inv_sqrt_e1 = rsqrt(v);
         if (arg0 == 1.0) c->r_n = sqrt(v);
         if (arg0 == 2.0) c->r_m = sqrt(v);
     } else if constexpr (OP == OP_SAV_R) {
@@ -77,14 +85,13 @@ __device__ __forceinline__ bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, doub
         }
         c->r_new = r;
     } else if constexpr (OP == OP_PSD_CHECK) {
-        const double ratio = sqrt(S0) / sqrt(S1); // ||d|| / ||v_{s+1}||, h cancels
+        // ||d|| / ||v_{s+1}|| < i_tol on the squares (h cancels)
         c->psd_iter++;
         c->n_psd_iter++;
-        c->psd_ratio = ratio;
-        if (!isfinite(ratio)) {
+        if (!isfinite(S0) || !isfinite(S1) || !(ord(S1) > 0)) {
             c->status = FCH_ENONFINITE;
             c->done = 1;
-        } else if (S0 < c->itol * c->itol * S1) {
+        } else if (ord(S0) < ord(c->itol * c->itol * S1)) {
             c->psd_conv = 1;
             c->last_psd_iter = c->psd_iter;
         } else if (c->psd_iter >= c->psd_max_iter) {
@@ -95,21 +102,21 @@ __device__ __forceinline__ bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, doub
     } else if constexpr (OP == OP_DECIDE) {
         // Steps 3-4 of the adaptive algorithm, Sec. 3.2, with e^2 = S0/S1:
         // accept iff S0 <= sigma^2 S1 (or k <= k_min);
-        // A_dp = rho_s k (sigma/e)^(1/3) = rho_s k (sigma^2 S1 / S0)^(1/6), e >= 1e-16
+        // A_dp = rho_s k (sigma/e)^(1/3) = rho_s k (S0 / (sigma^2 S1))^(-1/6), e >= 1e-16
         c->n_attempts++;
-        if (!isfinite(S0) || !isfinite(S1) || !(S1 > 0)) {
+        if (!isfinite(S0) || !isfinite(S1) || !(ord(S1) > 0)) {
             c->status = FCH_ENONFINITE;
             c->done = 1;
             return false;
         }
         c->lte_num = S0;
         c->lte_den = S1;
-        const double k1 = c->k1;
-        const double x = fmin(c->sigma2 * S1 * rcp_nr(fmax(S0, 1e-32 * S1)), 1e30);
-        double kn = c->rho_s * k1 * root6_nr(x);
-        if (c->cap) kn = fmin(kn, 2.414213562373095 * k1); // (1 + sqrt 2) k
-        kn = fmax(c->kmin, fmin(kn, c->kmax));
-        if (S0 <= c->sigma2 * S1 || k1 <= c->kmin) {
+        const double k1 = c->k1, m = c->sigma2 * S1;
+        const double x = pmin(pmax(pmax(S0, 1e-32 * S1) * rcp_nr(pmax(m, 1e-36)), 1e-30), 1e36);
+        double kn = c->rho_s * k1 * rroot6_nr(x);
+        if (c->cap) kn = pmin(kn, 2.414213562373095 * k1); // (1 + sqrt 2) k
+        kn = pmax(c->kmin, pmin(kn, c->kmax));
+        if (ord(S0) <= ord(m) || ord(k1) <= ord(c->kmin)) {
             const int un = c->iu_n, um = c->iu_m, fn = c->if_n, fm = c->if_m;
             c->iu_m = un;
             c->iu_n = c->iu_new;
@@ -152,67 +159,74 @@ __device__ __forceinline__ bool ctrl_op(fch_ctrl *c, const fch_kparams &kp, doub
     return !c->done;
 }
 
-// The set-up of a trial of size arg0 (fixed step) or, where arg0 <= 0, of the next adaptive
-// trial: by one warp. Lane 0 has run whatever came before; the lanes compute the same
-// coefficients, and ten of them look the PSD search step up at once.
-__device__ __forceinline__ void ctrl_init_trial(fch_ctrl *c, double arg0, int lane)
+// The size of the next trial: arg0 (fixed step), or the controller's proposal clipped so
+// that the run ends exactly at t_final; 0 where it has ended (done is set).
+__device__ __forceinline__ double ctrl_next_size(fch_ctrl *c, double arg0)
 {
-    double k1;
-    if (arg0 > 0) {
-        k1 = arg0; // fixed step
-    } else {
-        const double rem = c->t_final - c->t;
-        if (rem <= 1e-12 * fmax(1.0, fabs(c->t_final))) {
-            __syncwarp();
-            c->done = 1;
-            return;
-        }
-        k1 = fmin(c->ktrial, rem); // the run ends exactly at t_final
+    if (arg0 > 0) return arg0;
+    const double rem = c->t_final - c->t;
+    if (ord(rem) <= ord(1e-12 * pmax(1.0, fabs(c->t_final)))) {
+        c->done = 1;
+        return 0.0;
     }
+    return pmin(c->ktrial, rem);
+}
+
+// The set-up of a trial of size k1, by the first four warps of a block (each on a
+// sub-partition of its own; every thread of the block calls it): eq. (BDF2Coef), the eq.
+// (Predictor) weights and the PSD search step.
+__device__ __forceinline__ void ctrl_init_trial(fch_ctrl *c, double k1, int warp, int lane)
+{
+    __shared__ double iv[5]; // 1/k1, 1/(k1 + kn), 1/kn, gam, k1/6
     const double kn = c->kn;
-    double a, b, cc, g, w1 = c->w1, w2 = c->w2, w3 = c->w3;
-    if (kn <= 0) { // backward-Euler start: k_{n-1} -> infinity in eq. (BDF2Coef)
-        a = rcp_nr(k1);
-        b = -a;
-        cc = 0.0;
-        g = 0.0;
-    } else {
-        // eq. (BDF2Coef) and the eq. (Predictor) weights from three independent
-        // reciprocals (1/(1+gam) = k_n/(k_{n+1}+k_n)), so their latencies overlap
-        const double r1 = rcp_nr(k1), rn = rcp_nr(kn), rs = rcp_nr(k1 + kn);
-        a = r1 + rs;
-        b = -r1 - rn;
-        cc = rn - rs;
-        g = k1 * rn;
-        const double k6 = k1 * (1.0 / 6.0), ig = kn * rs; // 1/(1+g)
-        w1 = k6 * (3.0 + 2.0 * g) * ig;
-        w2 = k6 * (3.0 + g);
-        w3 = -k6 * g * g * ig;
+    const bool start = ord(kn) <= 0; // backward-Euler start: k_{n-1} -> infinity in eq. (BDF2Coef)
+    double v = 0.0;
+    if (warp == 0) {
+        v = rcp_nr(k1);
+        if (lane == 0) iv[0] = v;
+    } else if (warp == 1 && !start) {
+        v = rcp_nr(k1 + kn); // 1/(1+gam) = k_n/(k_{n+1}+k_n)
+        if (lane == 0) iv[1] = v;
+    } else if (warp == 2 && !start) {
+        v = rcp_nr(kn);
+        const double g = k1 * v;
+        if (lane == 0) {
+            iv[2] = v;
+            iv[3] = g;
+        }
+    } else if (warp == 3) {
+        if (lane == 0) iv[4] = k1 * (1.0 / 6.0);
+        // Table SearchSize row, linear in k, clamped (slopes precomputed); ten lanes look it up
+        const unsigned above =
+            __ballot_sync(0xffffffffu, lane < 10 && ord(k1) > ord(c->lam_k[lane < 10 ? lane : 0]));
+        const int j = ord(c->lam_k[0]) < 0 ? -1 : __popc(above) - 1; // last knot below k1
+        if (lane == 0)
+            c->lam = j < 0                           ? c->lam_tab[0]
+                     : ord(k1) >= ord(c->lam_k[9]) ? c->lam_tab[9]
+                                                     : c->lam_tab[j] + (k1 - c->lam_k[j]) * c->lam_slope[j];
     }
-    // PSD search step: Table SearchSize row, linear in k, clamped (slopes precomputed)
-    const unsigned above = __ballot_sync(0xffffffffu, lane < 10 && k1 > c->lam_k[lane < 10 ? lane : 0]);
-    const int j = c->lam_k[0] < 0 ? -1 : __popc(above) - 1; // last knot below k1
-    double lam;
-    if (j < 0)
-        lam = c->lam_tab[0];
-    else if (k1 >= c->lam_k[9])
-        lam = c->lam_tab[9];
-    else
-        lam = c->lam_tab[j] + (k1 - c->lam_k[j]) * c->lam_slope[j];
-    __syncwarp(); // every lane has read the old values
-    if (lane == 0) {
-        c->k1 = k1;
-        c->a = a;
-        c->b = b;
-        c->c = cc;
-        c->gam = g;
-        c->w1 = w1;
-        c->w2 = w2;
-        c->w3 = w3;
-        c->lam = lam;
-        c->psd_conv = 0;
-        c->psd_iter = 0;
+    __syncthreads();
+    if (lane == 0 && warp < 4) {
+        const double r1 = iv[0], rs = iv[1], rn = iv[2], g = iv[3], k6 = iv[4];
+        if (warp == 0) {
+            c->k1 = k1;
+            c->psd_conv = 0;
+            c->psd_iter = 0;
+            c->a = start ? r1 : r1 + rs;
+            c->c = start ? 0.0 : rn - rs;
+            if (!start) c->w2 = k6 * (3.0 + g);
+        } else if (warp == 1) {
+            c->gam = start ? 0.0 : g;
+            c->b = start ? -r1 : -r1 - rn;
+        } else if (!start) {
+            const double ig = kn * rs; // 1/(1+g)
+            if (warp == 2)
+                c->w1 = k6 * (3.0 + 2.0 * g) * ig;
+            else
+                c->w3 = -k6 * g * g * ig;
+        }
     }
+    __syncthreads();
 }
 
 // Float, double and double-float mirrors of the per-trial coefficients read by
@@ -241,25 +255,27 @@ template <int OP> constexpr int ctrl_slots()
     return OP == OP_DECIDE_INIT || OP == OP_SAV_R || OP == OP_PSD_CHECK ? 2 : OP == OP_SAV_E1 || OP == OP_ENERGY ? 1 : 0;
 }
 
-// The whole control step by one block (any multiple of 32 threads up to 1024): the control
-// block is staged through shared memory with coalesced copies, the first na partials of
-// the slots the operation reads are summed in a fixed order, warp 0 runs the operation, and
-// the block writes the control block back. What it costs is double-precision instructions
-// (one warp instruction holds the pipe 16 cycles whatever its lanes do) and their chains:
-// both slots are reduced in the two halves of a warp at once, and the warp sums by a second
-// shuffle tree.
+// The whole control step by one block (any multiple of 32 threads up to 1024; the set-up of
+// a trial, 128 or more): the control block is staged through shared memory with coalesced
+// copies, the first na partials of the slots the operation reads are summed in a fixed
+// order, warp 0 runs the operation, and the block writes the control block back. Both slots
+// are reduced in the two halves of a warp at once, by the warps that hold partials.
 template <int OP> __device__ __forceinline__ void ctrl_block(const fch_kparams &kp, int na, double arg0)
 {
     constexpr int slots = ctrl_slots<OP>();
+    constexpr bool init = OP == OP_INIT_TRIAL || OP == OP_DECIDE_INIT || OP == OP_ACCEPT_INIT;
     __shared__ double sh[2][32];
     __shared__ fch_ctrl cs;
+    __shared__ double k1s;
     const int nw = (int)(sizeof(fch_ctrl) / 8);
     const int nthr = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < nw; i += nthr) ((long long *)&cs)[i] = ((const long long *)kp.ctrl)[i];
     // the partial sums load while the control block arrives (discarded if it says done)
-    double s0 = 0, s1 = 0;
-    if (slots > 0) {
-        for (int i = threadIdx.x; i < na; i += 4 * nthr) {
+    const int wact = min((na + 31) >> 5, nthr >> 5); // warps with partials
+    if (slots > 0 && warp < wact) {
+        const int i0 = threadIdx.x;
+        double s0 = i0 < na ? kp.part[i0] : 0.0, s1 = slots > 1 && i0 < na ? kp.part[FCH_MAXBLK + i0] : 0.0;
+        for (int i = i0 + nthr; i < na; i += 4 * nthr) {
             double v0[4], v1[4];
 #pragma unroll
             for (int k = 0; k < 4; k++) {
@@ -286,24 +302,29 @@ template <int OP> __device__ __forceinline__ void ctrl_block(const fch_kparams &
     if (warp == 0) {
         double S0 = 0, S1 = 0;
         if (slots > 0) {
-            const int w = nthr >> 5, l = lane & 15, h = lane >> 4;
-            double v = l < w ? sh[h][l] : 0.0;
-            if (w > 16) v += l + 16 < w ? sh[h][l + 16] : 0.0;
-            for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, 16);
+            const int l = lane & 15, h = lane >> 4;
+            double v = l < wact ? sh[h][l] : 0.0;
+            if (wact > 16) v += l + 16 < wact ? sh[h][l + 16] : 0.0;
+            for (int o = 8; o > 0; o >>= 1)
+                if (o < wact) v += __shfl_down_sync(0xffffffffu, v, o, 16);
             S0 = __shfl_sync(0xffffffffu, v, 0);
             S1 = __shfl_sync(0xffffffffu, v, 16);
         }
         // the combined operations: the decision (adaptive) or the acceptance of a fixed
         // step, then the set-up of the next trial (adaptive: -1; fixed: arg0 = dt)
         constexpr int FIRST = OP == OP_DECIDE_INIT ? OP_DECIDE : OP == OP_ACCEPT_INIT ? OP_ACCEPT : OP;
-        bool go = true;
-        if (FIRST != OP_INIT_TRIAL) {
-            if (lane == 0) go = ctrl_op<FIRST>(&cs, kp, S0, S1, OP == OP_ACCEPT_INIT ? 0.0 : arg0);
-            go = __shfl_sync(0xffffffffu, go, 0);
+        if (lane == 0) {
+            bool go = true;
+            if (FIRST != OP_INIT_TRIAL) go = ctrl_op<FIRST>(&cs, kp, S0, S1, OP == OP_ACCEPT_INIT ? 0.0 : arg0);
+            if (init) k1s = go ? ctrl_next_size(&cs, OP == OP_DECIDE_INIT ? -1.0 : arg0) : 0.0;
         }
-        __syncwarp();
-        if ((OP == OP_INIT_TRIAL || OP == OP_DECIDE_INIT || OP == OP_ACCEPT_INIT) && go)
-            ctrl_init_trial(&cs, OP == OP_DECIDE_INIT ? -1.0 : arg0, lane);
+    }
+    if (init) {
+        __syncthreads();
+        const double k1 = k1s;
+        if (ord(k1) > 0) ctrl_init_trial(&cs, k1, warp, lane);
+    }
+    if (warp == 0) {
         __syncwarp();
         sync_coef_lanes(&cs, lane);
     }

@@ -44,7 +44,7 @@ struct fch_ctrl {
     double lam, itol;               // PSD search step and stopping tolerance
     double r_n, r_m, r_new;         // SAV auxiliary variable history
     double e1, inv_sqrt_e1;         // SAV E1(u*) and 1/sqrt(E1 + D0)
-    double e_last, psd_ratio, energy;
+    double e_last, energy;
     double kmin, kmax, rho_s;
     int cap;                        // zero-stability cap on A_dp
     int iu_n, iu_m, iu_new;         // which of the three state spectra hold u^n, u^{n-1}, trial
