@@ -36,7 +36,7 @@ inline cudaError_t set_smem(pass_fn f, int bytes, int floor_bytes, int &cur)
 
 // the passes built for a grid size (fch_reg.cu): tile 0, N = 64 ... 2048, where the
 // twiddle tables are at hand (the radix-4 one: contexts and plans, not fch_fft_r2c_noalloc,
-// whose single-precision passes need the radix-8 one only)
+// whose single-precision transforms need the radix-8 one only)
 template <typename T> bool reg_applies(const fch_kparams &kp, int tile)
 {
     return tile == 0 && kp.logN >= 6 && kp.logN <= 11 && (sizeof(T) == 4 || kp.tw4);

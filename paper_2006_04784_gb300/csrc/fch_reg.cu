@@ -24,7 +24,7 @@ inline cudaError_t launch_reg(pass_fn f, int blocks, int threads, int smem, bool
 
 template <typename T, int M, int LOGN> cudaError_t col(const fch_kparams &kp, cudaStream_t s)
 {
-    typedef fch::RegCfg<T, LOGN> G;
+    typedef fch::RegCfg<T, LOGN, fch::col_xf(M)> G;
     static bool set = false;
     pass_fn f;
     if constexpr (G::cl)
@@ -36,7 +36,7 @@ template <typename T, int M, int LOGN> cudaError_t col(const fch_kparams &kp, cu
 
 template <typename T, int M, int LOGN> cudaError_t row(const fch_kparams &kp, cudaStream_t s)
 {
-    typedef fch::RegCfg<T, LOGN> G;
+    typedef fch::RegCfg<T, LOGN, fch::row_xf(M)> G;
     static bool set = false;
     return launch_reg(fch::row_pass_r<T, M, LOGN>, G::N / G::rpb, G::row_threads, G::row_smem, set, s, kp);
 }

@@ -34,23 +34,42 @@ __device__ __forceinline__ double flip(double x, unsigned m)
 }
 __device__ __forceinline__ df flip(df x, unsigned m) { return df(flip(x.hi, m), flip(x.lo, m)); }
 
+// the passes standalone transforms run
+constexpr bool row_xf(int mode) { return mode == RM_R2C_LOAD || mode == RM_C2R_STORE; }
+constexpr bool col_xf(int mode) { return mode == CM_FWD_STORE || mode == CM_INV_LOAD; }
+
 // What a pass is built for, by element (16 bytes: double and double-float; 8: single) and
-// size. Points a thread: four (radix-4 stages) where a pass is a few warps an SM and its
-// dependent chain is the time, up to 256^2 and in double-float to 1024^2; eight (radix-8
-// stages, fewer exchanges and twiddle products) where the FP64 pipe is the bound or the
-// blocks would get too large. Blocks an SM: enough registers that nothing spills; at 1024^2
-// four blocks of 256 threads (two waves whose loads, transforms and stores overlap) beat
-// seven of 128 in one wave, whose phases run in step.
+// size. Points a thread: two (radix-2 stages) where a pass is a few warps on the 608
+// sub-partitions and the time is the dependent chain of one of them, in double to 128^2 and
+// in the others to 256^2; four (radix-4) in double at 256^2, in double-float to 1024^2 and
+// in single at 512^2; eight (radix-8 stages, fewer exchanges and twiddle products) where
+// the pipes are the bound or the blocks would get too large. Two points cost more
+// operations (24 a point of a 128-point transform, 22 at four) and twice the exchanges, but
+// halve the instructions of a warp, and a double-precision one holds its sub-partition for
+// 64 cycles whatever its lanes do. Blocks an SM: enough registers that nothing spills; at
+// 1024^2 four blocks of 256 threads (two waves whose loads, transforms and stores overlap)
+// beat seven of 128 in one wave, whose phases run in step.
 // Adaptive IMEX passes, GB300, us a run of the case: double-float 1024^2, 48 trials: 8
 // points x 7 blocks 6346, x 5 6313, 4 points x 3 6484, x 4 6198, two buffers 6133;
-// 2048^2, 32 trials: 8 points 14.4k, 4 points 17.0k; 256^2, 64 trials: 4 points 2240, 8
-// points 3130; 512^2 (q > 0), 32 trials: 2430, 2830. Double 1024^2, 12 trials: 8 points x 5
-// 7426, x 7 7568, 4 points x 4 7632; 512^2 SAV, 32 trials: 8 points 6424, 4 points 6672;
-// 128^2, 100 fixed steps: 4 points 3350, 8 points 5430.
-template <typename T, int LOGN> struct RegCfg {
+// 2048^2, 32 trials: 8 points 14.4k, 4 points 17.0k; 512^2, 24 trials: 4 points 1125, 2
+// points 1280; 256^2, 64 trials: 4 points 1984, 2 points 1726, PSD 2573, 2345 (in a sweep
+// with 512^2 and 1024^2 grids, which fill the GPU, 2 points lose 1.7 %: 8073, 8210; six 256^2
+// grids alone gain: 1844, 1578); 128^2, 24 trials: 749, 602, PSD 2101, 1718. Double 1024^2, 12 trials: 8 points x 5 7426, x 7 7568, 4 points x 4 7632;
+// 512^2 SAV, 32 trials: 8 points 6424, 4 points 6672; 256^2 PSD, 24 trials: 4 points 4703, 2
+// points 4826; 128^2, 100 fixed steps: 8 points 5430, 4 points 2946 (with what came
+// between), 2 points 2111. Single, 50 fixed IMEX steps: 128^2 8 points 767, 4 points 606, 2
+// points 557; 256^2 760, 664, 658; 512^2 SAV, 24 steps: 761, 695, 747.
+// Transforms on their own (XF) run many fields at once: eight points in single at all sizes
+// (33 fields of 256^2 there and back 31.6 us, 4 points 32.6, 2 points 43.1); in double as
+// the steps (128^2, one pair 19.7 -> 14.6 us at 2 points, 8 pairs 33.3 -> 35.1, 16 pairs and
+// an odd field 77.8 -> 73.8). One choice for every batch: a field's result does not depend
+// on how many are transformed with it.
+template <typename T, int LOGN, bool XF> struct RegCfg {
     static constexpr bool single = sizeof(T) == 4, dfl = std::is_same<T, df>::value;
     static constexpr int N = 1 << LOGN;
-    static constexpr int ppt = !single && LOGN <= (dfl ? 10 : 8) ? 4 : 8;
+    static constexpr int ppt = single ? (XF ? 8 : LOGN <= 8 ? 2 : LOGN == 9 ? 4 : 8)
+                               : dfl  ? (LOGN <= 8 ? 2 : LOGN <= 10 ? 4 : 8)
+                                      : (LOGN <= 7 ? 2 : LOGN <= 8 ? 4 : 8);
     static constexpr int tps = N / ppt;
     // rows: whole warps
     static constexpr int rpb = tps >= 32 ? 1 : 32 / tps;
@@ -95,11 +114,30 @@ template <bool WS> __device__ __forceinline__ void seq_sync()
         __syncthreads();
 }
 
+// The stage of two points a thread and sub-length Ns = 2^S: its factor exp(-2 pi i j / 2 Ns),
+// j < Ns, from the table of radix-4 stages (entry Ns' - 4 + (r - 1) Ns' + j =
+// exp(-2 pi i r j / 4 Ns')): where Ns is a power of four it is r = 2 of Ns (r = 1 where the
+// table ends in a radix-2 stage), else r = 1 of Ns / 2 and, in the upper half, a turn by -i.
+template <int LOGN, int S, typename C> __device__ __forceinline__ C reg_twist2(C x, const C *__restrict__ tw, int t)
+{
+    constexpr int Ns = 1 << S;
+    if (S == 0) return x;
+    if (S % 2 == 0) return btw(x, ldg(tw + Ns - 4 + (S + 1 == LOGN ? 0 : Ns) + (t & (Ns - 1))));
+    constexpr int Nh = Ns >> 1;
+    if (S > 1) x = btw(x, ldg(tw + Nh - 4 + (t & (Nh - 1))));
+    return t & Nh ? mk<C>(x.y, flip(x.x, 0x80000000u)) : x;
+}
+
+// (Double-float is renormalised after the fourth radix-2 stage too, not only at the end: the
+// rounding of twice as many stages would otherwise exceed that of radix 4. F(u) of a bilayer
+// at 64^2, q = 0.5, against double: radix 4 9.5e-12, radix 2 without 1.04e-11, with 8.1e-12;
+// after every second stage 7.2e-12, after every one 6.1e-12, but 24 PSD trials of 256^2 take
+// 2345, 2394 and 2400 us.)
 // (TWG: the twiddles lie in global memory, read through the read-only cache; else shared)
 template <int LOGN, int PPT, int LR, int S, bool DB, bool WS, bool TWG = true, typename C>
 __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__restrict__ tw, int t)
 {
-    constexpr int N = 1 << LOGN, tps = N / PPT, LP = PPT == 8 ? 3 : 2;
+    constexpr int N = 1 << LOGN, tps = N / PPT, LP = PPT == 8 ? 3 : PPT == 4 ? 2 : 1;
     constexpr int R = 1 << LR, NB = PPT / R;
     constexpr int lNs = S * LP, Ns = 1 << lNs;
     constexpr bool last = (Ns << LR) == N;
@@ -109,7 +147,9 @@ __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__re
         C x[R];
 #pragma unroll
         for (int r = 0; r < R; r++) x[r] = v[b + NB * r];
-        if (Ns > 1) {
+        if (PPT == 2) {
+            x[1] = reg_twist2<LOGN, S>(x[1], tw, j);
+        } else if (Ns > 1) {
             const C *tws = tw + (Ns - PPT) + (j & (Ns - 1));
 #pragma unroll
             for (int r = 1; r < R; r++) x[r] = btw(x[r], TWG ? ldg(tws + (r - 1) * Ns) : tws[(r - 1) * Ns]);
@@ -121,7 +161,7 @@ __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__re
         else
             bfly2<-1>(x[0], x[1]);
 #pragma unroll
-        for (int r = 0; r < R; r++) v[b + NB * r] = last ? bnorm(x[r]) : x[r];
+        for (int r = 0; r < R; r++) v[b + NB * r] = last || (PPT == 2 && S == 3) ? bnorm(x[r]) : x[r];
     }
     if (!last) {
         if (!DB) seq_sync<WS>();
@@ -146,13 +186,16 @@ __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__re
 template <int LOGN, int PPT, bool DB, bool WS, typename C>
 __device__ __forceinline__ void fft_reg(C *v, C *&buf, C *&buf2, const C *__restrict__ tw, int t)
 {
-    constexpr int LP = PPT == 8 ? 3 : 2, NF = LOGN / LP, REM = LOGN % LP;
-    static_assert(NF >= 1 && NF <= 5, "two to six stages");
+    constexpr int LP = PPT == 8 ? 3 : PPT == 4 ? 2 : 1, NF = LOGN / LP, REM = LOGN % LP;
+    static_assert(NF >= 1 && NF <= 8, "two to eight stages");
     reg_stage<LOGN, PPT, LP, 0, DB, WS>(v, buf, buf2, tw, t);
     if constexpr (NF > 1) reg_stage<LOGN, PPT, LP, 1, DB, WS>(v, buf, buf2, tw, t);
     if constexpr (NF > 2) reg_stage<LOGN, PPT, LP, 2, DB, WS>(v, buf, buf2, tw, t);
     if constexpr (NF > 3) reg_stage<LOGN, PPT, LP, 3, DB, WS>(v, buf, buf2, tw, t);
     if constexpr (NF > 4) reg_stage<LOGN, PPT, LP, 4, DB, WS>(v, buf, buf2, tw, t);
+    if constexpr (NF > 5) reg_stage<LOGN, PPT, LP, 5, DB, WS>(v, buf, buf2, tw, t);
+    if constexpr (NF > 6) reg_stage<LOGN, PPT, LP, 6, DB, WS>(v, buf, buf2, tw, t);
+    if constexpr (NF > 7) reg_stage<LOGN, PPT, LP, 7, DB, WS>(v, buf, buf2, tw, t);
     if constexpr (REM > 0) reg_stage<LOGN, PPT, REM, NF, DB, WS>(v, buf, buf2, tw, t);
 }
 
@@ -169,11 +212,11 @@ __device__ __forceinline__ int pair_slot(int e, int N)
 
 // ---------------------------------------------------------------------------
 template <typename T, int MODE, int LOGN>
-__global__ void __launch_bounds__((RegCfg<T, LOGN>::row_threads), (RegCfg<T, LOGN>::row_minb))
+__global__ void __launch_bounds__((RegCfg<T, LOGN, row_xf(MODE)>::row_threads), (RegCfg<T, LOGN, row_xf(MODE)>::row_minb))
 row_pass_r(const fch_kparams kp)
 {
     typedef typename CT<T>::t C;
-    typedef RegCfg<T, LOGN> G;
+    typedef RegCfg<T, LOGN, row_xf(MODE)> G;
     constexpr int N = G::N, PPT = G::ppt, TPS = G::tps;
     constexpr bool WS = TPS <= 32;
     constexpr bool INV = MODE != RM_R2C_LOAD && MODE != RM_NIMEX_DIRECT && MODE != RM_SAV_DIRECT;
@@ -230,7 +273,7 @@ row_pass_r(const fch_kparams kp)
     constexpr bool has_red = MODE == RM_SAV || MODE == RM_SAV_DIRECT || MODE == RM_ENERGY;
     // the pointwise stage on the natural slots (and its block sums)
     auto pointwise_stage = [&]() {
-        if (PT && PPT == 4) {
+        if (PT && PPT <= 4) {
 #pragma unroll
             for (int m = 0; m < PPT; m++) v[m] = pointwise_elem<T, MODE>(kp, K, v[m], red);
         } else if (PT) {
@@ -301,7 +344,7 @@ __device__ __forceinline__ void col_body_r(const fch_kparams &kp)
 {
     typedef typename CT<T>::t C;
     typedef ColTraits<MODE> TR;
-    typedef RegCfg<T, LOGN> G;
+    typedef RegCfg<T, LOGN, col_xf(MODE)> G;
     namespace cg = cooperative_groups;
     constexpr int N = G::N, PPT = G::ppt, TPS = G::tps, H = PPT / 2;
     constexpr bool CL = G::cl, WS = G::col_threads <= 32;
@@ -461,7 +504,7 @@ __device__ __forceinline__ void col_body_r(const fch_kparams &kp)
 }
 
 template <typename T, int MODE, int LOGN>
-__global__ void __launch_bounds__((RegCfg<T, LOGN>::col_threads), (RegCfg<T, LOGN>::col_minb))
+__global__ void __launch_bounds__((RegCfg<T, LOGN, col_xf(MODE)>::col_threads), (RegCfg<T, LOGN, col_xf(MODE)>::col_minb))
 col_pass_r(const fch_kparams kp)
 {
     col_body_r<T, MODE, LOGN>(kp);
@@ -470,7 +513,7 @@ col_pass_r(const fch_kparams kp)
 // the same as clusters of two blocks, one column of a pair each
 template <typename T, int MODE, int LOGN>
 __global__ void __cluster_dims__(2, 1, 1)
-    __launch_bounds__((RegCfg<T, LOGN>::col_threads), (RegCfg<T, LOGN>::col_minb))
+    __launch_bounds__((RegCfg<T, LOGN, col_xf(MODE)>::col_threads), (RegCfg<T, LOGN, col_xf(MODE)>::col_minb))
 col_pass_rcl(const fch_kparams kp)
 {
     col_body_r<T, MODE, LOGN>(kp);

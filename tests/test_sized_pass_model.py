@@ -77,3 +77,33 @@ def test_column_pairs_with_a_conjugated_column(n):
     # the pair-layout slot of a natural index is a bijection
     slot = [2 * e if e < n // 2 else 1 if e == n // 2 else 2 * (n - e) + 1 for e in range(n)]
     assert sorted(slot) == list(range(n))
+
+
+@pytest.mark.parametrize("logn", [6, 7, 8])
+def test_two_point_stages_from_the_radix4_table(logn):
+    # radix-2 stages on two points a thread, their factors taken from the table of radix-4
+    # stages (one of radix 2 at its end where log2 n is odd), against numpy's transform
+    from paper_2006_04784_gb300 import fch
+    n = 1 << logn
+    tw = fch.stage_twiddles(n, 2)
+    tps = n // 2
+    x = np.random.default_rng(n).standard_normal(2 * n).view(complex)
+    v = np.stack([x[:tps], x[tps:]], axis=1)
+    for s in range(logn):
+        ns = 1 << s
+        buf = np.full(n, np.nan, dtype=complex)
+        for t in range(tps):
+            b = v[t, 1]
+            if s % 2 == 0 and s > 0:
+                b *= tw[ns - 4 + (0 if s + 1 == logn else ns) + (t & (ns - 1))]
+            elif s % 2:
+                nh = ns >> 1
+                if s > 1:
+                    b *= tw[nh - 4 + (t & (nh - 1))]
+                if t & nh:
+                    b *= -1j
+            d = ((t >> s) << (s + 1)) + (t & (ns - 1))
+            buf[d], buf[d + ns] = v[t, 0] + b, v[t, 0] - b
+        v = np.stack([buf[:tps], buf[tps:]], axis=1)
+    out = np.concatenate([v[:, 0], v[:, 1]])
+    assert np.abs(out - np.fft.fft(x)).max() < 1e-13 * n
