@@ -36,8 +36,8 @@ fch_geom fch_geometry(int N, int prec)
         g.col_blocks = N;
         g.col_smem = SL * csz;
     }
-    // rows per block: one at N = 1024 (the compile-time kernel's 128 threads), else
-    // 256 threads' worth; the row pass keeps its twiddles in global memory
+    // rows per block of the generic kernel: one at N = 1024 (128 threads), else 256
+    // threads' worth; the row pass keeps its twiddles in global memory
     const int tps = N / 8;
     int rpb = N == 1024 ? 1 : 256 / tps;
     if (rpb < 1) rpb = 1;
@@ -62,7 +62,7 @@ fch_geom fch_geometry_tiled(int N, int prec, int tile_row, int tile_col)
     fch_geom g = fch_geometry(N, prec);
     const int csz = prec == 1 ? 8 : 16, SL = N + N / 8;
     if ((tile_col == -1 || tile_col == -2) && N == 1024) {
-        // without clusters: the compile-time kernel (-1) with 1 (16-byte) or 2 (8-byte)
+        // without clusters: the generic kernel (-1) with 1 (16-byte) or 2 (8-byte)
         // column pairs per block, or the warp-level kernel (-2, single precision) with
         // two pairs per block
         const int P = csz == 16 ? 1 : 2;
@@ -688,7 +688,7 @@ extern "C" fch_status fch_create(const fch_grid *g, const fch_params *p, void *s
         ctx->own_stream = true;
     }
     int trow = p->tile_row, tcol = p->tile_col;
-    // fft_path 2 asks for the warp-level passes where they exist (single precision, 1024^2)
+    // fft_path 2 asks for the warp-level column pass where it exists (single precision, 1024^2)
     if (p->fft_path == 2 && p->prec == FCH_MIXED && g->n == 1024 && tcol == 0) tcol = -2;
     if (e == cudaSuccess && p->autotune) {
         fch_tile t;
@@ -2074,9 +2074,9 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
                : prec == FCH_FP32X2 ? fch_launch_row_dfl(RM_R2C_LOAD, k, s)
                                     : fch_launch_row_f64(RM_R2C_LOAD, k, s);
     };
-    // candidates: the default tiles (timed first), the shared-memory kernels where the
-    // default is the warp-level path, and the generic kernel at 1..16 rows (column
-    // pairs) a block; another tile replaces the default only if 3 % faster
+    // candidates: the default tiles (timed first: the passes built for the size), at 1024^2
+    // the generic kernel at its default geometry and the warp-level columns, and the generic
+    // kernel at 1..16 rows (column pairs) a block; another tile replaces the default only if 3 % faster
     fch_tile best;
     memset(&best, 0, sizeof(best));
     const int reps = n >= 1024 ? 10 : 20;

@@ -74,15 +74,15 @@ struct fch_kparams {
     void *Rs[3];                    // real-space (u, Lap u) of the three state slots, N x N complex
     void *Z;                        // N x N complex pair-layout work array
     const void *tw;                 // per-stage Stockham twiddles of radix-8 stages (see fft_smem)
-    const void *tw4;                // the same for radix-4 stages (contexts; null in plans)
+    const void *tw4;                // the same for radix-4 stages (contexts and plans; null in fch_fft_r2c_noalloc)
     const void *tw2;                // N = 1024 warp transform: [k2][n1] exp(-2 pi i n1 k2 / 1024), float
     double *part;                   // [FCH_NRED][FCH_MAXBLK] per-block partial sums
     fch_ctrl *ctrl;
     unsigned long long *nfft;       // 2D real-transform counter (may be null)
     const void *in0, *in1;          // explicit inputs (standalone transforms, device fields)
     void *out0, *out1;              // explicit outputs
-    int tile_row, tile_col;         // pass tiles: 0 default; -1 shared-memory kernel without the
-                                    // warp-level path; > 0 generic kernel with that many rows
+    int tile_row, tile_col;         // pass tiles: 0 the passes built for the size; -1 generic
+                                    // kernel at its default geometry; > 0 with that many rows
                                     // (column pairs) per block
     int npairs;                     // standalone transforms: field pairs of one launch (grid y; 0 = 1)
     long long pstride_in, pstride_out; // bytes from one pair's in0/in1 (out0/out1) to the next's

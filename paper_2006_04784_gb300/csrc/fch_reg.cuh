@@ -54,10 +54,10 @@ constexpr bool col_xf(int mode) { return mode == CM_FWD_STORE || mode == CM_INV_
 // 2048^2, 32 trials: 8 points 14.4k, 4 points 17.0k; 512^2, 24 trials: 4 points 1125, 2
 // points 1280; 256^2, 64 trials: 4 points 1984, 2 points 1726, PSD 2573, 2345 (in a sweep
 // with 512^2 and 1024^2 grids, which fill the GPU, 2 points lose 1.7 %: 8073, 8210; six 256^2
-// grids alone gain: 1844, 1578); 128^2, 24 trials: 749, 602, PSD 2101, 1718. Double 1024^2, 12 trials: 8 points x 5 7426, x 7 7568, 4 points x 4 7632;
-// 512^2 SAV, 32 trials: 8 points 6424, 4 points 6672; 256^2 PSD, 24 trials: 4 points 4703, 2
-// points 4826; 128^2, 100 fixed steps: 8 points 5430, 4 points 2946 (with what came
-// between), 2 points 2111. Single, 50 fixed IMEX steps: 128^2 8 points 767, 4 points 606, 2
+// grids alone gain: 1844, 1578); 128^2, 24 trials: 749, 602, PSD 2101, 1718. Double
+// 1024^2, 12 trials: 8 points x 5 7426, x 7 7568, 4 points x 4 7632; 512^2 SAV, 32 trials: 8
+// points 6424, 4 points 6672; 256^2 PSD, 24 trials: 4 points 4703, 2 points 4826; 128^2, 100
+// fixed steps: 8 points 5430, 4 points 2946 (with what came between), 2 points 2111. Single, 50 fixed IMEX steps: 128^2 8 points 767, 4 points 606, 2
 // points 557; 256^2 760, 664, 658; 512^2 SAV, 24 steps: 761, 695, 747.
 // Transforms on their own (XF) run many fields at once: eight points in single at all sizes
 // (33 fields of 256^2 there and back 31.6 us, 4 points 32.6, 2 points 43.1); in double as
