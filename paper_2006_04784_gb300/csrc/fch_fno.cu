@@ -1347,6 +1347,7 @@ void free_buffers(fch_fno *f)
     if (f->plan) fch_fft_plan_destroy(f->plan);
     f->plan = nullptr;
     f->B = f->n = 0;
+    f->have_fwd = false;
 }
 
 fch_status ensure_buffers(fch_fno *f, int B, int n)
@@ -1582,11 +1583,12 @@ static fch_status forward_impl(fch_fno *f, int batch, int n, const float *a, flo
         fch_set_thread_error(f->err);
         return FCH_ECUDA;
     }
-    f->a = a;
-    f->have_fwd = true;
     // keep y for the backward pass (the caller owns its array)
     e = cudaMemcpyAsync(f->y, y, (size_t)pts * 4, cudaMemcpyDeviceToDevice, s);
-    return e == cudaSuccess ? FCH_OK : FCH_ECUDA;
+    if (e != cudaSuccess) return FCH_ECUDA;
+    f->a = a;
+    f->have_fwd = true;
+    return FCH_OK;
 }
 
 // tables and work arrays of the truncated-DFT forward pass for (B, n)
@@ -1729,8 +1731,10 @@ extern "C" fch_status fch_fno_forward(fch_fno *f, int batch, int n, const float 
                                  "proj a multiple of 16 and n a multiple of 128");
             return FCH_EINVAL;
         }
+        f->have_fwd = false;
         return forward_tc(f, batch, n, a, y);
     }
+    f->have_fwd = false; // until the pass is enqueued whole: a failed one leaves nothing to go back through
     return f->pbf ? forward_impl(f, batch, n, a, y, (const __nv_bfloat16 *)f->pbf)
                   : forward_impl(f, batch, n, a, y, (const float *)f->params);
 }
