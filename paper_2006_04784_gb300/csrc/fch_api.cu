@@ -728,6 +728,7 @@ extern "C" fch_status fch_create(const fch_grid *g, const fch_params *p, void *s
     for (int i = 0; i < 3 && e == cudaSuccess; i++) e = cudaMemsetAsync(ctx->Rs[i], 0, (size_t)N * N * csz, ctx->stream);
     if (e != cudaSuccess) {
         snprintf(ctx->errbuf, sizeof(ctx->errbuf), "fch_create: %s", cudaGetErrorString(e));
+        cudaGetLastError(); // reported here: the next launch's check does not meet it again
         fch_destroy(ctx);
         return e == cudaErrorMemoryAllocation ? FCH_ENOMEM : FCH_ECUDA;
     }
@@ -1728,6 +1729,7 @@ extern "C" fch_status fch_ensemble_create(int m, const fch_grid *grids, const fc
     if (ce == cudaSuccess) ce = cudaMallocHost((void **)&e->hflags, m * sizeof(int));
     if (ce != cudaSuccess) {
         snprintf(g_plan_err, sizeof(g_plan_err), "fch_ensemble_create: %s", cudaGetErrorString(ce));
+        cudaGetLastError();
         fch_ensemble_destroy(e);
         return ce == cudaErrorMemoryAllocation ? FCH_ENOMEM : FCH_ECUDA;
     }
@@ -2286,6 +2288,7 @@ extern "C" fch_status fch_fft_plan_create(int n, int prec, void *stream, fch_fft
     if (e == cudaSuccess) e = cudaMalloc(&pl->err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(pl->err, 0, sizeof(int), pl->stream);
     if (e != cudaSuccess) {
+        cudaGetLastError();
         fch_fft_plan_destroy(pl);
         return e == cudaErrorMemoryAllocation ? FCH_ENOMEM : FCH_ECUDA;
     }

@@ -1382,6 +1382,7 @@ fch_status ensure_buffers(fch_fno *f, int B, int n)
     if (e == cudaSuccess && !f->modes) e = cudaMemsetAsync(f->Ysp, 0, spec, f->stream);
     if (e != cudaSuccess) {
         snprintf(f->err, sizeof(f->err), "fch_fno: %s", cudaGetErrorString(e));
+        cudaGetLastError(); // reported here: the next launch's check does not meet it again
         free_buffers(f);
         return e == cudaErrorMemoryAllocation ? FCH_ENOMEM : FCH_ECUDA;
     }
@@ -1462,6 +1463,7 @@ extern "C" fch_status fch_fno_create(int width, int layers, int modes, int proj,
     if (e == cudaSuccess) e = cudaMemsetAsync(f->av, 0, f->np * 4, f->stream);
     if (e != cudaSuccess) {
         fch_set_thread_error(cudaGetErrorString(e));
+        cudaGetLastError();
         fch_fno_destroy(f);
         return FCH_ECUDA;
     }
@@ -1620,6 +1622,7 @@ static fch_status ensure_tc(fch_fno *f, int B, int n)
     if (e != cudaSuccess) {
         snprintf(f->err, sizeof(f->err), "fch_fno (truncated DFT): %s", cudaGetErrorString(e));
         fch_set_thread_error(f->err);
+        cudaGetLastError(); // as in ensure_buffers
         return e == cudaErrorMemoryAllocation ? FCH_ENOMEM : FCH_ECUDA;
     }
     f->tc_B = B;
@@ -1704,6 +1707,7 @@ extern "C" fch_status fch_fno_set_bf16(fch_fno *f, int on)
     if (on && !f->pbf) {
         if (cudaMalloc((void **)&f->pbf, f->np * sizeof(__nv_bfloat16)) != cudaSuccess) {
             f->pbf = nullptr;
+            cudaGetLastError();
             return FCH_ENOMEM;
         }
         f->tc = on == 2;

@@ -51,3 +51,21 @@ def test_backward_is_refused_after_a_failed_forward(first):
     assert loss.value == -1.0
     torch.cuda.synchronize()
     net.close()
+
+
+def test_a_failed_forward_leaves_no_error_for_the_next_call():
+    # neither the library's next launch check nor another library's finds the allocation's error
+    net, a, y = _net()
+    net.forward(a, y)
+    ref = y.clone()
+    _fail(net, a, y)
+    net.set_bf16(1)  # launches a kernel and checks
+    net.set_bf16(0)
+    _fail(net, a, y)
+    net.set_params(net.params())
+    net.forward(a, y)
+    assert torch.equal(y, ref)
+    net.backward(ref)
+    _fail(net, a, y)
+    assert float((torch.ones(8, device=DEV) + 1).sum()) == 16.0
+    net.close()
