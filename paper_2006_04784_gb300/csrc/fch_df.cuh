@@ -11,8 +11,8 @@
 // Addition sums the high parts with TwoSum and the low parts with one rounding
 // (error bounded relative to the operands); multiplication adds the cross terms to
 // the exact product of the high parts; division refines a float quotient with two
-// correction terms, the reciprocal takes one Newton step. exp and expm1 (the q > 0 well and the ETD phi
-// functions) are table-driven on the FP32 pipe.
+// correction terms, the reciprocal takes one Newton step. exp and expm1 (the q > 0 well
+// and the ETD phi functions) are table-driven on the FP32 pipe.
 // Compile without fast-math: the transformations rely on IEEE rounding of each step.
 #pragma once
 #include <math.h>
@@ -242,24 +242,36 @@ __device__ __forceinline__ df copysign(df a, df s)
 // exp and expm1 on the FP32 pipe, table-driven (P. T. P. Tang, "Table-driven implementation
 // of the exponential function in IEEE floating-point arithmetic", 1989): a = n ln2/32 + r,
 // |r| <= ln2/64; e^a = 2^(n/32) (1 + p), p = e^r - 1 by the series (terms from r^4/4! on in
-// single precision: they are below 2^-30), 2^(n/32) = 2^e T_j from the table. ln2/32 is split
-// in three floats: n L1 cancels against a.hi without rounding (fused multiply-add), n L2 is
-// an exact product. Relative error below 2^-47 (the format's own rounding is 2^-48); the
-// double pipe's exp costs some twenty double operations a point, 64 FP32 issue slots each.
-__device__ const float2 kExp2Tab[32] = { // 2^(j/32) = hi + lo
-    {0x1.0p+0f, 0x0.0p+0f}, {0x1.059b0ep+0f, -0x1.9d4f52p-25f}, {0x1.0b5586p+0f, 0x1.9f3122p-25f}, {0x1.11301ep+0f, -0x1.fdb496p-25f},
-    {0x1.172b84p+0f, -0x1.c15742p-27f}, {0x1.1d4874p+0f, -0x1.d2e8cap-25f}, {0x1.2387a6p+0f, 0x1.ceac48p-25f}, {0x1.29e9ep+0f, -0x1.5c0424p-25f},
-    {0x1.306fep+0f, 0x1.4636e2p-25f}, {0x1.371a74p+0f, -0x1.18aac6p-25f}, {0x1.3dea64p+0f, 0x1.824684p-25f}, {0x1.44e086p+0f, 0x1.8624b4p-30f},
-    {0x1.4bfdaep+0f, -0x1.593abcp-25f}, {0x1.5342b6p+0f, -0x1.2c561p-25f}, {0x1.5ab07ep+0f, -0x1.5bd5ecp-27f}, {0x1.6247ecp+0f, -0x1.f8b55p-25f},
-    {0x1.6a09e6p+0f, 0x1.9fcef4p-26f}, {0x1.71f75ep+0f, 0x1.1d8beep-25f}, {0x1.7a1148p+0f, -0x1.829fdp-25f}, {0x1.82589ap+0f, -0x1.accc7cp-26f},
-    {0x1.8ace54p+0f, 0x1.15506ep-27f}, {0x1.93737cp+0f, -0x1.e64744p-25f}, {0x1.9c4918p+0f, 0x1.51f848p-27f}, {0x1.a5503cp+0f, -0x1.b83b54p-25f},
-    {0x1.ae89fap+0f, -0x1.a94b14p-26f}, {0x1.b7f77p+0f, -0x1.a09438p-25f}, {0x1.c199bep+0f, -0x1.3d56b2p-27f}, {0x1.cb720ep+0f, -0x1.8837ccp-27f},
-    {0x1.d5818ep+0f, -0x1.822dbcp-27f}, {0x1.dfc974p+0f, -0x1.908c94p-25f}, {0x1.ea4afap+0f, 0x1.52486cp-27f}, {0x1.f50766p+0f, -0x1.246ebp-26f},
+// single precision: they are below 2^-30), 2^(n/32) = 2^e T_j from the table. ln2/32 and T_j
+// are split in three floats: n L1 cancels against a.hi without rounding (fused multiply-add),
+// n L2 is an exact product. Everything is carried to about 2^-52 of the result, so that its
+// one rounding to the format (2^-49, the low word's) is the error, as it was of the double
+// pipe's exp rounded to double-float: rms 2^-50.6 of both. (With T_j in two floats and sums
+// of one rounding a word it was 2^-49.4.) The double exp costs some twenty double operations a
+// point, 64 FP32 issue slots each.
+__device__ const float4 kExp2Tab[32] = { // 2^(j/32) = x + y + z
+    {0x1.0p+0f, 0x0.0p+0f, 0x0.0p+0f, 0.f}, {0x1.059b0ep+0f, -0x1.9d4f52p-25f, 0x1.0eb9f2p-50f, 0.f},
+    {0x1.0b5586p+0f, 0x1.9f3122p-25f, -0x1.3ace8ep-53f, 0.f}, {0x1.11301ep+0f, -0x1.fdb496p-25f, 0x1.49d77ep-53f, 0.f},
+    {0x1.172b84p+0f, -0x1.c15742p-27f, -0x1.232084p-52f, 0.f}, {0x1.1d4874p+0f, -0x1.d2e8cap-25f, -0x1.61fe92p-50f, 0.f},
+    {0x1.2387a6p+0f, 0x1.ceac48p-25f, -0x1.e64f82p-50f, 0.f}, {0x1.29e9ep+0f, -0x1.5c0424p-25f, 0x1.2c25d2p-52f, 0.f},
+    {0x1.306fep+0f, 0x1.4636e2p-25f, 0x1.4b7a36p-50f, 0.f}, {0x1.371a74p+0f, -0x1.18aac6p-25f, -0x1.563aeap-50f, 0.f},
+    {0x1.3dea64p+0f, 0x1.824684p-25f, 0x1.1ada0ap-51f, 0.f}, {0x1.44e086p+0f, 0x1.8624b4p-30f, 0x1.89b7ap-59f, 0.f},
+    {0x1.4bfdaep+0f, -0x1.593abcp-25f, 0x1.c750e6p-50f, 0.f}, {0x1.5342b6p+0f, -0x1.2c561p-25f, 0x1.df0a84p-52f, 0.f},
+    {0x1.5ab07ep+0f, -0x1.5bd5ecp-27f, 0x1.58c93p-52f, 0.f}, {0x1.6247ecp+0f, -0x1.f8b55p-25f, 0x1.2c7c3ep-50f, 0.f},
+    {0x1.6a09e6p+0f, 0x1.9fcef4p-26f, -0x1.b7ba68p-51f, 0.f}, {0x1.71f75ep+0f, 0x1.1d8beep-25f, 0x1.ee91b8p-51f, 0.f},
+    {0x1.7a1148p+0f, -0x1.829fdp-25f, 0x1.b5f544p-50f, 0.f}, {0x1.82589ap+0f, -0x1.accc7cp-26f, 0x1.4567c4p-51f, 0.f},
+    {0x1.8ace54p+0f, 0x1.15506ep-27f, -0x1.48b076p-53f, 0.f}, {0x1.93737cp+0f, -0x1.e64744p-25f, 0x1.3d1408p-50f, 0.f},
+    {0x1.9c4918p+0f, 0x1.51f848p-27f, 0x1.c7c46cp-56f, 0.f}, {0x1.a5503cp+0f, -0x1.b83b54p-25f, -0x1.ba5edep-51f, 0.f},
+    {0x1.ae89fap+0f, -0x1.a94b14p-26f, -0x1.50bc66p-51f, 0.f}, {0x1.b7f77p+0f, -0x1.a09438p-25f, 0x1.baa9ecp-50f, 0.f},
+    {0x1.c199bep+0f, -0x1.3d56b2p-27f, 0x1.110658p-55f, 0.f}, {0x1.cb720ep+0f, -0x1.8837ccp-27f, 0x1.1503ccp-52f, 0.f},
+    {0x1.d5818ep+0f, -0x1.822dbcp-27f, -0x1.b44bf4p-53f, 0.f}, {0x1.dfc974p+0f, -0x1.908c94p-25f, -0x1.469736p-52f, 0.f},
+    {0x1.ea4afap+0f, 0x1.52486cp-27f, 0x1.858f74p-52f, 0.f}, {0x1.f50766p+0f, -0x1.246ebp-26f, 0x1.9d3e12p-54f, 0.f},
 };
 
 struct df_exp_parts {
-    df T, p; // 2^(j/32), e^r - 1
-    int e;   // binary exponent
+    df T, p;  // 2^(j/32) without its third word, e^r - 1
+    float T2; // the third word
+    int e;    // binary exponent
 };
 __device__ __forceinline__ df_exp_parts exp_parts(df a)
 {
@@ -278,17 +290,26 @@ __device__ __forceinline__ df_exp_parts exp_parts(df a)
     df_exp_parts o;
     o.p = add_lazy(r, mul_lazy(mul_lazy(r, r), h)); // r + r^2 (1/2 + r (1/6 + r q))
     const int N = (int)n;
-    const float2 t = __ldg(kExp2Tab + (N & 31));
+    const float4 t = __ldg(kExp2Tab + (N & 31));
     o.T = df(t.x, t.y);
+    o.T2 = t.z;
     o.e = N >> 5;
     return o;
 }
 // x 2^e for any e (two factors where 2^e is below the normal range)
-__device__ __forceinline__ df scale2(df x, int e)
+__device__ __forceinline__ float scale2(float x, int e)
 {
     const int e1 = max(e, -126), e2 = max(e - e1, -126);
-    const float f1 = __int_as_float((e1 + 127) << 23), f2 = __int_as_float((e2 + 127) << 23);
-    return df(x.hi * f1 * f2, x.lo * f1 * f2);
+    return x * __int_as_float((e1 + 127) << 23) * __int_as_float((e2 + 127) << 23);
+}
+// hi + x + l0 + l1 + rest with one rounding, of the result's low word: |hi| >= |x|, l0 and
+// l1 of the size of that sum's rounding or below, rest below theirs
+__device__ __forceinline__ df sum_once(float hi, float x, float l0, float l1, float rest)
+{
+    const df s = two_sum(hi, x), l = two_sum(s.lo, l0), k = two_sum(l.hi, l1);
+    df o = fast_two_sum(s.hi, k.hi);
+    o.lo += l.lo + k.lo + rest;
+    return o;
 }
 __device__ __forceinline__ df exp(df a)
 {
@@ -296,33 +317,33 @@ __device__ __forceinline__ df exp(df a)
     a = renorm_exact(a);
     if (!(a.hi < 88.0f)) return df(::exp((double)a)); // near and above the overflow of a float, NaN
     const df_exp_parts x = exp_parts(a);
-    return scale2(renorm(add_lazy(x.T, mul_lazy(x.T, x.p))), x.e);
+    const df m = mul_lazy(x.T, x.p), y = sum_once(x.T.hi, m.hi, x.T.lo, m.lo, x.T2);
+    return df(scale2(y.hi, x.e), scale2(y.lo, x.e));
 }
-// expm1: the series below 0.35, where e^a - 1 would cancel
+// expm1: the series below 0.1, where e^a - 1 would cancel
 __device__ __forceinline__ df expm1(df a)
 {
     if (a.hi < -200.0f) return df(-1.f, 0.f);
     a = renorm_exact(a);
     if (!(a.hi < 88.0f)) return df(::expm1((double)a));
-    if (::fabsf(a.hi) < 0.35f) {
-        // a + a^2 (1/2! + a (1/3! + ...)), terms from a^9/9! on in single precision
-        float t = (float)(1.0 / 87178291200.0);
-        t = fmaf(t, a.hi, (float)(1.0 / 6227020800.0));
-        t = fmaf(t, a.hi, (float)(1.0 / 479001600.0));
-        t = fmaf(t, a.hi, (float)(1.0 / 39916800.0));
+    if (::fabsf(a.hi) < 0.1f) {
+        // a + a^2 (1/2! + a (1/3! + ...)), terms from a^7/7! on in single precision
+        float t = (float)(1.0 / 39916800.0);
         t = fmaf(t, a.hi, (float)(1.0 / 3628800.0));
         t = fmaf(t, a.hi, (float)(1.0 / 362880.0));
+        t = fmaf(t, a.hi, (float)(1.0 / 40320.0));
+        t = fmaf(t, a.hi, (float)(1.0 / 5040.0));
         df s(t, 0.f);
-        const double c[7] = {1.0 / 40320, 1.0 / 5040, 1.0 / 720, 1.0 / 120, 1.0 / 24, 1.0 / 6, 1.0 / 2};
+        const double c[5] = {1.0 / 720, 1.0 / 120, 1.0 / 24, 1.0 / 6, 1.0 / 2};
 #pragma unroll
-        for (int i = 0; i < 7; i++) s = add_lazy(df(c[i]), mul_lazy(s, a));
-        return renorm(add_lazy(a, mul_lazy(mul_lazy(a, a), s)));
+        for (int i = 0; i < 5; i++) s = add_lazy(df(c[i]), mul_lazy(s, a));
+        const df w = mul_lazy(mul_lazy(a, a), s);
+        return sum_once(a.hi, w.hi, a.lo, w.lo, 0.f);
     }
     const df_exp_parts x = exp_parts(a);
-    const df T = scale2(x.T, x.e);
-    df d = two_sum(T.hi, -1.0f);
-    d.lo += T.lo;
-    return renorm(add_lazy(d, mul_lazy(T, x.p)));
+    const df T(scale2(x.T.hi, x.e), scale2(x.T.lo, x.e)), m = mul_lazy(T, x.p), d = two_sum(T.hi, -1.0f);
+    const df l = two_sum(d.lo, T.lo);
+    return sum_once(d.hi, m.hi, l.hi, m.lo, l.lo + scale2(x.T2, x.e));
 }
 
 } // namespace fch

@@ -1,0 +1,52 @@
+"""GPU: the double-float functions of the pointwise and ETD stages against extended
+precision, at the accuracy of the format."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+from paper_2006_04784_gb300 import build as B  # noqa: E402
+
+B.build()
+from paper_2006_04784_gb300 import fch  # noqa: E402
+
+LD = np.longdouble
+
+
+def _split(x):
+    """x rounded to double-float, as extended precision"""
+    h = x.astype(np.float32)
+    return h.astype(LD) + (x - h.astype(LD)).astype(np.float32).astype(LD)
+
+
+def _args(lo, hi, n=50000):
+    return _split(np.random.default_rng(11).uniform(lo, hi, n).astype(LD)).astype(np.float64)
+
+
+def _rms(x):
+    return float(np.sqrt((x * x).mean()))
+
+
+@pytest.mark.parametrize("lo,hi", [(-0.01, 0.01), (-0.1, 0.1), (0.1, 1.0), (-1.0, -0.1), (-5.0, 0.0), (-20.0, 0.0), (0.0, 80.0)])
+def test_exp_and_expm1_round_once(lo, hi):
+    # the error is that of rounding the exact value to double-float: what remains (2^-52 and
+    # below, expm1 near 0.1 2^-51) adds at most a twentieth to its rms and a bit to its largest
+    x = _args(lo, hi)
+    xt = torch.tensor(x, device="cuda:0")
+    out = [torch.empty_like(xt) for _ in range(2)]
+    torch.cuda.synchronize()
+    f = fch.lib().fch_debug_dfl_exp
+    f.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_long, C.c_void_p]
+    assert f(xt.data_ptr(), out[0].data_ptr(), out[1].data_ptr(), x.size, None) == 0
+    for o, ref in zip(out, (np.exp(x.astype(LD)), np.expm1(x.astype(LD)))):
+        err, own = o.cpu().numpy().astype(LD) / ref - 1, _split(ref) / ref - 1
+        assert _rms(err) <= 1.05 * _rms(own)
+        assert np.abs(err).max() <= 2.0 ** -48
+
+
