@@ -9,7 +9,7 @@
 #include <vector>
 
 #include "../../include/fch.h"
-#include "fch_ctrl.cuh"
+#include "fch_kernels.cuh"
 #include "fch_internal.h"
 
 // ---------------------------------------------------------------------------
@@ -2474,6 +2474,34 @@ extern "C" int fch_debug_dfl_exp(const double *x, double *ex, double *em, long c
     if (!x || !ex || !em || cnt < 1) return FCH_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     fch_debug_dfl_exp_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(x, ex, em, cnt);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e == cudaSuccess ? FCH_OK : FCH_ECUDA;
+}
+
+__global__ void fch_debug_dfl_point_kernel(const fch_consts<fch::df> k, int phi, const double *x, double *out, long cnt)
+{
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= cnt) return;
+    fch::df a, b, c;
+    if (phi)
+        fch::etd_phi<fch::df>(fch::df(x[i]), a, b, c);
+    else
+        fch::well<fch::df>(k, fch::df(x[i]), a, b, c, true);
+    out[i] = (double)a;
+    out[cnt + i] = (double)b;
+    out[2 * cnt + i] = (double)c;
+}
+
+// test hook: the double-float (e^z, phi1, phi2) of the ETD scheme (phi = 1) or (W, W', W'')
+// of the well of p (phi = 0) on cnt device doubles, out [3][cnt]; 0 or a status
+extern "C" int fch_debug_dfl_point(const fch_params *p, int phi, const double *x, double *out, long cnt, void *stream)
+{
+    if (!p || !x || !out || cnt < 1) return FCH_EINVAL;
+    fch_consts<fch::df> k;
+    fill_consts(k, *p, 1.0, 1.0, 1.0);
+    cudaStream_t s = (cudaStream_t)stream;
+    fch_debug_dfl_point_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(k, phi, x, out, cnt);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     return e == cudaSuccess ? FCH_OK : FCH_ECUDA;

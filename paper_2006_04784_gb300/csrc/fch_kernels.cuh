@@ -366,22 +366,23 @@ __device__ __forceinline__ bool pass_skipped(const fch_kparams &kp)
 
 // ---------------------------------------------------------------------------
 // ETD phi functions in precision T: phi1 = (e^z - 1)/z, phi2 = (e^z - 1 - z)/z^2.
-// Below a threshold (1e-2 in double, 0.1 in float and double-float, where the direct forms
-// lose digits to cancellation) the Taylor series sum_j z^j/(j+1)!, sum_j z^j/(j+2)!
-// in Horner form, j < 10; the direct forms above (double-float: one reciprocal).
+// Below a threshold (1e-2 in double, 0.1 in float, 0.2 in double-float, where the direct
+// forms lose digits to cancellation) the Taylor series sum_j z^j/(j+1)!, sum_j z^j/(j+2)!
+// in Horner form, j < 10 (double-float: j < 12); the direct forms above.
 template <typename T> __device__ __forceinline__ void etd_phi(T z, T &ez, T &p1, T &p2)
 {
     constexpr bool dfl = std::is_same<T, df>::value;
+    constexpr int J = dfl ? 12 : 10;
     ez = exp(z);
-    const T thr = std::is_same<T, double>::value ? (T)1e-2 : (T)0.1;
+    const T thr = std::is_same<T, double>::value ? (T)1e-2 : dfl ? (T)0.2 : (T)0.1;
     if (fabs(z) < thr) {
-        // inverse factorials 1/1! .. 1/11!
-        const T f[11] = {(T)1.0, (T)(1.0 / 2), (T)(1.0 / 6), (T)(1.0 / 24), (T)(1.0 / 120),
+        // inverse factorials 1/1! .. 1/13!
+        const T f[13] = {(T)1.0, (T)(1.0 / 2), (T)(1.0 / 6), (T)(1.0 / 24), (T)(1.0 / 120),
                          (T)(1.0 / 720), (T)(1.0 / 5040), (T)(1.0 / 40320), (T)(1.0 / 362880),
-                         (T)(1.0 / 3628800), (T)(1.0 / 39916800)};
-        T a = f[9], b = f[10];
+                         (T)(1.0 / 3628800), (T)(1.0 / 39916800), (T)(1.0 / 479001600), (T)(1.0 / 6227020800.0)};
+        T a = f[J - 1], b = f[J];
 #pragma unroll
-        for (int j = 8; j >= 0; j--) {
+        for (int j = J - 2; j >= 0; j--) {
             a = radd(rmul(a, z), f[j]);
             b = radd(rmul(b, z), f[j + 1]);
         }
@@ -389,14 +390,8 @@ template <typename T> __device__ __forceinline__ void etd_phi(T z, T &ez, T &p1,
         p2 = b;
     } else {
         const T em = expm1(z);
-        if constexpr (dfl) {
-            const T iz = recip(z);
-            p1 = rmul(em, iz);
-            p2 = rmul(rmul(rsub(em, z), iz), iz);
-        } else {
-            p1 = em / z;
-            p2 = (em - z) / (z * z);
-        }
+        p1 = em / z;
+        p2 = (em - z) / (z * z);
     }
 }
 

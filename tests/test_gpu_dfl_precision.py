@@ -50,3 +50,36 @@ def test_exp_and_expm1_round_once(lo, hi):
         assert np.abs(err).max() <= 2.0 ** -48
 
 
+def _point(phi, q, x):
+    xt = torch.tensor(x, device="cuda:0")
+    out = torch.empty((3, x.size), dtype=torch.float64, device="cuda:0")
+    torch.cuda.synchronize()
+    f = fch.lib().fch_debug_dfl_point
+    f.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_long, C.c_void_p]
+    p = fch.params_default(q)
+    assert f(C.byref(p), phi, xt.data_ptr(), out.data_ptr(), x.size, None) == 0
+    return out.cpu().numpy().astype(LD)
+
+
+@pytest.mark.parametrize("lo,hi,t1,t2", [(1e-4, 0.2, -50.5, -50.5), (0.199, 0.201, -49.0, -46.0), (0.2, 1.0, -49.0, -46.8),
+                                         (1.0, 30.0, -49.0, -47.8), (30.0, 1e4, -49.3, -48.0)])
+def test_etd_phi(lo, hi, t1, t2):
+    # rms bounds (bits): the series to its 2^-51; the quotients to half a bit above what they
+    # measure, e^z - 1 - z having lost 1 / (z/2) of its size below z = 2
+    z = -np.exp(_args(np.log(lo), np.log(hi)))
+    z = _split(z.astype(LD)).astype(np.float64)
+    ez, p1, p2 = _point(1, 0.0, z)
+    z = z.astype(LD)
+    if hi <= 1.0:
+        r1, r2 = np.zeros_like(z), np.zeros_like(z)
+        fact = np.cumprod(np.arange(1, 24).astype(LD))
+        for j in range(20, -1, -1):
+            r1, r2 = r1 * z + 1 / fact[j], r2 * z + 1 / fact[j + 1]
+    else:
+        r1, r2 = np.expm1(z) / z, (np.expm1(z) - z) / (z * z)
+    ok = np.exp(z) > 1e-25  # (below, the low word leaves the range of a float)
+    assert np.abs(ez / np.exp(z) - 1)[ok].max() <= 2.0 ** -48 if ok.any() else True
+    assert _rms(p1 / r1 - 1) <= 2.0 ** t1
+    assert _rms(p2 / r2 - 1) <= 2.0 ** t2
+
+
