@@ -491,7 +491,6 @@ static void fill_consts(fch_consts<T> &k, const fch_params &p, double kf, double
     k.bm = (T)p.b_minus;
     k.bp = (T)p.b_plus;
     k.eps = (T)p.eps;
-    k.ieps = (T)(1.0 / p.eps);
     k.q = (T)p.q;
     k.qeps = (T)(p.q * p.eps);
     k.qoe = (T)(p.q / p.eps);

@@ -83,3 +83,22 @@ def test_etd_phi(lo, hi, t1, t2):
     assert _rms(p2 / r2 - 1) <= 2.0 ** t2
 
 
+@pytest.mark.parametrize("q,bits", [(0.2, (-45.9, -46.8, -46.9)), (0.5, (-45.9, -46.8, -46.3))])
+def test_regularised_well(q, bits):
+    # W, W', W'' over the range of a solution: rms bounds (bits of the rms value) a third of a
+    # bit above what renormalised sums and the quotient (u - b_-) / eps measure
+    p = fch.params_default(q)
+    u = _args(-1.6, 1.6)
+    got = _point(0, q, u)
+    c = lambda v: _split(np.array([v], dtype=LD))[0]  # noqa: E731  (constants as the library holds them)
+    u = u.astype(LD)
+    v, w = u - c(p.b_minus), u - c(p.b_plus)
+    x = v / c(p.eps)
+    e = np.exp(-np.abs(x))
+    s, th = 2 * e / (1 + e * e), np.sign(x) * (1 - e * e) / (1 + e * e)
+    A, A1 = v * v / 2 + c(p.q * p.eps) * (1 - s), v + c(p.q) * s * th
+    A2 = 1 + c(p.q / p.eps) * s * (2 * s * s - 1)
+    g3, c3 = c(p.gamma / 3.0), c(0.5 * (3.0 * p.b_plus - p.b_minus))
+    Bq, B1 = w * w / 2 + g3 * (u - c3), w + g3
+    for a, r, t in zip(got, (A * Bq, A1 * Bq + A * B1, A2 * Bq + 2 * A1 * B1 + A), bits):
+        assert _rms(a - r) <= 2.0 ** t * _rms(r), t
