@@ -39,12 +39,12 @@ constexpr bool row_xf(int mode) { return mode == RM_R2C_LOAD || mode == RM_C2R_S
 constexpr bool col_xf(int mode) { return mode == CM_FWD_STORE || mode == CM_INV_LOAD; }
 
 // What a pass is built for, by element (16 bytes: double and double-float; 8: single) and
-// size. Points a thread: two (radix-2 stages) where a pass is a few warps on the 608
-// sub-partitions and the time is the dependent chain of one of them, in double to 128^2 and
-// in the others to 256^2; four (radix-4) in double at 256^2, in double-float to 1024^2 and
+// size. Points a thread: two (radix-8 stages level by level) where a pass is a few warps on
+// the 608 sub-partitions and the time is the dependent chain of one of them, in double to
+// 128^2 and in the others to 256^2; four (radix-4) in double at 256^2, in double-float to 1024^2 and
 // in single at 512^2; eight (radix-8 stages, fewer exchanges and twiddle products) where
-// the pipes are the bound or the blocks would get too large. Two points cost more
-// operations (24 a point of a 128-point transform, 22 at four) and twice the exchanges, but
+// the pipes are the bound or the blocks would get too large. Two points cost as many
+// operations as four (22 a point of a 128-point transform) and twice the exchanges, but
 // halve the instructions of a warp, and a double-precision one holds its sub-partition for
 // 64 cycles whatever its lanes do. Blocks an SM: enough registers that nothing spills; at
 // 1024^2 four blocks of 256 threads (two waves whose loads, transforms and stores overlap)
@@ -114,30 +114,96 @@ template <bool WS> __device__ __forceinline__ void seq_sync()
         __syncthreads();
 }
 
-// The stage of two points a thread and sub-length Ns = 2^S: its factor exp(-2 pi i j / 2 Ns),
-// j < Ns, from the table of radix-4 stages (entry Ns' - 4 + (r - 1) Ns' + j =
-// exp(-2 pi i r j / 4 Ns')): where Ns is a power of four it is r = 2 of Ns (r = 1 where the
-// table ends in a radix-2 stage), else r = 1 of Ns / 2 and, in the upper half, a turn by -i.
-template <int LOGN, int S, typename C> __device__ __forceinline__ C reg_twist2(C x, const C *__restrict__ tw, int t)
+// A stage of radix R = 2^LR and sub-length Ns = 8^S by threads of two points. Its butterflies
+// run level by level in the order of eight points a thread (bfly8: the same products and
+// sums, twiddles from the table of radix-8 stages), the threads (j, c) = (t mod N/R, t / (N/R))
+// of butterfly j trading values between the levels through the natural slots j + (N/R) q:
+// level 1 takes the points c and c + R/2, level 2 the sums (c even) or differences (c odd) of
+// the even (c < 2) or odd points, level 3 the outputs k = c of both halves. (Radix-2 stages
+// with a twiddle product each cost as many instructions and exchanges and take the same time,
+// but round more. F(u) in single precision at 64^2, q = 0.5: 1.16e-4 from 64 bits, as here
+// 1.08e-4; a double transform of noise at 64^2: 3.16e-16, here 2.70e-16.)
+// Double-float is renormalised at the end of every stage: F(u) at 256^2, q = 0, 8.9e-13 from
+// 64 bits, after the first and last 1.03e-12, after the last alone 1.27e-12 (radix-2 stages
+// 1.09e-12); 64 IMEX trials 1723, 1721, 1722 us.
+// The twiddles of all stages are read before the first: read in their stages, the first
+// point's in a branch, the same trials take 1838 us.
+template <bool DB, bool WS, typename C>
+__device__ __forceinline__ void reg_trade2(C *v, C *&buf, C *&buf2, int w0, int w1, int t, int half)
 {
-    constexpr int Ns = 1 << S;
-    if (S == 0) return x;
-    if (S % 2 == 0) return btw(x, ldg(tw + Ns - 4 + (S + 1 == LOGN ? 0 : Ns) + (t & (Ns - 1))));
-    constexpr int Nh = Ns >> 1;
-    if (S > 1) x = btw(x, ldg(tw + Nh - 4 + (t & (Nh - 1))));
-    return t & Nh ? mk<C>(x.y, flip(x.x, 0x80000000u)) : x;
+    if (!DB) seq_sync<WS>();
+    buf[skew(w0)] = v[0];
+    buf[skew(w1)] = v[1];
+    seq_sync<WS>();
+    v[0] = buf[skew(t)];
+    v[1] = buf[skew(t + half)];
+    if (DB) {
+        C *o = buf;
+        buf = buf2;
+        buf2 = o;
+    }
+}
+// the twiddles of a stage's two points (the first where c > 0), read before the transform
+template <int LOGN, int LR, int S, typename C>
+__device__ __forceinline__ void reg_twiddles2(C *w, const C *__restrict__ tw, int t)
+{
+    constexpr int LB = LOGN - LR, Ns = 1 << (3 * S);
+    const int c = t >> LB;
+    tw += (Ns - 8) + (t & ((1 << LB) - 1) & (Ns - 1));
+    w[0] = ldg(tw + (c > 0 ? c - 1 : 0) * Ns);
+    w[1] = ldg(tw + (c + (1 << LR >> 1) - 1) * Ns);
+}
+template <int LOGN, int LR, int S, bool DB, bool WS, typename C>
+__device__ __forceinline__ void reg_stage2(C *v, C *&buf, C *&buf2, const C *w, int t)
+{
+    typedef decltype(C().x) R;
+    constexpr int N = 1 << LOGN, LB = LOGN - LR, NB = 1 << LB, Ns = 1 << (3 * S);
+    constexpr bool last = (Ns << LR) == N;
+    static_assert(LR == 3 || last, "stages of radix 2 and 4 come last");
+    const int j = t & (NB - 1), c = t >> LB;
+    if (Ns > 1) {
+        if (c > 0) v[0] = btw(v[0], w[0]);
+        v[1] = btw(v[1], w[1]);
+    }
+    bfly2<-1>(v[0], v[1]);
+    if (LR >= 2) {
+        const int q = LR == 3 ? 2 * (c & 1) + 4 * (c >> 1) : 2 * c;
+        reg_trade2<DB, WS>(v, buf, buf2, j + q * NB, j + (q + 1) * NB, t, N / 2);
+        if (c & 1) v[1] = mk<C>(v[1].y, flip(v[1].x, 0x80000000u));
+        bfly2<-1>(v[0], v[1]);
+    }
+    if (LR == 3) {
+        const int q = (c & 1) + 4 * (c >> 1);
+        reg_trade2<DB, WS>(v, buf, buf2, j + q * NB, j + (q + 2) * NB, t, N / 2);
+        const C e = v[0];
+        C o = v[1];
+        if (c & 2) o = mk<C>(o.y, flip(o.x, 0x80000000u));
+        const R s = (R)0.70710678118654752440;
+        if (NB >= 32) { // whole warps of one c
+            if (c & 1) {
+                bscaled(e, mk<C>(radd(o.x, o.y), rsub(o.y, o.x)), s, v[0], v[1]);
+            } else {
+                v[0] = badd(e, o);
+                v[1] = bsub(e, o);
+            }
+        } else {
+            const C x = mk<C>(radd(o.x, o.y), rsub(o.y, o.x));
+            bscaled(e, c & 1 ? x : o, c & 1 ? s : (R)1, v[0], v[1]);
+        }
+    }
+    v[0] = bnorm(v[0]);
+    v[1] = bnorm(v[1]);
+    if (!last) {
+        const int d = ((j >> (3 * S)) << (3 * S + LR)) + (j & (Ns - 1)) + c * Ns;
+        reg_trade2<DB, WS>(v, buf, buf2, d, d + 4 * Ns, t, N / 2);
+    }
 }
 
-// (Double-float is renormalised after the fourth radix-2 stage too, not only at the end: the
-// rounding of twice as many stages would otherwise exceed that of radix 4. F(u) of a bilayer
-// at 64^2, q = 0.5, against double: radix 4 9.5e-12, radix 2 without 1.04e-11, with 8.1e-12;
-// after every second stage 7.2e-12, after every one 6.1e-12, but 24 PSD trials of 256^2 take
-// 2345, 2394 and 2400 us.)
 // (TWG: the twiddles lie in global memory, read through the read-only cache; else shared)
 template <int LOGN, int PPT, int LR, int S, bool DB, bool WS, bool TWG = true, typename C>
 __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__restrict__ tw, int t)
 {
-    constexpr int N = 1 << LOGN, tps = N / PPT, LP = PPT == 8 ? 3 : PPT == 4 ? 2 : 1;
+    constexpr int N = 1 << LOGN, tps = N / PPT, LP = PPT == 8 ? 3 : 2;
     constexpr int R = 1 << LR, NB = PPT / R;
     constexpr int lNs = S * LP, Ns = 1 << lNs;
     constexpr bool last = (Ns << LR) == N;
@@ -147,9 +213,7 @@ __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__re
         C x[R];
 #pragma unroll
         for (int r = 0; r < R; r++) x[r] = v[b + NB * r];
-        if (PPT == 2) {
-            x[1] = reg_twist2<LOGN, S>(x[1], tw, j);
-        } else if (Ns > 1) {
+        if (Ns > 1) {
             const C *tws = tw + (Ns - PPT) + (j & (Ns - 1));
 #pragma unroll
             for (int r = 1; r < R; r++) x[r] = btw(x[r], TWG ? ldg(tws + (r - 1) * Ns) : tws[(r - 1) * Ns]);
@@ -161,7 +225,7 @@ __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__re
         else
             bfly2<-1>(x[0], x[1]);
 #pragma unroll
-        for (int r = 0; r < R; r++) v[b + NB * r] = last || (PPT == 2 && S == 3) ? bnorm(x[r]) : x[r];
+        for (int r = 0; r < R; r++) v[b + NB * r] = last ? bnorm(x[r]) : x[r];
     }
     if (!last) {
         if (!DB) seq_sync<WS>();
@@ -186,17 +250,24 @@ __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__re
 template <int LOGN, int PPT, bool DB, bool WS, typename C>
 __device__ __forceinline__ void fft_reg(C *v, C *&buf, C *&buf2, const C *__restrict__ tw, int t)
 {
-    constexpr int LP = PPT == 8 ? 3 : PPT == 4 ? 2 : 1, NF = LOGN / LP, REM = LOGN % LP;
-    static_assert(NF >= 1 && NF <= 8, "two to eight stages");
-    reg_stage<LOGN, PPT, LP, 0, DB, WS>(v, buf, buf2, tw, t);
-    if constexpr (NF > 1) reg_stage<LOGN, PPT, LP, 1, DB, WS>(v, buf, buf2, tw, t);
-    if constexpr (NF > 2) reg_stage<LOGN, PPT, LP, 2, DB, WS>(v, buf, buf2, tw, t);
-    if constexpr (NF > 3) reg_stage<LOGN, PPT, LP, 3, DB, WS>(v, buf, buf2, tw, t);
-    if constexpr (NF > 4) reg_stage<LOGN, PPT, LP, 4, DB, WS>(v, buf, buf2, tw, t);
-    if constexpr (NF > 5) reg_stage<LOGN, PPT, LP, 5, DB, WS>(v, buf, buf2, tw, t);
-    if constexpr (NF > 6) reg_stage<LOGN, PPT, LP, 6, DB, WS>(v, buf, buf2, tw, t);
-    if constexpr (NF > 7) reg_stage<LOGN, PPT, LP, 7, DB, WS>(v, buf, buf2, tw, t);
-    if constexpr (REM > 0) reg_stage<LOGN, PPT, REM, NF, DB, WS>(v, buf, buf2, tw, t);
+    constexpr int LP = PPT == 4 ? 2 : 3, NF = LOGN / LP, REM = LOGN % LP;
+    if constexpr (PPT == 2) {
+        static_assert(LOGN >= 6 && LOGN <= 8, "two stages of radix 8");
+        C w1[2], w2[2];
+        reg_twiddles2<LOGN, 3, 1>(w1, tw, t);
+        if constexpr (REM > 0) reg_twiddles2<LOGN, REM, 2>(w2, tw, t);
+        reg_stage2<LOGN, 3, 0, DB, WS>(v, buf, buf2, w1, t);
+        reg_stage2<LOGN, 3, 1, DB, WS>(v, buf, buf2, w1, t);
+        if constexpr (REM > 0) reg_stage2<LOGN, REM, 2, DB, WS>(v, buf, buf2, w2, t);
+    } else {
+        static_assert(NF >= 1 && NF <= 5, "one to five stages");
+        reg_stage<LOGN, PPT, LP, 0, DB, WS>(v, buf, buf2, tw, t);
+        if constexpr (NF > 1) reg_stage<LOGN, PPT, LP, 1, DB, WS>(v, buf, buf2, tw, t);
+        if constexpr (NF > 2) reg_stage<LOGN, PPT, LP, 2, DB, WS>(v, buf, buf2, tw, t);
+        if constexpr (NF > 3) reg_stage<LOGN, PPT, LP, 3, DB, WS>(v, buf, buf2, tw, t);
+        if constexpr (NF > 4) reg_stage<LOGN, PPT, LP, 4, DB, WS>(v, buf, buf2, tw, t);
+        if constexpr (REM > 0) reg_stage<LOGN, PPT, REM, NF, DB, WS>(v, buf, buf2, tw, t);
+    }
 }
 
 __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
@@ -228,7 +299,7 @@ row_pass_r(const fch_kparams kp)
     __shared__ double red_scratch[FCH_NRED * 32];
     if (kp.nfft && blockIdx.x == 0 && threadIdx.x == 0)
         atomicAdd(kp.nfft, (MODE == RM_R2C_LOAD || MODE == RM_C2R_STORE || MODE == RM_ENERGY) ? 2ull : 4ull);
-    const C *tw = (const C *)(PPT == 8 ? kp.tw : kp.tw4);
+    const C *tw = (const C *)(PPT == 4 ? kp.tw4 : kp.tw);
     const int rr = threadIdx.x / TPS, t = threadIdx.x % TPS, y = blockIdx.x * G::rpb + rr;
     C *buf = (C *)smem_raw + rr * G::SL, *buf2 = buf + (G::db ? G::rpb * G::SL : 0);
     C *Zrow = pair_Z<C>(kp, N) + (long)y * N;
@@ -353,7 +424,7 @@ __device__ __forceinline__ void col_body_r(const fch_kparams &kp)
     if (pass_skipped(kp)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red_scratch[FCH_NRED * 32];
-    const C *tw = (const C *)(PPT == 8 ? kp.tw : kp.tw4);
+    const C *tw = (const C *)(PPT == 4 ? kp.tw4 : kp.tw);
     const fch_consts<T> &K = consts<T>(kp);
     const bool inv = TR::INV_ALWAYS || (TR::INV_OPT && (kp.flags & (FCH_FL_PACK_F | FCH_FL_PACK_USTAR)));
     const bool has_red = MODE == CM_SAV_PQ || MODE == CM_PSD_ITER ||
