@@ -199,6 +199,10 @@ __device__ __forceinline__ void reg_stage2(C *v, C *&buf, C *&buf2, const C *w, 
     }
 }
 
+// Radix-4 stages renormalise double-float after the third as well as at the end, their
+// rounding being that of more stages than radix 8 has: F(u) at 512^2, q = 0, 1.14e-12 from 64
+// bits, without 1.45e-12 (eight points 1.39e-12), at 1024^2 1.21e-12, 1.57e-12 (1.54e-12);
+// 48 IMEX trials of 1024^2 6007 -> 6058 us.
 // (TWG: the twiddles lie in global memory, read through the read-only cache; else shared)
 template <int LOGN, int PPT, int LR, int S, bool DB, bool WS, bool TWG = true, typename C>
 __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__restrict__ tw, int t)
@@ -225,7 +229,7 @@ __device__ __forceinline__ void reg_stage(C *v, C *&buf, C *&buf2, const C *__re
         else
             bfly2<-1>(x[0], x[1]);
 #pragma unroll
-        for (int r = 0; r < R; r++) v[b + NB * r] = last ? bnorm(x[r]) : x[r];
+        for (int r = 0; r < R; r++) v[b + NB * r] = last || (PPT == 4 && S == 2) ? bnorm(x[r]) : x[r];
     }
     if (!last) {
         if (!DB) seq_sync<WS>();

@@ -62,3 +62,10 @@ def test_two_points_a_thread(n, prec):
     # the mean error over six fields is known to about 1 % (its seeds differ by 2-3 %)
     built, generic = _errors(n, prec, 6, LD)
     assert built <= 1.04 * generic
+
+
+@pytest.mark.parametrize("n", [512, 1024])
+def test_four_points_a_thread_in_double_float(n):
+    # two fields: the mean error over a million points is known to half a per cent
+    built, generic = _errors(n, 2, 2, np.float64)
+    assert built <= 1.01 * generic
