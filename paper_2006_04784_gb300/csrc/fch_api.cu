@@ -9,7 +9,7 @@
 #include <vector>
 
 #include "../../include/fch.h"
-#include "fch_kernels.cuh"
+#include "fch_reg.cuh"
 #include "fch_internal.h"
 
 // ---------------------------------------------------------------------------
@@ -2456,6 +2456,22 @@ extern "C" int fch_debug_twiddles(int n, int lp, double *out)
     if (!pow2_in_range(n) || (lp != 2 && lp != 3) || !out) return 1;
     make_twiddles(n, out, lp);
     return 0;
+}
+
+// points a thread of the built passes that a launch at the default tiles takes (0: another
+// kernel): xf 1 those of standalone transforms, 0 of steps; tw4: with the radix-4 table at
+// hand (CPU tests)
+extern "C" int fch_debug_built_pass(int n, int prec, int xf, int tw4)
+{
+    if (!pow2_in_range(n) || prec < 0 || prec > 2) return -1;
+    fch_kparams kp;
+    memset(&kp, 0, sizeof(kp));
+    kp.logN = ilog2(n);
+    kp.tw = &kp;
+    kp.tw4 = tw4 ? &kp : nullptr;
+    return prec == FCH_MIXED    ? fch::reg_pass<float>(kp, 0, xf != 0)
+           : prec == FCH_FP32X2 ? fch::reg_pass<fch::df>(kp, 0, xf != 0)
+                                : fch::reg_pass<double>(kp, 0, xf != 0);
 }
 
 __global__ void fch_debug_dfl_exp_kernel(const double *x, double *ex, double *em, long cnt)

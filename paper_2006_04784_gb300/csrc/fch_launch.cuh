@@ -34,14 +34,6 @@ inline cudaError_t set_smem(pass_fn f, int bytes, int floor_bytes, int &cur)
     return e;
 }
 
-// the passes built for a grid size (fch_reg.cu): tile 0, N = 64 ... 2048, where the
-// twiddle tables are at hand (the radix-4 one: contexts and plans, not fch_fft_r2c_noalloc,
-// whose single-precision transforms need the radix-8 one only)
-template <typename T> bool reg_applies(const fch_kparams &kp, int tile)
-{
-    return tile == 0 && kp.logN >= 6 && kp.logN <= 11 && (sizeof(T) == 4 || kp.tw4);
-}
-
 // single precision at N = 1024: the warp-transform columns (tile -2)
 template <int M> cudaError_t launch_col_w(const fch_kparams &kp, cudaStream_t s)
 {
@@ -171,7 +163,7 @@ template <typename T, int M> cudaError_t launch_row(const fch_kparams &kp, cudaS
 #ifndef FCH_NO_COL
 cudaError_t FCH_CAT(fch_launch_col_, FCH_SUFFIX)(int mode, const fch_kparams &kp, cudaStream_t s)
 {
-    if (reg_applies<FCH_T>(kp, kp.tile_col) && !cols_staged<FCH_T>(mode, kp)) {
+    if (fch::reg_pass<FCH_T>(kp, kp.tile_col, fch::col_xf(mode)) && !cols_staged<FCH_T>(mode, kp)) {
         switch (kp.logN) {
         case 6: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 6)(mode, kp, s);
         case 7: return FCH_REG(fch_reg_col_, FCH_SUFFIX, 7)(mode, kp, s);
@@ -201,7 +193,7 @@ cudaError_t FCH_CAT(fch_launch_col_, FCH_SUFFIX)(int mode, const fch_kparams &kp
 #ifndef FCH_NO_ROW
 cudaError_t FCH_CAT(fch_launch_row_, FCH_SUFFIX)(int mode, const fch_kparams &kp, cudaStream_t s)
 {
-    if (reg_applies<FCH_T>(kp, kp.tile_row)) {
+    if (fch::reg_pass<FCH_T>(kp, kp.tile_row, fch::row_xf(mode))) {
         switch (kp.logN) {
         case 6: return FCH_REG(fch_reg_row_, FCH_SUFFIX, 6)(mode, kp, s);
         case 7: return FCH_REG(fch_reg_row_, FCH_SUFFIX, 7)(mode, kp, s);

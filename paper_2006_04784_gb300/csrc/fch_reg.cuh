@@ -64,12 +64,27 @@ constexpr bool col_xf(int mode) { return mode == CM_FWD_STORE || mode == CM_INV_
 // the steps (128^2, one pair 19.7 -> 14.6 us at 2 points, 8 pairs 33.3 -> 35.1, 16 pairs and
 // an odd field 77.8 -> 73.8). One choice for every batch: a field's result does not depend
 // on how many are transformed with it.
+template <typename T> constexpr int reg_points(int logn, bool xf)
+{
+    return sizeof(T) == 4                  ? (xf ? 8 : logn <= 8 ? 2 : logn == 9 ? 4 : 8)
+           : std::is_same<T, df>::value ? (logn <= 8 ? 2 : logn <= 10 ? 4 : 8)
+                                           : (logn <= 7 ? 2 : logn <= 8 ? 4 : 8);
+}
+
+// points a thread of the built pass that a launch takes, 0 where it takes another kernel: tile
+// 0, N = 64 ... 2048, and the twiddle table that the pass reads at hand (the radix-4 one is
+// kept by contexts and plans, not by fch_fft_r2c_noalloc)
+template <typename T> inline int reg_pass(const fch_kparams &kp, int tile, bool xf)
+{
+    if (tile != 0 || kp.logN < 6 || kp.logN > 11) return 0;
+    const int p = reg_points<T>(kp.logN, xf);
+    return (p == 4 ? kp.tw4 : kp.tw) ? p : 0;
+}
+
 template <typename T, int LOGN, bool XF> struct RegCfg {
     static constexpr bool single = sizeof(T) == 4, dfl = std::is_same<T, df>::value;
     static constexpr int N = 1 << LOGN;
-    static constexpr int ppt = single ? (XF ? 8 : LOGN <= 8 ? 2 : LOGN == 9 ? 4 : 8)
-                               : dfl  ? (LOGN <= 8 ? 2 : LOGN <= 10 ? 4 : 8)
-                                      : (LOGN <= 7 ? 2 : LOGN <= 8 ? 4 : 8);
+    static constexpr int ppt = reg_points<T>(LOGN, XF);
     static constexpr int tps = N / ppt;
     // rows: whole warps
     static constexpr int rpb = tps >= 32 ? 1 : 32 / tps;
