@@ -375,14 +375,16 @@ fch_status fch_fno_learned_start(fch_ctx *ctx, fch_fno *net, double dt, void *v0
  * fch_autotune times the forward row pass (real fields -> pair-layout work array)
  * and the forward column pass (work array -> half spectra) at n x n in precision
  * prec as a standalone transform plan launches them (as many field pairs per launch
- * as a plan's work array holds; one pair for FCH_FP32X2), for each candidate tile: the default, the
- * generic kernels at their default geometry at n = 1024 (the default being the passes
- * built for the size), the warp-level column passes (FCH_MIXED, n = 1024), and
- * the generic kernels at 1, 2, 4, 8, 16 rows (column pairs) per
- * block that fit. It allocates and frees its own scratch arrays on the given
+ * as a plan's work array holds; one pair for FCH_FP32X2), for each candidate tile: the
+ * default (the passes built for the size; FCH_MIXED at n = 1024: the columns plans stage by
+ * TMA), the generic kernels at their default geometry at n = 1024, the warp-level column
+ * passes (FCH_MIXED, n = 1024), and the generic kernels at 1, 2, 4, 8, 16 rows (column
+ * pairs) per block that fit. It allocates and frees its own scratch arrays on the given
  * stream (NULL: the legacy default stream), synchronizes it, and keeps the fastest
  * tiles per (n, prec) for the process: later calls return them without timing,
- * contexts created with params.autotune = 1 and plans created afterwards use them.
+ * contexts created with params.autotune = 1 and plans created afterwards use them
+ * (contexts of FCH_MIXED at n = 1024, whose default columns are others, the tile that is
+ * faster than those).
  * Tiles change launch shapes only; every tile computes the same transform (results
  * may differ in rounding where the transforms' radices differ).
  * Errors: FCH_EINVAL (n not a power of two in [16, 2048], prec not 0..2, out NULL),

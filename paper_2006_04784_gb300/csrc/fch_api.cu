@@ -654,6 +654,8 @@ static fch_status rowt(fch_ctx *ctx, int mode, int flags, int op, double arg = 0
         if (s_ != FCH_OK) return s_;                                                      \
     } while (0)
 
+static int tuned_context_col(int n, int prec); // fch_autotune's choice of column tile for contexts
+
 extern "C" fch_status fch_create(const fch_grid *g, const fch_params *p, void *stream, fch_ctx **out)
 {
     if (!g || !p || !out) return FCH_EINVAL;
@@ -699,7 +701,7 @@ extern "C" fch_status fch_create(const fch_grid *g, const fch_params *p, void *s
             return ts;
         }
         trow = t.tile_row;
-        tcol = t.tile_col;
+        tcol = p->autotune == 2 ? t.tile_col : tuned_context_col(N, ctx->prec);
     }
     ctx->geom = fch_geometry_tiled(N, ctx->prec == FCH_MIXED, trow, tcol);
     if (tcol == 0 && fch_reg_col_blocks(N, ctx->prec == FCH_MIXED))
@@ -1980,6 +1982,9 @@ extern "C" fch_status fch_get_sav_r(fch_ctx *ctx, double *r_n, double *r_nm1)
 static std::mutex g_tune_mutex;
 static fch_tile g_tune[3][12];
 static bool g_tune_ok[3][12];
+// the column tile for contexts, where their default is another kernel than the plans' (single
+// precision at 1024^2: plans run the TMA-staged columns, contexts the built ones)
+static int g_tune_ctx_col[3][12];
 
 // the tiles fch_autotune chose for (n, prec) in this process, if it ran
 static bool tuned_tiles(int n, int prec, int *row, int *col)
@@ -1990,6 +1995,12 @@ static bool tuned_tiles(int n, int prec, int *row, int *col)
     *row = g_tune[prec][l].tile_row;
     *col = g_tune[prec][l].tile_col;
     return true;
+}
+
+static int tuned_context_col(int n, int prec)
+{
+    std::lock_guard<std::mutex> lock(g_tune_mutex);
+    return g_tune_ctx_col[prec][ilog2(n)];
 }
 
 // Mean time (us) of `reps` launches of one pass after two untimed ones.
@@ -2035,7 +2046,10 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
     const int np = prec == FCH_FP32X2 ? 1 : plan_chunk(n, prec);
     const size_t rb = (size_t)n * n * rsz, cb = (size_t)(n / 2 + 1) * n * csz;
     void *x = nullptr, *Z = nullptr, *X = nullptr, *tw = nullptr, *tw4 = nullptr, *tw2 = nullptr;
-    cudaError_t e = cudaMalloc(&x, 2 * np * rb);
+    int *err = nullptr, herr = 0;
+    cudaError_t e = cudaMalloc(&err, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
+    if (e == cudaSuccess) e = cudaMalloc(&x, 2 * np * rb);
     if (e == cudaSuccess) e = cudaMalloc(&Z, (size_t)np * n * n * csz);
     if (e == cudaSuccess) e = cudaMalloc(&X, 2 * np * cb);
     if (e == cudaSuccess) e = cudaMalloc(&tw, (size_t)n * csz);
@@ -2063,6 +2077,7 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
     kp.out1 = (char *)X + cb;
     kp.npairs = np;
     kp.pdl = prec == FCH_FP32X2 ? 0 : 1; // as plans launch
+    kp.err = prec == FCH_FP32X2 ? nullptr : err;
     auto launch = [&](bool is_col, const fch_kparams &kk) {
         fch_kparams k = kk; // pair j reads fields 2j, 2j+1 and writes their spectra
         k.pstride_in = is_col ? 0 : 2 * (long long)rb;
@@ -2075,15 +2090,18 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
                : prec == FCH_FP32X2 ? fch_launch_row_dfl(RM_R2C_LOAD, k, s)
                                     : fch_launch_row_f64(RM_R2C_LOAD, k, s);
     };
-    // candidates: the default tiles (timed first: the passes built for the size), at 1024^2
-    // the generic kernel at its default geometry and the warp-level columns, and the generic
+    // candidates: the default tiles (timed first: the passes built for the size, in single
+    // precision at 1024^2 the plans' staged columns), at 1024^2 the generic kernel at its
+    // default geometry and the warp-level columns, and the generic
     // kernel at 1..16 rows (column pairs) a block; another tile replaces the default only if 3 % faster
     fch_tile best;
     memset(&best, 0, sizeof(best));
+    int ctx_t = 0; // contexts' columns (the last loop's)
     const int reps = n >= 1024 ? 10 : 20;
     for (int is_col = 0; is_col < 2 && e == cudaSuccess; is_col++) {
-        double best_us = 1e30, def_us = 0;
+        double best_us = 1e30, def_us = 0, ctx_us = 0, ctx_def_us = 0;
         int best_t = 0;
+        ctx_t = 0;
         const int cands[] = {0, -1, -2, 1, 2, 4, 8, 16};
         for (int c : cands) {
             if (c < 0 && n != 1024) continue;
@@ -2099,9 +2117,21 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
             if (c == 0) {
                 def_us = us;
                 best_us = us;
-            } else if (us < best_us && us < 0.97 * def_us) { // the default unless 3 % faster
+                if (is_col && single && n == 1024) { // the contexts' default
+                    k.err = nullptr;
+                    e = time_pass([&] { return launch(true, k); }, s, reps, &us);
+                    if (e != cudaSuccess) break;
+                }
+                ctx_us = ctx_def_us = us;
+                continue;
+            }
+            if (us < best_us && us < 0.97 * def_us) { // the default unless 3 % faster
                 best_us = us;
                 best_t = c;
+            }
+            if (us < ctx_us && us < 0.97 * ctx_def_us) {
+                ctx_us = us;
+                ctx_t = c;
             }
         }
         if (is_col) {
@@ -2114,15 +2144,18 @@ extern "C" fch_status fch_autotune(int n, int prec, void *stream, fch_tile *out)
             best.row_default_us = def_us;
         }
     }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (void *b : {x, Z, X, tw, tw4, tw2})
+    for (void *b : {(void *)err, x, Z, X, tw, tw4, tw2})
         if (b) cudaFree(b);
-    if (e != cudaSuccess) {
-        snprintf(g_plan_err, sizeof(g_plan_err), "fch_autotune: %s", cudaGetErrorString(e));
+    if (e != cudaSuccess || herr) {
+        snprintf(g_plan_err, sizeof(g_plan_err), "fch_autotune: %s",
+                 e != cudaSuccess ? cudaGetErrorString(e) : "a column pass's wait on a bulk copy ran out of time");
         return FCH_ECUDA;
     }
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     g_tune[prec][ilog2(n)] = best;
+    g_tune_ctx_col[prec][ilog2(n)] = ctx_t;
     g_tune_ok[prec][ilog2(n)] = true;
     *out = best;
     return FCH_OK;
