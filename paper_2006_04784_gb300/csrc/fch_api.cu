@@ -49,14 +49,6 @@ fch_geom fch_geometry(int N, int prec)
     return g;
 }
 
-// blocks of the column passes built for a grid size (RegCfg in fch_reg.cuh): a column pair
-// each in 16-byte elements, at N = 1024 a column; two pairs in 8-byte ones; 0: none built
-int fch_reg_col_blocks(int N, int prec)
-{
-    if (N < 64 || N > 2048) return 0;
-    return prec == 1 ? N / 4 : N == 1024 ? N : N / 2;
-}
-
 fch_geom fch_geometry_tiled(int N, int prec, int tile_row, int tile_col)
 {
     fch_geom g = fch_geometry(N, prec);
@@ -2505,6 +2497,48 @@ extern "C" int fch_debug_built_pass(int n, int prec, int xf, int tw4)
     return prec == FCH_MIXED    ? fch::reg_pass<float>(kp, 0, xf != 0)
            : prec == FCH_FP32X2 ? fch::reg_pass<fch::df>(kp, 0, xf != 0)
                                 : fch::reg_pass<double>(kp, 0, xf != 0);
+}
+
+// the index maps of the built passes at n points: out[i] the skewed place of element i,
+// out[n + i] the pair-layout slot of natural index i (CPU tests)
+extern "C" int fch_debug_maps(int n, int *out)
+{
+    if (!pow2_in_range(n) || !out) return 1;
+    for (int i = 0; i < n; i++) {
+        out[i] = fch::skew(i);
+        out[n + i] = fch::pair_slot(i, n);
+    }
+    return 0;
+}
+
+// their launch configuration, for steps (xf 0) or standalone transforms: points a thread, rows
+// a block, row threads, row shared memory, columns a block, column blocks, column threads,
+// column shared memory (CPU tests); 0, or 1 where none is built
+template <typename T, bool XF> static int built_config(int logn, int *out)
+{
+    auto fill = [&](auto g) {
+        typedef decltype(g) G;
+        const int v[8] = {G::ppt, G::rpb, G::row_threads, G::row_smem, G::ncol, G::col_blocks, G::col_threads, G::col_smem};
+        memcpy(out, v, sizeof(v));
+        return 0;
+    };
+    switch (logn) {
+    case 6: return fill(fch::RegCfg<T, 6, XF>());
+    case 7: return fill(fch::RegCfg<T, 7, XF>());
+    case 8: return fill(fch::RegCfg<T, 8, XF>());
+    case 9: return fill(fch::RegCfg<T, 9, XF>());
+    case 10: return fill(fch::RegCfg<T, 10, XF>());
+    case 11: return fill(fch::RegCfg<T, 11, XF>());
+    }
+    return 1;
+}
+extern "C" int fch_debug_built_config(int n, int prec, int xf, int *out)
+{
+    if (!pow2_in_range(n) || prec < 0 || prec > 2 || !out) return -1;
+    const int l = ilog2(n);
+    if (prec == FCH_MIXED) return xf ? built_config<float, true>(l, out) : built_config<float, false>(l, out);
+    if (prec == FCH_FP32X2) return xf ? built_config<fch::df, true>(l, out) : built_config<fch::df, false>(l, out);
+    return xf ? built_config<double, true>(l, out) : built_config<double, false>(l, out);
 }
 
 __global__ void fch_debug_dfl_exp_kernel(const double *x, double *ex, double *em, long cnt)

@@ -192,8 +192,13 @@ cudaError_t fch_launch_row_dfl(int mode, const fch_kparams &kp, cudaStream_t s);
 FCH_REG_DECL(f64)
 FCH_REG_DECL(f32)
 FCH_REG_DECL(dfl)
-// blocks of their column pass at grid size N (one partial sum each), prec as fch_geometry
-int fch_reg_col_blocks(int N, int prec);
+// blocks of their column pass at grid size N (one partial sum each; RegCfg in fch_reg.cuh is
+// checked against it), prec as fch_geometry: a column pair each in 16-byte elements, at
+// N = 1024 a column; two pairs in 8-byte ones; 0: none built
+constexpr int fch_reg_col_blocks(int N, int prec)
+{
+    return N < 64 || N > 2048 ? 0 : prec == 1 ? N / 4 : N == 1024 ? N : N / 2;
+}
 // launch configuration with programmatic stream serialization (when enabled)
 bool fch_pdl_enabled();
 void fch_pdl_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, dim3 grid, dim3 block, size_t smem,

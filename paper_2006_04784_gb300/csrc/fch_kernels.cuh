@@ -176,7 +176,7 @@ template <int DIR, typename C> __device__ __forceinline__ void bfly8(C *v)
 
 // Shared-memory skew: element n of a sequence is stored at n + n/8, which spreads
 // the stride-R stores of the first Stockham stages over the banks.
-__device__ __forceinline__ int skew(int n) { return n + (n >> 3); }
+__host__ __device__ __forceinline__ int skew(int n) { return n + (n >> 3); }
 __host__ __device__ inline int skewed_len(int n) { return n + (n >> 3); }
 
 // One Stockham stage of radix R = 2^LR on a length-N sequence at

@@ -3,6 +3,9 @@
 // kernels build in parallel.
 #include "fch_reg.cuh"
 
+static_assert(fch::RegCfg<FCH_T, FCH_LOGN, false>::col_blocks == fch_reg_col_blocks(1 << FCH_LOGN, sizeof(FCH_T) == 4),
+              "a partial sum for every block of the columns");
+
 namespace {
 
 typedef void (*pass_fn)(const fch_kparams);

@@ -295,7 +295,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
 }
 
 // slot of natural index e in a pair-layout row (the inverse of pair_kx)
-__device__ __forceinline__ int pair_slot(int e, int N)
+__host__ __device__ __forceinline__ int pair_slot(int e, int N)
 {
     return e < (N >> 1) ? 2 * e : (e == (N >> 1) ? 1 : 2 * (N - e) + 1);
 }
