@@ -161,7 +161,7 @@ def _profile_value(name: str, prec: str, kernel: str, n: int):
 
 
 def compulsory_bytes(name: str, n: int, csz: int):
-    """Compulsory HBM bytes of one launch of a pass (SURVEY 8(d) accounting): the
+    """Compulsory HBM bytes of one launch of a pass: the
     arrays of the step's own inputs and outputs it must read or write, once. The
     trial reads u^n, u^{n-1}, F(u^n), F(u^{n-1}) and writes u~, F(u~) (6H in all);
     the work array between the passes and the real-space fields a trial keeps for the
@@ -179,8 +179,8 @@ def compulsory_bytes(name: str, n: int, csz: int):
 
 
 def method_flops(name: str, n: int):
-    """Floating-point operations the method itself needs in one launch of a pass
-    (SURVEY 8(d)): 2.5 n^2 log2(n^2) per 2D real transform, a row or column pass
+    """Floating-point operations the method itself needs in one launch of a pass:
+    2.5 n^2 log2(n^2) per 2D real transform, a row or column pass
     doing one half of each transform it touches, plus the pointwise flops of the
     pass per grid point (the IMEX step's ~60 a point split over its passes)."""
     T = 2.5 * n * n * math.log2(n * n)
@@ -1287,8 +1287,8 @@ def fno_bench(args):
 
 
 def error_budget(args):
-    """Per-field error of each precision against the FP64 oracle (the benchmark spec's mixed-
-    precision budget) on the random bilayer network (critical parameters) at 1024^2
+    """Per-field error of each precision against the FP64 oracle (the mixed-precision
+    error budget) on the random bilayer network (critical parameters) at 1024^2
     and 2048^2: F(u) of the initial data; u, F(u), mass and energy after one and after
     budget_steps fixed IMEX steps of budget_dt (one step at 2048^2); SAV's u and r after
     one step; the LTE estimate e and the state after the backward-Euler start and one

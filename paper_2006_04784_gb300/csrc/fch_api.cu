@@ -30,8 +30,8 @@ fch_geom fch_geometry(int N, int prec)
     const int SL = N + N / 8; // skewed sequence length in shared memory
     g.col_smem = (N + 2 * P * SL) * csz;
     if (N == 1024 && csz == 16) {
-        // two-block clusters, one column of a pair per block (the passes built for 1024 keep
-        // this grid; the generic kernel takes the tile -1 geometry below)
+        // the grid of the passes built for 1024: two-block clusters, one column of a pair per
+        // block (the generic kernel takes the tile -1 geometry below)
         g.col_threads = N / 8;
         g.col_blocks = N;
         g.col_smem = SL * csz;
@@ -899,8 +899,6 @@ extern "C" fch_status fch_get_state_device(fch_ctx *ctx, void *u_dev, int dtype)
     return store_state(ctx, u_dev, dtype == 0);
 }
 
-// one trial step from the current history into the trial slot (parameters already
-// in the control block). pack_f: leave (u_new, Lap u_new) packed for F(u_new).
 // PSD iterations, eqs. (residual), (recurrence), from the iterate in Vb (packed in Z
 // by the pass before) until the stopping test holds; the trial slot then receives
 // the converged iterate
@@ -986,8 +984,9 @@ __global__ void fch_psd_loop_kernel(cudaGraphConditionalHandle h, const fch_ctrl
 
 // PSD iterations inside a stream capture: a while node whose body is one chunk of
 // iterations and the condition launch, then the copy of the converged iterate. The
-// launches next to the node go without programmatic serialization (a programmatic
-// edge joins two kernel nodes only), and so do the body's.
+// launches next to the node, the body's first and the condition launch go without
+// programmatic serialization (a programmatic edge joins two kernel nodes of one graph only);
+// the body's other passes launch with it.
 static fch_status psd_loop_captured(fch_ctx *ctx)
 {
     if (!ctx->bstream) CKC(ctx, cudaStreamCreateWithFlags(&ctx->bstream, cudaStreamNonBlocking));
@@ -1036,7 +1035,8 @@ static fch_status psd_loop_captured(fch_ctx *ctx)
     return s;
 }
 
-// packed: Z holds (u*, Lap u*) already (the solve of the fixed step before packed it);
+// one trial step from the current history into the trial slot (parameters already in the
+// control block). packed: Z holds (u*, Lap u*) already (the solve of the fixed step before packed it);
 // pack: FCH_FL_PACK_F, FCH_FL_PACK_USTAR or 0
 static fch_status enqueue_trial(fch_ctx *ctx, fch_scheme scheme, int pf, bool packed = false)
 {

@@ -50,6 +50,7 @@ template <int M> cudaError_t launch_col_w(const fch_kparams &kp, cudaStream_t s)
 // default geometry; -2 (columns, single precision at N = 1024) the warp-level column pass;
 // > 0 the generic kernel with that many column pairs (rows) per block; <= -3 the same at
 // four points a thread. The generic column kernel reads P from kp.P, which the caller sets.
+
 // N = 1024, single precision, the column passes of standalone transform plans (which
 // carry an error word): the persistent TMA-staged kernel, as many blocks as are
 // resident at once; the inverse needs 16-byte aligned half spectra (bulk copies)
@@ -112,7 +113,7 @@ template <typename T, int M> cudaError_t launch_col(const fch_kparams &kp, cudaS
     }
     if (kp.tile_col <= -3) {
         // the generic kernel at four points a thread: needs the radix-4 twiddle table
-        // (contexts carry one, standalone plans do not)
+        // (contexts and plans carry one, fch_fft_r2c_noalloc does not)
         if (!kp.tw4) return cudaErrorInvalidValue;
         static int attr4 = 0;
         const fch_geom g = fch_geometry_tiled(kp.N, sizeof(T) == 4, 0, kp.tile_col);
@@ -135,7 +136,7 @@ template <typename T, int M> cudaError_t launch_col(const fch_kparams &kp, cudaS
 template <typename T, int M> cudaError_t launch_row(const fch_kparams &kp, cudaStream_t s)
 {
     if (kp.tile_row <= -3) {
-        // the generic kernel at four points a thread (radix-4 twiddle table: contexts only)
+        // the generic kernel at four points a thread (radix-4 twiddle table, as the columns)
         if (!kp.tw4) return cudaErrorInvalidValue;
         static int attr4 = 0;
         const fch_geom g = fch_geometry_tiled(kp.N, sizeof(T) == 4, kp.tile_row, 0);
